@@ -1,6 +1,7 @@
 // Register-level int4 -> bf16 dequantisation shared by every kernel of the
 // library (the exported dequant, the GEMM and the small-M path), so that the
-// GEMM's weights are bit-identical to w4a16_dequant's output.
+// GEMM's weights are w4a16_dequant's output, value for value (only the sign of
+// a zero may differ).
 //
 // A packed 32-bit word holds eight consecutive codes q_0..q_7 of one row
 // (q_i in bits 4i..4i+3: byte j carries the even k in its low nibble and the
@@ -46,6 +47,54 @@ __device__ __forceinline__ void dequant_word(uint32_t w, uint32_t s2, uint32_t* 
         uint32_t t = prmt_b32(w, w4, static_cast<uint32_t>(j | ((4 + j) << 8)));
         t = (t & 0x000F000Fu) | 0x43004300u;               // (128 + q_2j, 128 + q_2j+1)
         out[j] = bf16x2_mul(bf16x2_sub(t, 0x43084308u), s2);  // (q - 8) * s, one rounding
+    }
+}
+
+// The same values with one rounding step per pair: RNE_bf16(q s - 8 s) as a
+// single bf16x2 FMA.  Bits 0..7 of a bf16 with the other bits zero are the
+// integer times 2^-133 (the subnormals and the first binade are one linear
+// range), so a masked nibble is already a number: the even code moved to bits
+// 3..6 of its byte is 8 q 2^-133, the odd code left in bits 4..7 is
+// 16 q 2^-133, and the FMA's multiplier takes the power of two back.
+// Exact before its one rounding for |s| < 2^-2 (the multiplier s 2^130 has to
+// be finite); scale_is_wide marks the others, which take dequant_word.  A zero
+// (q = 8) is always +0 here.
+struct ScaleFma {
+    uint32_t mul;  // (s 2^130, s 2^129): for the even, the odd code of a pair
+    uint32_t add;  // (-8 s, -8 s)
+};
+
+__device__ __forceinline__ bool scale_is_wide(uint16_t s) { return (s & 0x7FFFu) >= 0x3E80u; }
+
+__device__ __forceinline__ uint32_t bf16x2_fma(uint32_t a, uint32_t b, uint32_t c) {
+    uint32_t r;
+    asm("fma.rn.bf16x2 %0, %1, %2, %3;" : "=r"(r) : "r"(a), "r"(b), "r"(c));
+    return r;
+}
+
+__device__ __forceinline__ ScaleFma scale_fma(uint32_t s2) {
+    ScaleFma f;
+    f.mul = bf16x2_mul(bf16x2_mul(s2, 0x60006000u), 0x5F806000u);  // 2^65, then (2^65, 2^64)
+    f.add = bf16x2_mul(s2, 0xC100C100u);
+    return f;
+}
+
+// 8 codes -> 4 bf16x2 words as dequant_word: six integer ops (two masks, four
+// byte selects; a selector of 8 + j repeats the sign bit of byte j, here the
+// zero that fills the upper byte of each half), one multiply, four FMAs --
+// 11 instructions where dequant_word takes 17.  Integer and bf16x2 operations
+// issue at half rate, so this is what the GEMM's dequant warps are bound by:
+// 256 x 12288 x 49152 215 -> 204 us, gate/up + SwiGLU at 8192 tokens
+// 12.54 -> 12.17 ms (power cap), 2048 x 12288 x 12288 with g = 64 390 -> 370 us.
+__device__ __forceinline__ void dequant_word_fma(uint32_t w, const ScaleFma& f, uint32_t* out) {
+    uint32_t w8;
+    asm("mul.lo.u32 %0, %1, 8;" : "=r"(w8) : "r"(w));
+    const uint32_t e = w8 & 0x78787878u, o = w & 0xF0F0F0F0u;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const uint32_t z = 8u + static_cast<uint32_t>(j);
+        const uint32_t sel = static_cast<uint32_t>(j) | (z << 4) | (static_cast<uint32_t>(4 + j) << 8) | (z << 12);
+        out[j] = bf16x2_fma(prmt_b32(e, o, sel), f.mul, f.add);
     }
 }
 

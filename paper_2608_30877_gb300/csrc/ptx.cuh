@@ -163,6 +163,7 @@ template <bool kCluster = false>
 __device__ __forceinline__ bool wait_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag,
                                           int* status, uint64_t limit_ns) {
     const uint32_t lane = threadIdx.x & 31u;
+    if (__all_sync(0xffffffffu, mbar_try_wait<kCluster>(bar, parity))) return true;
     const uint64_t t0 = global_timer_ns();
     for (uint32_t it = 0;; ++it) {
         const bool done = mbar_try_wait<kCluster>(bar, parity);
@@ -191,6 +192,7 @@ __device__ __forceinline__ bool wait_warp_sleep(uint32_t bar, uint32_t parity,
                                                 volatile int* abort_flag, int* status,
                                                 uint64_t limit_ns, uint32_t sleep_ns) {
     const uint32_t lane = threadIdx.x & 31u;
+    if (__all_sync(0xffffffffu, mbar_try_wait<kCluster>(bar, parity))) return true;
     const uint64_t t0 = global_timer_ns();
     for (uint32_t it = 0;; ++it) {
         const bool done = mbar_try_wait<kCluster>(bar, parity);

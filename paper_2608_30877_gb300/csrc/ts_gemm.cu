@@ -533,14 +533,27 @@ __global__ void __launch_bounds__(threads_for<DQ, EP>(), MIN_BLOCKS)
                 const uint4 w1 = *reinterpret_cast<const uint4*>(wrow + (16u ^ swz));
                 const uint32_t s2 = splat_bf16(s_cur);
                 uint32_t v[32];
-                dequant_word(w0.x, s2, v + 0);
-                dequant_word(w0.y, s2, v + 4);
-                dequant_word(w0.z, s2, v + 8);
-                dequant_word(w0.w, s2, v + 12);
-                dequant_word(w1.x, s2, v + 16);
-                dequant_word(w1.y, s2, v + 20);
-                dequant_word(w1.z, s2, v + 24);
-                dequant_word(w1.w, s2, v + 28);
+                // one FMA per pair unless some row's scale is outside its range
+                if (!__any_sync(0xffffffffu, scale_is_wide(s_cur))) {
+                    const ScaleFma f = scale_fma(s2);
+                    dequant_word_fma(w0.x, f, v + 0);
+                    dequant_word_fma(w0.y, f, v + 4);
+                    dequant_word_fma(w0.z, f, v + 8);
+                    dequant_word_fma(w0.w, f, v + 12);
+                    dequant_word_fma(w1.x, f, v + 16);
+                    dequant_word_fma(w1.y, f, v + 20);
+                    dequant_word_fma(w1.z, f, v + 24);
+                    dequant_word_fma(w1.w, f, v + 28);
+                } else {
+                    dequant_word(w0.x, s2, v + 0);
+                    dequant_word(w0.y, s2, v + 4);
+                    dequant_word(w0.z, s2, v + 8);
+                    dequant_word(w0.w, s2, v + 12);
+                    dequant_word(w1.x, s2, v + 16);
+                    dequant_word(w1.y, s2, v + 20);
+                    dequant_word(w1.z, s2, v + 24);
+                    dequant_word(w1.w, s2, v + 28);
+                }
                 if (dbg_check(L::A_COL + (sa + 1) * (kBK / 2) <= L::TMEM_COLS, p.status))
                     tmem_st_32x32b_x32(lane_base + L::A_COL + sa * (kBK / 2), v);
                 tmem_st_wait();
