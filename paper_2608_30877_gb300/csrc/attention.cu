@@ -441,6 +441,11 @@ __global__ void __launch_bounds__(kThreads, 2)
                         tma_load_2d(ks + L::KBOX, &tmap_kv, k_full(s), Hd + jb.h * kD + 64, row);
                     }
                     ++nk;
+                    if (g == 0 &&
+                        !short_limit_ok(k_full(0), 0, abort_flag, p.status, p.wait_ns)) {
+                        ok = false;
+                        break;
+                    }
                     if (!wait_one(v_empty(s), par, abort_flag, p.status, p.wait_ns)) {
                         ok = false;
                         break;
@@ -468,12 +473,16 @@ __global__ void __launch_bounds__(kThreads, 2)
         }
     } else if (warp == 1) {
         // ------------------------------------------------------------ MMA issuers
-        // Two threads: this warp's issues the S products, warp 6's the PV
+        // Two warps: this one issues the S products, the next the PV
         // products, each waiting only on what its own products need and
         // committing its own barriers, so neither's waits hold up the other's
         // MMAs.  S runs two blocks ahead of PV: S of block g + 2 goes into S
         // buffer g & 1 as soon as the PV product of block g has read P from
-        // it, so it overlaps the softmax of block g + 1.
+        // it, so it overlaps the softmax of block g + 1.  The whole warp runs the
+        // loop and one elected lane issues, which keeps the descriptors in uniform
+        // registers (issued from a lane-0 branch an MMA took ~120 clocks, twice
+        // its run time: 64 x 1024 tokens x 96 heads 2195 -> 2114 us, one sequence of
+        // 10007 under a window of 4096 1511 -> 1440).
         constexpr uint32_t idesc_s = idesc_bf16_f32(kBQ, kBKV);
         bool ok = run;
         BlockWalk ws;  // the next block to take its S product
@@ -484,36 +493,35 @@ __global__ void __launch_bounds__(kThreads, 2)
         uint32_t gs = 0;
         while (ok && ws.valid) {
             const uint32_t b = gs & 1u;
-            if (lane == 0) {
-                // the buffer's previous block (gs - 2) has had its PV product
-                ok = gs < 2 || wait_one(o_ready(b), ((gs - 2) >> 1) & 1u, abort_flag, p.status,
-                                        p.wait_ns);
-                if (ok && ws.j == 0)
-                    ok = wait_one(q_full, ws.jn & 1u, abort_flag, p.status, p.wait_ns);
-                if (ok) ok = wait_one(k_full(b), (gs >> 1) & 1u, abort_flag, p.status, p.wait_ns);
-                if (ok) {
-                    tc_fence_after();
-                    const uint32_t qs = sbase + L::Q_OFF, ks = sbase + L::K_OFF + b * L::KV_TILE;
+            // the buffer's previous block (gs - 2) has had its PV product
+            ok = gs < 2 ||
+                 wait_warp(o_ready(b), ((gs - 2) >> 1) & 1u, abort_flag, p.status, p.wait_ns);
+            if (ok && ws.j == 0) ok = wait_warp(q_full, ws.jn & 1u, abort_flag, p.status, p.wait_ns);
+            if (ok) ok = wait_warp(k_full(b), (gs >> 1) & 1u, abort_flag, p.status, p.wait_ns);
+            if (!ok) break;
+            tc_fence_after();
+            const uint64_t qd = sdesc_kmajor_sw128(sbase + L::Q_OFF);
+            const uint64_t kd = sdesc_kmajor_sw128(sbase + L::K_OFF + b * L::KV_TILE);
+            const uint32_t d = tmem + L::S_COL + b * kBKV;
+            if (elect_one()) {
 #pragma unroll
-                    for (int kk = 0; kk < kD / 16; ++kk) {
-                        tc_mma_ss(tmem + L::S_COL + b * kBKV,
-                                  sdesc_kmajor_sw128(qs + (kk >> 2) * L::QBOX + (kk & 3) * 32),
-                                  sdesc_kmajor_sw128(ks + (kk >> 2) * L::KBOX + (kk & 3) * 32),
-                                  idesc_s, kk > 0 ? 1u : 0u);
-                    }
-                    tc_commit(s_full(b));
-                    tc_commit(k_empty(b));
-                    if (ws.j == ws.nblk - 1) tc_commit(q_empty);  // the job's last S frees Q
-                }
+                for (int kk = 0; kk < kD / 16; ++kk)
+                    tc_mma_ss(d, qd + (((kk >> 2) * L::QBOX + (kk & 3) * 32) >> 4),
+                              kd + (((kk >> 2) * L::KBOX + (kk & 3) * 32) >> 4), idesc_s,
+                              kk > 0 ? 1u : 0u);
+                tc_commit(s_full(b));
+                tc_commit(k_empty(b));
+                if (ws.j == ws.nblk - 1) tc_commit(q_empty);  // the job's last S frees Q
             }
-            ok = __shfl_sync(0xffffffffu, ok, 0);
+            __syncwarp();
             ++gs;
             walk_next(p, njobs, t_step, lane, ws);
         }
-        if (lane == 0) {
+        if (elect_one()) {
             tc_commit(drain(0));  // every MMA issued has completed before tensor memory is freed
             settle(drain(0), 0);
         }
+        __syncwarp();
     } else if (warp == kPvWarp) {
         // ------------------------------------------------------------ PV issuer
         constexpr uint32_t idesc_o = idesc_bf16_f32(kBQ, kD) | (1u << 16);  // B MN-major
@@ -526,33 +534,34 @@ __global__ void __launch_bounds__(kThreads, 2)
         uint32_t g = 0;
         while (ok && wp.valid) {
             const uint32_t b = g & 1u;
-            if (lane == 0) {
-                // O += P V once the softmax warps have written P of block g (for
-                // a job's first block, after they read out the previous job's O)
-                ok = wait_one(p_full(b), (g >> 1) & 1u, abort_flag, p.status, p.wait_ns) &&
-                     wait_one(v_full(b), (g >> 1) & 1u, abort_flag, p.status, p.wait_ns);
-                if (ok) {
-                    tc_fence_after();
-                    const uint32_t vs = sbase + L::V_OFF + b * L::KV_TILE;
+            // O += P V once the softmax warps have written P of block g (for
+            // a job's first block, after they read out the previous job's O)
+            ok = wait_warp(p_full(b), (g >> 1) & 1u, abort_flag, p.status, p.wait_ns) &&
+                 wait_warp(v_full(b), (g >> 1) & 1u, abort_flag, p.status, p.wait_ns);
+            if (!ok) break;
+            tc_fence_after();
+            const uint64_t vd =
+                sdesc_mnmajor_sw128(sbase + L::V_OFF + b * L::KV_TILE, L::KBOX, 1024);
+            const uint32_t ptm = tmem + L::S_COL + b * kBKV;
+            const uint32_t more = wp.j > 0 ? 1u : 0u;
+            if (elect_one()) {
 #pragma unroll
-                    for (int kk = 0; kk < kBKV / 16; ++kk) {
-                        // keys 16 kk .. 16 kk + 15: rows of the V tile; P columns 8 kk ..
-                        tc_mma_ts(tmem + L::O_COL, tmem + L::S_COL + b * kBKV + kk * 8,
-                                  sdesc_mnmajor_sw128(vs + kk * 16 * 128, L::KBOX, 1024), idesc_o,
-                                  (wp.j > 0 || kk > 0) ? 1u : 0u);
-                    }
-                    tc_commit(o_ready(b));
-                    tc_commit(v_empty(b));
-                }
+                for (int kk = 0; kk < kBKV / 16; ++kk)
+                    // keys 16 kk .. 16 kk + 15: rows of the V tile; P columns 8 kk ..
+                    tc_mma_ts(tmem + L::O_COL, ptm + kk * 8, vd + ((kk * 16 * 128) >> 4), idesc_o,
+                              kk > 0 ? 1u : more);
+                tc_commit(o_ready(b));
+                tc_commit(v_empty(b));
             }
-            ok = __shfl_sync(0xffffffffu, ok, 0);
+            __syncwarp();
             ++g;
             walk_next(p, njobs, t_step, lane, wp);
         }
-        if (lane == 0) {
+        if (elect_one()) {
             tc_commit(drain(1));
             settle(drain(1), 0);
         }
+        __syncwarp();
     } else {
         // ------------------------------------------------------------ softmax + epilogue
         // Two warps per TMEM sub-partition: warp (sub, hh) takes the 16 rows

@@ -17,6 +17,17 @@ __device__ __forceinline__ uint64_t global_timer_ns() {
     return t;
 }
 
+// One lane of a converged warp (the same one every time).
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "elect.sync _|p, 0xffffffff;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(p));
+    return p != 0;
+}
+
 // ---------------------------------------------------------------- mbarrier
 
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
@@ -39,44 +50,33 @@ __device__ __forceinline__ void mbar_arrive_expect_tx(uint32_t bar, uint32_t byt
 // A thread whose phase has not completed may be suspended for up to
 // kSuspendHintNs (it resumes as soon as the phase completes), so waiting
 // warps do not take issue slots from the working ones.
-#ifndef W4A16_SUSPEND_HINT_NS
-#define W4A16_SUSPEND_HINT_NS 0x20000
-#endif
-constexpr uint32_t kSuspendHintNs = W4A16_SUSPEND_HINT_NS;
+constexpr uint32_t kSuspendHintNs = 0x20000;
 
-#ifndef W4A16_CLUSTER_HINT_NS
-#define W4A16_CLUSTER_HINT_NS 0x20000
-#endif
-constexpr uint32_t kClusterHintNs = W4A16_CLUSTER_HINT_NS;
+// Whether the phase has completed, without suspending the thread.
+__device__ __forceinline__ bool mbar_test_wait(uint32_t bar, uint32_t parity) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
 
 // kCluster: acquire at cluster scope, for barriers that threads or tensor-core
 // commits of the other CTA of a pair arrive on.
 template <bool kCluster = false>
 __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
     uint32_t ok;
-    if constexpr (kCluster && kClusterHintNs == 0) {
-        asm volatile(
-            "{\n\t.reg .pred p;\n\t"
-            "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
-            "selp.u32 %0, 1, 0, p;\n\t}"
-            : "=r"(ok)
-            : "r"(bar), "r"(parity)
-            : "memory");
-    } else if constexpr (kCluster) {
+    if constexpr (kCluster) {
         asm volatile(
             "{\n\t.reg .pred p;\n\t"
             "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2, %3;\n\t"
             "selp.u32 %0, 1, 0, p;\n\t}"
             : "=r"(ok)
-            : "r"(bar), "r"(parity), "r"(kClusterHintNs)
-            : "memory");
-    } else if (kSuspendHintNs == 0) {
-        asm volatile(
-            "{\n\t.reg .pred p;\n\t"
-            "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-            "selp.u32 %0, 1, 0, p;\n\t}"
-            : "=r"(ok)
-            : "r"(bar), "r"(parity)
+            : "r"(bar), "r"(parity), "r"(kSuspendHintNs)
             : "memory");
     } else {
         asm volatile(
@@ -138,13 +138,36 @@ __device__ __forceinline__ bool tma_box_ok(uint32_t dst, uint32_t box_bytes, uin
 constexpr uint64_t kWaitLimitNs = 4000000000ull;  // 4 s
 constexpr uint32_t kWaitIterCap = 1u << 26;
 
+// The producers' check for a lowered limit (a test of the abort path): a poll of the
+// waits below may suspend its thread until the phase completes, whatever the
+// limit, so each producer waits for its first copy here, with polls that do not.
+// Always true with the default limit.
+__device__ __forceinline__ bool short_limit_ok(uint32_t bar, uint32_t parity,
+                                               volatile int* abort_flag, int* status,
+                                               uint64_t limit_ns) {
+    if (limit_ns >= kWaitLimitNs) return true;
+    const uint64_t t0 = global_timer_ns();
+    while (!mbar_test_wait(bar, parity)) {
+        if (global_timer_ns() - t0 > limit_ns) {
+            *abort_flag = 1;
+            record_status(status, 5 /* W4A16_ERR_TIMEOUT */);
+            return false;
+        }
+    }
+    return true;
+}
+
 // Wait by one thread.  Returns false if the wait ran out or the CTA aborted.
-template <bool kCluster = false>
+// With SLEEP_NS the thread sleeps between polls, for waits that have stages in
+// hand (a TMA producer with a full ring): its polls then take no issue slots
+// from the warps doing the work.
+template <bool kCluster = false, uint32_t SLEEP_NS = 0>
 __device__ __forceinline__ bool wait_one(uint32_t bar, uint32_t parity, volatile int* abort_flag,
                                          int* status, uint64_t limit_ns) {
     if (mbar_try_wait<kCluster>(bar, parity)) return true;
     const uint64_t t0 = global_timer_ns();
     for (uint32_t it = 1;; ++it) {
+        if (SLEEP_NS > 0) __nanosleep(SLEEP_NS);
         if (mbar_try_wait<kCluster>(bar, parity)) return true;
         if ((it & 31u) == 0u || limit_ns < kWaitLimitNs) {
             if (*abort_flag) return false;
@@ -159,46 +182,20 @@ __device__ __forceinline__ bool wait_one(uint32_t bar, uint32_t parity, volatile
 
 // Wait by a whole warp; every lane polls the barrier and the exit is
 // warp-uniform (so that .sync.aligned instructions after it stay converged).
-template <bool kCluster = false>
+// SLEEP_NS as above: for long, latency-tolerant waits (an epilogue waiting for
+// a whole tile's MMAs).
+template <bool kCluster = false, uint32_t SLEEP_NS = 0>
 __device__ __forceinline__ bool wait_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag,
                                           int* status, uint64_t limit_ns) {
-    const uint32_t lane = threadIdx.x & 31u;
+    // (the timer is slow to read: only once a poll has failed)
     if (__all_sync(0xffffffffu, mbar_try_wait<kCluster>(bar, parity))) return true;
+    const uint32_t lane = threadIdx.x & 31u;
     const uint64_t t0 = global_timer_ns();
-    for (uint32_t it = 0;; ++it) {
+    for (uint32_t it = 1;; ++it) {
+        if (SLEEP_NS > 0) __nanosleep(SLEEP_NS);
         const bool done = mbar_try_wait<kCluster>(bar, parity);
         if (__all_sync(0xffffffffu, done)) return true;
-        if ((it & 31u) == 31u || limit_ns < kWaitLimitNs) {
-            int give_up = 0;
-            if (lane == 0) {
-                if (*abort_flag) {
-                    give_up = 1;
-                } else if (it > kWaitIterCap || global_timer_ns() - t0 > limit_ns) {
-                    *abort_flag = 1;
-                    record_status(status, 5 /* W4A16_ERR_TIMEOUT */);
-                    give_up = 1;
-                }
-            }
-            if (__shfl_sync(0xffffffffu, give_up, 0)) return false;
-        }
-    }
-}
-
-// Warp-wide wait for long, latency-tolerant waits (an epilogue waiting for a
-// whole tile's MMAs): between polls the warp sleeps sleep_ns, so it takes no
-// issue slots from the warps doing the work.
-template <bool kCluster = false>
-__device__ __forceinline__ bool wait_warp_sleep(uint32_t bar, uint32_t parity,
-                                                volatile int* abort_flag, int* status,
-                                                uint64_t limit_ns, uint32_t sleep_ns) {
-    const uint32_t lane = threadIdx.x & 31u;
-    if (__all_sync(0xffffffffu, mbar_try_wait<kCluster>(bar, parity))) return true;
-    const uint64_t t0 = global_timer_ns();
-    for (uint32_t it = 0;; ++it) {
-        const bool done = mbar_try_wait<kCluster>(bar, parity);
-        if (__all_sync(0xffffffffu, done)) return true;
-        __nanosleep(sleep_ns);
-        if ((it & 7u) == 7u || limit_ns < kWaitLimitNs) {
+        if ((it & (SLEEP_NS > 0 ? 7u : 31u)) == 0u || limit_ns < kWaitLimitNs) {
             int give_up = 0;
             if (lane == 0) {
                 if (*abort_flag) {

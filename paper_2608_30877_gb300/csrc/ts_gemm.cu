@@ -396,6 +396,12 @@ __global__ void __launch_bounds__(threads_for<DQ, EP>(), MIN_BLOCKS)
                                              sbase + L::BAR_OFF, kt * (kBK / 2), 1) && n0 >= 0,
                                   p.status))
                         tma_load_2d(wd, &tmap_w, full_tma(s), kt * (kBK / 2), n0);
+                    if (it == 0 &&
+                        !short_limit_ok(full_tma(0), 0, abort_flag, p.status, p.wait_ns)) {
+                        ok = false;
+                        ++it;
+                        break;
+                    }
                 }
             }
             // Drain: every load this thread issued has landed before exit.
@@ -404,7 +410,12 @@ __global__ void __launch_bounds__(threads_for<DQ, EP>(), MIN_BLOCKS)
         }
     } else if (warp == 1) {
         // ------------------------------------------------------------ MMA issuer
-        if (lane == 0 && leader) {
+        // The whole warp runs the loops and one elected lane issues, so that the
+        // MMAs' operands stay in uniform registers: moved there per MMA from a
+        // lane-0 branch, they made the issue take ~100 clocks an MMA, as long as a
+        // 192-column MMA runs (256 x 12288 x 49152 204 -> 187 us, 333 x 12288 x
+        // 12288 107 -> 100 us).
+        if (leader) {
             constexpr uint32_t idesc = idesc_bf16_f32(kRows * CW, T / NB);
             uint32_t it = 0, tcount = 0, tiles_done = 0;
             bool ok = true;
@@ -420,59 +431,67 @@ __global__ void __launch_bounds__(threads_for<DQ, EP>(), MIN_BLOCKS)
                 }
             };
             for (int unit = unit_first<CW>(); ok && unit < unit_count<CW>(p); unit += unit_stride<CW>(), ++tcount) {
-                if (!wait_one<PAIR>(d_empty, (tcount & 1u) ^ 1u, abort_flag, p.status, p.wait_ns)) break;
+                if (!wait_warp<PAIR>(d_empty, (tcount & 1u) ^ 1u, abort_flag, p.status, p.wait_ns)) break;
                 tc_fence_after();
                 for (int kt = 0; kt < KT; ++kt, ++it) {
                     const int s = it % S_SMEM;
                     const int sa = it % S_TMEM;
-                    if (!wait_one(full_tma(s), (it / S_SMEM) & 1u, abort_flag, p.status, p.wait_ns) ||
-                        !wait_one<PAIR>(full_a(sa), (it / S_TMEM) & 1u, abort_flag, p.status, p.wait_ns)) {
+                    // the A stage is written in every CTA, whose dequant warps
+                    // waited for their copies: x has landed too
+                    if (!wait_warp<PAIR>(full_a(sa), (it / S_TMEM) & 1u, abort_flag, p.status, p.wait_ns)) {
                         ok = false;
                         break;
                     }
                     tc_fence_after();
-                    const uint32_t xs = sbase + L::X_OFF + s * L::X_BYTES;
+                    const uint64_t bdesc = sdesc_kmajor_sw128(sbase + L::X_OFF + s * L::X_BYTES);
+                    const uint32_t a_tm = tmem + L::A_COL + sa * (kBK / 2);
                     if (!dbg_check(L::A_COL + (sa + 1) * (kBK / 2) <= L::TMEM_COLS &&
                                        L::D_COL + T <= L::A_COL,
                                    p.status))
                         continue;
+                    if (elect_one()) {
 #pragma unroll
-                    for (int ks = 0; ks < kBK / 16; ++ks) {
-                        const uint32_t a = tmem + L::A_COL + sa * (kBK / 2) + ks * 8;
+                        for (int ks = 0; ks < kBK / 16; ++ks) {
 #pragma unroll
-                        for (int nb = 0; nb < NB; ++nb) {
-                            const uint32_t d = tmem + L::D_COL + nb * (T / NB);
-                            const uint64_t b = sdesc_kmajor_sw128(xs + nb * L::X_BOX + ks * 32);
-                            if constexpr (PAIR)
-                                tc_mma_ts_pair(d, a, b, idesc, (kt | ks) != 0);
-                            else
-                                tc_mma_ts(d, a, b, idesc, (kt | ks) != 0);
+                            for (int nb = 0; nb < NB; ++nb) {
+                                const uint32_t d = tmem + L::D_COL + nb * (T / NB);
+                                const uint64_t b = bdesc + static_cast<uint64_t>((nb * L::X_BOX + ks * 32) >> 4);
+                                if constexpr (PAIR)
+                                    tc_mma_ts_pair(d, a_tm + ks * 8, b, idesc, (kt | ks) != 0);
+                                else
+                                    tc_mma_ts(d, a_tm + ks * 8, b, idesc, (kt | ks) != 0);
+                            }
                         }
+                        commit(empty_smem(s));
+                        if constexpr (!kUnified) commit(empty_a(sa));
                     }
+                    __syncwarp();
                     issued = true;
-                    commit(empty_smem(s));
-                    if constexpr (!kUnified) commit(empty_a(sa));
                 }
                 if (!ok) break;
-                commit(d_full);
+                if (elect_one()) commit(d_full);
+                __syncwarp();
                 ++tiles_done;
             }
-            if (issued) {
-                // Drain: all MMAs issued by this thread have completed.
-                if constexpr (PAIR)
-                    tc_commit_pair(drain);
-                else
-                    tc_commit(drain);
-                settle(drain, 0);
+            if (elect_one()) {
+                if (issued) {
+                    // Drain: all MMAs issued by this thread have completed.
+                    if constexpr (PAIR)
+                        tc_commit_pair(drain);
+                    else
+                        tc_commit(drain);
+                    settle(drain, 0);
+                }
+                if constexpr (PAIR) {
+                    // what both CTAs must see land on their barriers before exit
+                    handoff[0] = it;
+                    handoff[1] = tiles_done;
+                    const uint32_t h = smem_u32(const_cast<uint32_t*>(handoff));
+                    st_shared_cluster_u32(mapa_shared(h, 1), it);
+                    st_shared_cluster_u32(mapa_shared(h + 4, 1), tiles_done);
+                }
             }
-            if constexpr (PAIR) {
-                // what both CTAs must see land on their barriers before exit
-                handoff[0] = it;
-                handoff[1] = tiles_done;
-                const uint32_t h = smem_u32(const_cast<uint32_t*>(handoff));
-                st_shared_cluster_u32(mapa_shared(h, 1), it);
-                st_shared_cluster_u32(mapa_shared(h + 4, 1), tiles_done);
-            }
+            __syncwarp();
         }
     } else if (warp < 2 + 4 * DQ) {
         // ------------------------------------------------------------ dequantisers
@@ -580,7 +599,7 @@ __global__ void __launch_bounds__(threads_for<DQ, EP>(), MIN_BLOCKS)
         for (int unit = unit_first<CW>(); unit < unit_count<CW>(p); unit += unit_stride<CW>(), ++tcount) {
             int tt, wt;
             unit_tile<CW>(unit, p, rank, tt, wt);
-            if (!wait_warp_sleep<PAIR>(d_full, tcount & 1u, abort_flag, p.status, p.wait_ns, kEpilogueSleepNs))
+            if (!wait_warp<PAIR, kEpilogueSleepNs>(d_full, tcount & 1u, abort_flag, p.status, p.wait_ns))
                 break;
             tc_fence_after();
             const int n = wt * kRows + sub * 32 + lane;
