@@ -74,12 +74,9 @@ EncodeTiledFn g_encode = nullptr;
 int g_group_t = 6;
 int g_group_t_wide = 3;
 int64_t g_group_bytes = 0;  // if > 0: groups sized so that a group's x takes at most this
-bool g_small_m_streaming = true;
-// Small M on the tcgen05 streaming kernel from this many tokens on, on the
-// warp-level mma.sync kernel below it (12288 x 49152: M = 32 94 against
-// 128 us; M = 16 95 against 83 us; M = 8 95 against 68 us).
-// W4A16_SMALL_M=mma / tc forces one of them.
-int g_small_m_tc_from = 17;
+// M <= 16 with g = 128: the warp-level mma.sync kernel or the tcgen05 streaming kernel,
+// by their modelled times (0).  W4A16_SMALL_M=mma / tc forces one of them.
+char g_small_m = 0;
 bool g_gemm_pair = true;  // large M on CTA pairs (cta_group::2); W4A16_GEMM_PAIR=0: one CTA per tile
 // CTA pairs with 384-token tiles (one dequantised weight stage serves 1.5x the
 // tokens) where they take fewer unit-costs per pair than the 256-token tiles
@@ -107,12 +104,8 @@ int device_state(DeviceState** out) {
                 q != cudaDriverEntryPointSuccess || fn == nullptr)
                 return W4A16_ERR_CUDA;
             g_encode = reinterpret_cast<EncodeTiledFn>(fn);
-            if (const char* e = std::getenv("W4A16_SMALL_M_TILED")) {
-                if (e[0] == '1') g_small_m_streaming = false;
-            }
             if (const char* e = std::getenv("W4A16_SMALL_M")) {
-                if (e[0] == 'm') g_small_m_tc_from = 33;
-                if (e[0] == 't') g_small_m_tc_from = 1;
+                if (e[0] == 'm' || e[0] == 't') g_small_m = e[0];
             }
             if (const char* e = std::getenv("W4A16_GEMM_PAIR")) {
                 if (e[0] == '1') g_gemm_pair = true;
@@ -225,23 +218,9 @@ int encode_2d(CUtensorMap* map, CUtensorMapDataType dtype, const void* base, uin
     return r == CUDA_SUCCESS ? W4A16_OK : W4A16_ERR_CUDA;
 }
 
-// M <= 128 with g = 128: the streaming kernels (rows spread evenly over the
-// SMs); the warp-level one takes at most 32 token columns.
-int launch_gemv(const DeviceState& st, const void* x, const void* w, const void* s, void* out,
-                int64_t M, int64_t N, int64_t K, int64_t g, const Epilogue& epi,
-                cudaStream_t stream) {
-    const bool tc = M > 32 || M >= g_small_m_tc_from;
-    const int T = tc ? gemv_tc_tokens(M) : gemv_tokens_per_tile(M);
-    const int RB = tc ? gemv_tc_rows_per_cta(N, st.sm_count) : gemv_rows_per_cta(N, st.sm_count);
-    alignas(64) CUtensorMap tx;
-    alignas(64) CUtensorMap tw;
-    int rc = encode_2d(&tx, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, x, K, M, K * 2, 64, T,
-                       CU_TENSOR_MAP_SWIZZLE_128B);
-    if (rc != W4A16_OK) return rc;
-    rc = encode_2d(&tw, CU_TENSOR_MAP_DATA_TYPE_UINT8, w, K / 2, N, K / 2, 64, RB / 2,
-                   CU_TENSOR_MAP_SWIZZLE_64B);
-    if (rc != W4A16_OK) return rc;
-    GemvParams p;
+GemvParams gemv_params(const DeviceState& st, const void* s, void* out, int64_t M, int64_t N,
+                       int64_t K, int64_t g, const Epilogue& epi) {
+    GemvParams p{};
     p.scales = static_cast<const uint16_t*>(s);
     p.out = static_cast<uint16_t*>(out);
     p.status = st.status;
@@ -249,32 +228,89 @@ int launch_gemv(const DeviceState& st, const void* x, const void* w, const void*
     p.N = static_cast<int>(N);
     p.K = static_cast<int>(K);
     p.g = static_cast<int>(g);
-    p.rows_per_cta = RB;
-    p.num_chunks = static_cast<int>((N + RB - 1) / RB);
-    p.nt = (RB + 127) / 128;
     p.epi = epi;
     p.wait_ns = wait_limit_ns();
-    const cudaError_t e = tc ? gemv_tc_launch(&tx, &tw, p, st.sm_count, stream)
-                             : gemv_launch(&tx, &tw, p, st.sm_count, stream);
-    return e == cudaSuccess ? W4A16_OK : W4A16_ERR_CUDA;
+    return p;
+}
+
+// M <= 16, g = 128: the warp-level streaming kernel.
+int launch_gemv(const DeviceState& st, const void* x, const void* w, const void* s, void* out,
+                int64_t M, int64_t N, int64_t K, int64_t g, const Epilogue& epi,
+                cudaStream_t stream) {
+    const int RB = gemv_rows_per_cta(N, st.sm_count);
+    alignas(64) CUtensorMap tx;
+    alignas(64) CUtensorMap tw;
+    int rc = encode_2d(&tx, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, x, K, M, K * 2, 64,
+                       gemv_tokens_per_tile(M), CU_TENSOR_MAP_SWIZZLE_128B);
+    if (rc != W4A16_OK) return rc;
+    rc = encode_2d(&tw, CU_TENSOR_MAP_DATA_TYPE_UINT8, w, K / 2, N, K / 2, 64, RB / 2,
+                   CU_TENSOR_MAP_SWIZZLE_64B);
+    if (rc != W4A16_OK) return rc;
+    GemvParams p = gemv_params(st, s, out, M, N, K, g, epi);
+    p.rows_per_cta = RB;
+    p.num_chunks = static_cast<int>((N + RB - 1) / RB);
+    return gemv_launch(&tx, &tw, p, st.sm_count, stream) == cudaSuccess ? W4A16_OK
+                                                                       : W4A16_ERR_CUDA;
+}
+
+// The tensor-core streaming kernel.
+int launch_gemv_tc(const DeviceState& st, const GemvTcPlan& plan, const void* x, const void* w,
+                   const void* s, void* out, int64_t M, int64_t N, int64_t K, int64_t g,
+                   const Epilogue& epi, cudaStream_t stream) {
+    const int RB = plan.rows_per_cta;
+    alignas(64) CUtensorMap tx;
+    alignas(64) CUtensorMap tw;
+    int rc = encode_2d(&tx, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, x, K, M, K * 2, 64, plan.tokens,
+                       CU_TENSOR_MAP_SWIZZLE_128B);
+    if (rc != W4A16_OK) return rc;
+    rc = encode_2d(&tw, CU_TENSOR_MAP_DATA_TYPE_UINT8, w, K / 2, N, K / 2, 64, RB / 2,
+                   CU_TENSOR_MAP_SWIZZLE_64B);
+    if (rc != W4A16_OK) return rc;
+    GemvParams p = gemv_params(st, s, out, M, N, K, g, epi);
+    p.rows_per_cta = RB;
+    p.num_chunks = plan.num_chunks;
+    p.nt = (RB + 127) / 128;
+    p.row_chunks = plan.row_chunks;
+    p.split = plan.split;
+    return gemv_tc_launch(&tx, &tw, p, plan.tokens, st.sm_count, stream) == cudaSuccess
+               ? W4A16_OK
+               : W4A16_ERR_CUDA;
 }
 
 // Validated arguments -> one kernel launch.
 int launch_linear(const DeviceState& st, const void* x, const void* w, const void* s, void* out,
                   int64_t M, int64_t N, int64_t K, int64_t g, const Epilogue& epi,
                   cudaStream_t stream) {
-    // up to 128 tokens the weights stream once per call on the streaming
-    // tensor-core kernel (12288 x 49152: M = 64 103 us there against 212 on the
-    // 256-token GEMM tiles, M = 128 141 against 214)
-    if (M <= 128 && g == 128 && K % 128 == 0 && g_small_m_streaming)
-        return launch_gemv(st, x, w, s, out, M, N, K, g, epi, stream);
-    const TsVariant v = M <= 32                      ? TsVariant::kGemv32
-                        : g_gemm_pair && (g_gemm_wide_from >= 0
-                                              ? M >= g_gemm_wide_from
-                                              : ts_prefer_wide(M, N, st.sm_count))
+    // Up to 128 tokens the weights stream once per call on the streaming kernels
+    // (12288 x 49152: M = 64 81 us there against 212 on the 256-token GEMM tiles,
+    // M = 128 112 against 214).  M <= 16: the warp-level kernel has the higher rate
+    // where every SM has many rows (M = 8: N = 49152 65 us against 73, 36864 53
+    // against 61), the tcgen05 one on narrow layers, whose K it splits (24576 47
+    // against 39, 12288 34 against 24, K = 49152 126 against 73) and from 9 tokens
+    // on (M = 16: N = 49152 81 against 74, 36864 65 against 61).
+    if (M <= 128) {
+        const GemvTcPlan plan = gemv_tc_plan(M, N, K, st.sm_count);
+        const bool rows = M <= 16 && g == 128 &&
+                          (g_small_m == 0 ? gemv_cost_us(M, N, K, st.sm_count) < plan.cost_us
+                                          : g_small_m == 'm');
+        return rows ? launch_gemv(st, x, w, s, out, M, N, K, g, epi, stream)
+                    : launch_gemv_tc(st, plan, x, w, s, out, M, N, K, g, epi, stream);
+    }
+    // Beyond that too, in tiles of up to 128 tokens, where the GEMM's CTA pairs do
+    // not fill the GPU (few weight rows, or a nearly empty last wave), by the two
+    // modelled times: 12288 x 12288 at M = 130 49 us against 69, 333 68 against 95,
+    // 512 108 against 136; at 1024 240 against 200, where the GEMM stays.
+    if (g_gemm_pair && g_gemm_wide_from < 0) {
+        const GemvTcPlan plan = gemv_tc_plan(M, N, K, st.sm_count);
+        if (plan.cost_us < 0.95 * ts_cost_us(M, N, K, st.sm_count))
+            return launch_gemv_tc(st, plan, x, w, s, out, M, N, K, g, epi, stream);
+    }
+    const TsVariant v = g_gemm_pair && (g_gemm_wide_from >= 0
+                                            ? M >= g_gemm_wide_from
+                                            : ts_prefer_wide(M, N, st.sm_count))
                             ? TsVariant::kGemmPairWide
-                        : g_gemm_pair                ? TsVariant::kGemmPair
-                                                     : TsVariant::kGemm256;
+                        : g_gemm_pair ? TsVariant::kGemmPair
+                                      : TsVariant::kGemm256;
     const int T = ts_tokens_per_tile(v);
     alignas(64) CUtensorMap tx;
     alignas(64) CUtensorMap tw;
@@ -295,8 +331,8 @@ int launch_linear(const DeviceState& st, const void* x, const void* w, const voi
     p.num_t_tiles = static_cast<int>((M + T - 1) / T);
     p.num_w_tiles = static_cast<int>((N + 127) / 128);
     p.num_tiles = p.num_t_tiles * p.num_w_tiles;
-    p.group_t = v == TsVariant::kGemv32 ? 1 : v == TsVariant::kGemmPairWide ? g_group_t_wide : g_group_t;
-    if (v != TsVariant::kGemv32 && g_group_bytes > 0) {
+    p.group_t = v == TsVariant::kGemmPairWide ? g_group_t_wide : g_group_t;
+    if (g_group_bytes > 0) {
         const int64_t per_tile = static_cast<int64_t>(T) * K * 2;
         const int64_t gt = g_group_bytes / per_tile;
         p.group_t = static_cast<int>(gt < 1 ? 1 : gt > 64 ? 64 : gt);

@@ -1,5 +1,8 @@
-// Small-M (M <= 32) int4-dequant + matmul for sm_103a: the bandwidth-bound
-// regime where the whole packed weight matrix streams from HBM once per call.
+// Small-M (M <= 16, g = 128) int4-dequant + matmul for sm_103a: the bandwidth-bound
+// regime where the whole packed weight matrix streams from HBM once per call, for
+// layers with enough rows to give every SM some 180 and more (below that, and from 9
+// tokens on where the rows are many, gemv_tc.cu's split of K over clusters is faster;
+// gemv_cost_us).
 //
 // Design, GB300-first:
 //   - persistent grid, one CTA per SM; CTA c owns a contiguous range of RB
@@ -7,7 +10,7 @@
 //     of bytes -- no tile-count quantisation;
 //   - one shared-memory stage covers 128 k = one scale group (g = 128): two
 //     TMA boxes of RB/2 rows x 64 B of packed weights (64-byte swizzle) and
-//     two 128-byte-swizzled boxes of x (T = 8, 16 or 32 token rows; rows >= M
+//     two 128-byte-swizzled boxes of x (T = 8 or 16 token rows; rows >= M
 //     are TMA zero fill); warp 0 keeps S stages in flight;
 //   - warp 1 reorders each staged x chunk once, in place, into the pair order
 //     the weight codes come out in (below), for all compute warps;
@@ -57,12 +60,6 @@
 #endif
 #ifndef W4A16_GEMV_U2
 #define W4A16_GEMV_U2 4
-#endif
-#ifndef W4A16_GEMV_S4
-#define W4A16_GEMV_S4 6
-#endif
-#ifndef W4A16_GEMV_U4
-#define W4A16_GEMV_U4 2
 #endif
 
 namespace w4a16 {
@@ -133,7 +130,7 @@ __device__ __forceinline__ float scale_at(const uint32_t (&blk)[W], int e) {
     }
 }
 
-// NT: 8-token MMA column tiles (T = 8 NT staged token rows); S: stage slots;
+// NT: 8-token MMA column tiles (T = 8 NT staged token rows, NT = 1 or 2); S: stage slots;
 // U: stages per unrolled round of the K loop, and scale groups per load (a
 // divisor of S); FUSED: the fused epilogue (bias, activation, residual).
 template <int NT, int S, int U, bool FUSED>
@@ -225,6 +222,11 @@ __global__ void __launch_bounds__(kMaxThreads, 1)
                         tma_load_2d(ws, &tmap_w, full(s), kk * (kBKS / 2), row0);
                         tma_load_2d(ws + L::W_HALF, &tmap_w, full(s), kk * (kBKS / 2),
                                     row0 + RB / 2);
+                    }
+                    if (it == 0 && !short_limit_ok(full(0), 0, abort_flag, p.status, p.wait_ns)) {
+                        ok = false;
+                        ++it;
+                        break;
                     }
                     if (++kk == KS) kk = 0;
                 }
@@ -518,16 +520,25 @@ int gemv_rows_per_cta(int64_t N, int sm_count) {
     return static_cast<int>(per);
 }
 
-int gemv_tokens_per_tile(int64_t M) { return M <= 8 ? 8 : M <= 16 ? 16 : 32; }
+double gemv_cost_us(int64_t M, int64_t N, int64_t K, int sm_count) {
+    const int64_t rb = gemv_rows_per_cta(N, sm_count);
+    const int64_t waves = ((N + rb - 1) / rb + sm_count - 1) / sm_count;
+    // per 128-k stage: a fixed part and one per row (K = 12288, M <= 8: 65.0 us in all
+    // at 324 rows per CTA, 52.8 at 244, 46.5 at 162, 33.8 at 82; M = 9..16: 81, 65,
+    // 59; K = 49152 at 82 rows 126 and 148)
+    const double stage = M <= 8 ? 0.20 + 0.00134 * static_cast<double>(rb)
+                                : 0.25 + 0.0017 * static_cast<double>(rb);
+    return 4.0 + static_cast<double>(waves * (K / kBKS)) * stage;
+}
+
+int gemv_tokens_per_tile(int64_t M) { return M <= 8 ? 8 : 16; }
 
 cudaError_t gemv_launch(const CUtensorMap* tx, const CUtensorMap* tw, const GemvParams& p,
                         int sm_count, cudaStream_t stream) {
     const int grid = p.num_chunks < sm_count ? p.num_chunks : sm_count;
     if (p.M <= 8)
         return launch_gemv_variant<1, W4A16_GEMV_S1, W4A16_GEMV_U1>(tx, tw, p, grid, stream);
-    if (p.M <= 16)
-        return launch_gemv_variant<2, W4A16_GEMV_S2, W4A16_GEMV_U2>(tx, tw, p, grid, stream);
-    return launch_gemv_variant<4, W4A16_GEMV_S4, W4A16_GEMV_U4>(tx, tw, p, grid, stream);
+    return launch_gemv_variant<2, W4A16_GEMV_S2, W4A16_GEMV_U2>(tx, tw, p, grid, stream);
 }
 
 }  // namespace w4a16

@@ -1,46 +1,50 @@
-// Small-M (M <= 128, g = 128) int4-dequant + matmul on the 5th-generation
-// tensor core: the regime where the whole packed weight matrix streams from
-// HBM once per call (the GEMM's 256-token tiles would leave most of their
-// columns empty and split the weight rows unevenly over the SMs).
+// Streaming int4-dequant + matmul on the 5th-generation tensor core for few
+// tokens (M = 17..128, every group size, and more tokens in 128-token tiles
+// where the GEMM's CTA pairs would leave SMs idle): the regime where the whole
+// packed weight matrix streams from HBM about once per call.
 //
 // out[m, n] = sum_k x[m, k] * wd[n, k],   wd = RNE_bf16((q[n, k] - 8) * s[n, k / g])
 //
 // (the same weights as w4a16_dequant and the large-M GEMM: the result differs
 // from theirs only in the fp32 summation order).
 //
-// Why the tensor core here: at M = 16-32 tokens the matmul is 19-39 GFLOP per
-// call, and warp-level mma.sync runs at ~610 TFLOP/s on this GPU -- 32-64 us,
-// more than the ~46 us the weights take to stream.  tcgen05.mma runs
-// asynchronously, leaving the SM's integer and half-precision pipes to the
-// dequantisation.
-//
 // Per CTA (persistent, one per SM): a contiguous range of RB <= 384 weight
-// rows (RB = N / #SMs rounded up to even), as three MMA tiles of 128 rows,
-// each with ONE fp32 accumulator of NTOK = 16, 32, 64 or 128 token columns in
-// tensor memory for the whole K walk.
-// Per scale group of 128 k:
+// rows as up to three MMA tiles of 128 rows, each with one fp32 accumulator of
+// NTOK = 32 to 128 token columns in tensor memory for the whole K walk.
+// Per stage of 128 k:
 //   warp 0      TMA: two 64-k boxes of x (NTOK token rows, 128-byte swizzle,
 //               rows >= M zero-filled) and two boxes of RB/2 rows x 64 B of
 //               packed weights (64-byte swizzle) into a ring of S stages;
-//   warp 2      reorders each staged x chunk in place into the (k, k+4) pair
-//               order in which the codes come out of a packed word;
-//   warps 4-15  dequant: thread = one weight row of one tile (its TMEM lane);
-//               per scale group, 16 words -> bf16 pairs (q - 8) * s (shift,
-//               three-input LOP3, one bf16x2 subtraction and one bf16x2
-//               multiply per pair) -> tcgen05.st into a ring of SA A stages
-//               (one per group);
-//               after the last group, the epilogue: tcgen05.ld of the row's
-//               NTOK accumulators in slices of up to 32, each slice's (fused)
-//               epilogue from registers;
-//   warps 1, 3, 16  one thread each, one per tile, issues
-//               D_t[128 x NTOK] += A_t[128 x 16] x B[NTOK x 16]^T (A from
-//               tensor memory, B = x in shared memory), 8 MMAs per group,
-//               accumulating into its tile's accumulator.
-// With the scale applied in the dequant there is no per-group accumulator to
-// fold: nothing waits on the MMAs inside the K walk except the A ring.  A
-// single thread issues these small MMAs at ~130 SM clocks each, slower than
-// the tensor pipe runs them, hence one issuing thread (and one A ring and
-// accumulator hand-off) per tile.
+//   warps 4..   dequant: thread = one weight row of one tile (its TMEM lane);
+//               wd as bf16 pairs in k order (one FMA per pair, dequant.cuh) ->
+//               tcgen05.st into the tile's ring of SA A stages of AK k; after the last
+//               stage, the epilogue: tcgen05.ld of the row's accumulators in slices
+//               of 32 tokens, each slice's (fused) epilogue from registers;
+//   warps 1..3  one per tile: D_t[128 x NTOK] += A_t[128 x 16] x B[NTOK x 16]^T (A
+//               from tensor memory, B = x in shared memory).  One commit frees
+//               the A stage, one the TMA stage (x by the MMAs, the weights by the
+//               row warps before them).
+// Narrow layers split K: `split` CTAs of a cluster share one chunk of rows, each
+// walks its slice of K, and the partial sums meet in distributed shared memory, 32
+// tokens at a time, each CTA finishing its share of them in the order of the
+// ranks (deterministic).  12288 rows on 152 SMs are 82 rows, one 128-row tile, per
+// CTA without a split, and a lone tile runs at the latency of its four row
+// warps (0.47 us per stage whatever M): K = 49152 at M = 100 with bias and residual 398
+// us (before) -> 126 us (clusters of 4, 342 rows each); 12288 x 12288 at M = 24
+// 56 -> 24 us.
+//
+// What bounds it (K = 12288, 152 SMs): the row warps' latency and issue slots, not the
+// tensor pipe: a stage costs 0.45-0.48, 0.60-0.73, 0.73-1.13 us for one, two, three
+// tiles (N = 49152: 74 us at M <= 32, 81 at 64, 88 at 90, 106 at 100, 112 at 128;
+// before this kernel dequantised in k order, through one FMA, with no x reorder warp,
+// operands in uniform registers and addresses that only advance: 92, 103, 137, 137,
+// 139).  tcgen05.mma with A in tensor memory runs at 18 / 32 / 64 clocks for 32 / 64 /
+// 128 columns with three independent accumulators, 44 with one (measured alone), so
+// the MMAs need 0.22-0.8 us of a stage.  From 97 tokens on three tiles leave the A ring
+// only two or three slots of a quarter stage.  Measured and not kept: two groups of row
+// warps per tile (M = 24: 99 us: the A ring is too short for them), barrier polls
+// issued ahead of the dequantisation (81), one issuing warp for all tiles (92), a
+// rolled dequant loop (78).
 //
 // Every wait is bounded (ptx.cuh); on a timeout the kernel records
 // W4A16_ERR_TIMEOUT, drains its copies and MMAs, frees tensor memory and
@@ -50,21 +54,16 @@
 #include "internal.h"
 #include "ptx.cuh"
 
+#include <atomic>
+
 namespace w4a16 {
 
 namespace {
 
-constexpr int kTilesMax = 3;              // MMA tiles of 128 rows per CTA, at most
-constexpr int kGroupK = 128;              // k per TMA stage = one scale group
-constexpr int kFirstRowWarp = 4;          // warps 4..15 (warp % 4 = TMEM sub-partition)
-constexpr int kRowWarps = 4 * kTilesMax;  // dequant + epilogue warps
-constexpr int kLastIssuerWarp = kFirstRowWarp + kRowWarps;  // warp 16: tile 2's MMAs
-constexpr int kThreads = 32 * (kLastIssuerWarp + 1);
 
-// MMA-issuing warp of tile t: 1, 3, 16.
-__device__ __forceinline__ int issuer_tile(int warp) {
-    return warp == 1 ? 0 : warp == 3 ? 1 : warp == kLastIssuerWarp ? 2 : -1;
-}
+constexpr int kTilesMax = 3;      // MMA tiles of 128 rows per CTA, at most
+constexpr int kGroupK = 128;      // k per TMA stage
+constexpr int kFirstRowWarp = 4;  // warps 1..3 issue the MMAs of tiles 0..2
 
 // 32 lanes x 16 columns of 32 bits (see tmem_st_32x32b_x32).
 __device__ __forceinline__ void tmem_st_32x32b_x16(uint32_t taddr, const uint32_t* v) {
@@ -77,55 +76,127 @@ __device__ __forceinline__ void tmem_st_32x32b_x16(uint32_t taddr, const uint32_
         : "memory");
 }
 
-template <int NTOK>
+// TILES: MMA tiles of 128 rows a CTA holds (2 or 3); NTOK: token columns.
+template <int NTOK, int TILES_>
 struct TLayout {
-    static_assert(NTOK == 16 || NTOK == 32 || NTOK == 64 || NTOK == 128, "MMA N for M = 128");
-    // MMA tiles of 128 rows per CTA (with 128 tokens, two tiles and 256 rows
-    // per CTA would leave room for more A stages but need a second wave of
-    // chunks at N = 49152: 207 against 141 us)
-    static constexpr int TILES = kTilesMax;
+    static_assert(NTOK % 16 == 0 && NTOK <= 128, "MMA N for M = 128");
+    static constexpr int TILES = TILES_;
     static constexpr int ROWS_MAX = 128 * TILES;                     // rows per CTA chunk
-    static constexpr int S = NTOK == 128 ? 3 : NTOK == 64 ? 5 : NTOK == 32 ? 6 : 7;  // TMA slots
-    // k per tensor-memory A stage: a whole scale group; half of one where the
-    // 64-token accumulators leave room for three half-group slots only; a
-    // quarter where the 128-token accumulators leave room for two
-    static constexpr int AK = NTOK == 128 ? 32 : NTOK == 64 ? 64 : 128;
-    static constexpr int CHUNKS = AK / 32;  // 16-byte chunks (32 codes) per row and A stage
-    // A stage slots: as many as fit next to the accumulators
-    static constexpr int SA = NTOK == 64 ? 3 : 2;
     static constexpr int X_BOX = NTOK * 128;                         // 64 k x NTOK tokens
     static constexpr int X_BYTES = 2 * X_BOX;
     static constexpr int W_HALF = (ROWS_MAX / 2) * (kGroupK / 2);    // ROWS_MAX / 2 rows x 64 B
     static constexpr int W_BYTES = 2 * W_HALF;
     static constexpr int STAGE = X_BYTES + W_BYTES;                  // x, then the weights
-    // full_tma[S], empty_smem[S], x_ready[S], then per tile: full_a[SA],
-    // empty_a[SA], d_full, d_empty, drain
-    static constexpr int BAR_OFF = S * STAGE;
-    static constexpr int TILE_BARS = 2 * SA + 3;
-    static constexpr int NBARS = 3 * S + TILES * TILE_BARS;
-    static constexpr int MISC_OFF = BAR_OFF + NBARS * 8;
-    static constexpr int SMEM_BYTES = MISC_OFF + 16 + 1024;          // + 1024-B alignment slack
-    // tensor memory: the accumulators (TILES x NTOK columns) at column 0,
-    // then from column A_COL SA A stages (TILES x AK / 2 columns each: AK k
-    // of bf16 pairs).  A stages of a whole group (two slots) measured ~3%
-    // faster than half-group stages (four slots): half the hand-offs.
+    // TMA slots: what 224 KB hold, at most 7
+    static constexpr int S_FIT = (222 * 1024) / STAGE;
+    static constexpr int S = S_FIT < 7 ? S_FIT : 7;
+    // tensor memory: the accumulators (TILES x NTOK columns), then SA A stages
+    // of AK k (TILES x AK / 2 columns each)
     static constexpr int D_COLS = TILES * NTOK;
-    static constexpr int A_COL = NTOK == 128 ? 384 : NTOK == 64 ? 192 : 128;
+    static constexpr int A_FREE = 512 - D_COLS;
+    static constexpr int AK = A_FREE / (TILES * 64) >= 2 ? 128 : A_FREE / (TILES * 32) >= 2 ? 64 : 32;
+    static constexpr int SA = A_FREE / (TILES * (AK / 2));
+    static constexpr int SUB = kGroupK / AK;   // A stages per TMA stage
+    static constexpr int CHUNKS = AK / 32;     // 16-byte chunks (32 codes) per row and A stage
+    static constexpr int A_COL = 512 - SA * TILES * (AK / 2);
     static constexpr int A_COLS = TILES * (AK / 2);
     static constexpr int TMEM_COLS = 512;
-    static_assert(D_COLS <= A_COL && A_COL + SA * A_COLS <= TMEM_COLS,
-                  "tensor memory holds 512 columns");
+    static constexpr int ROW_WARPS = 4 * TILES;
+    static constexpr int THREADS = 32 * (kFirstRowWarp + ROW_WARPS);
+    // full_tma[S], empty_smem[S], then per tile: full_a[SA], empty_a[SA],
+    // d_full, d_empty, drain
+    static constexpr int BAR_OFF = S * STAGE;
+    static constexpr int TILE_BARS = 2 * SA + 3;
+    static constexpr int NBARS = 2 * S + TILES * TILE_BARS;
+    static constexpr int MISC_OFF = BAR_OFF + NBARS * 8;
+    static constexpr int SMEM_BYTES = MISC_OFF + 16 + 1024;          // + 1024-B alignment slack
+    // split K: partial sums of a slice of EC tokens, double-buffered, over the
+    // stages once they are consumed
+    static constexpr int EC = 32;  // (reduce_slice)
+    static constexpr int PART = ROWS_MAX * EC * 4;
+    static_assert(2 * PART <= S * STAGE, "partial sums fit the stages");
+    static_assert(SA >= 2 && D_COLS <= A_COL, "tensor memory holds 512 columns");
     static_assert(X_BOX % 1024 == 0 && W_HALF % 1024 == 0 && STAGE % 1024 == 0,
                   "swizzled boxes keep 1024-byte alignment");
-    static_assert(SMEM_BYTES <= 227 * 1024, "shared memory");
+    static_assert(S >= 2 && SMEM_BYTES <= 227 * 1024, "shared memory");
 };
 
-template <int NTOK, bool FUSED>
-__global__ void __launch_bounds__(kThreads, 1)
+__device__ __forceinline__ float ld_shared_cluster_f32(uint32_t addr) {
+    float v;
+    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
+    return v;
+}
+
+// Residual of one row (lane) and token m of the fused epilogue, 0 where there is none.
+// Read for a whole slice before any of its outputs is stored: the residual may be
+// the output, so the compiler keeps loads and stores in order, and one at a time they
+// are a chain of memory latencies (333 x 12288 x 12288 with a residual 117 us, 93 so).
+template <bool FUSED>
+__device__ __forceinline__ float residual_at(const GemvParams& p, int m, int m_end, int n,
+                                             bool valid, int lane) {
+    const Epilogue& ep = p.epi;
+    const bool glu = ep.act == kActSwiGLU;
+    if (!FUSED || ep.residual == nullptr || !valid || m >= m_end || (glu && (lane & 1) != 0))
+        return 0.0f;
+    return bf16_to_f32(ep.residual[static_cast<int64_t>(m) * ep.n_out + (glu ? n >> 1 : n)]);
+}
+
+// Output of one row (lane) and token m (if below m_end) from the finished sum, with
+// the fused epilogue.  SwiGLU pairs rows (n, n ^ 1) = (gate, up): RB is even, so n
+// has the parity of its lane and the partner is lane ^ 1 (all lanes call).
+template <bool FUSED>
+__device__ __forceinline__ void finish(const GemvParams& p, float acc, float bias, float residual,
+                                       int m, int m_end, int n, bool valid, int lane) {
+    const Epilogue& ep = p.epi;
+    if constexpr (!FUSED) {
+        if (valid && m < m_end) p.out[static_cast<int64_t>(m) * p.N + n] = f32_to_bf16_rn(acc);
+    } else {
+        const float z = acc + bias;
+        if (ep.act == kActSwiGLU) {
+            const float up = __shfl_xor_sync(0xffffffffu, z, 1);
+            if ((lane & 1) == 0 && valid && m < m_end)
+                p.out[static_cast<int64_t>(m) * ep.n_out + (n >> 1)] =
+                    f32_to_bf16_rn(silu_f32(z) * up + residual);
+        } else if (valid && m < m_end) {
+            const float h = ep.act == kActGELU ? gelu_f32(z) : z;
+            p.out[static_cast<int64_t>(m) * ep.n_out + n] = f32_to_bf16_rn(h + residual);
+        }
+    }
+}
+
+// Sums of one row over the SP CTAs of the cluster, in the order of the ranks,
+// and their output: the tokens [rank 32 / SP, ..) of a slice of 32.  All the
+// remote loads are issued before the first sum (one round trip per slice).
+template <int SP, bool FUSED>
+__device__ __forceinline__ void reduce_slice(const GemvParams& p, uint32_t part, int pitch, int rank,
+                                             int r, float bias, int m, int m_end, int n, bool valid,
+                                             int lane) {
+    constexpr int PER = 32 / SP;
+    float v[SP][PER], res[PER];
+#pragma unroll
+    for (int j = 0; j < PER; ++j)
+        res[j] = residual_at<FUSED>(p, m + rank * PER + j, m_end, n, valid, lane);
+#pragma unroll
+    for (int c = 0; c < SP; ++c) {
+        const uint32_t at = mapa_shared(part + 4u * (rank * PER * pitch + r), c);
+#pragma unroll
+        for (int j = 0; j < PER; ++j) v[c][j] = ld_shared_cluster_f32(at + 4u * j * pitch);
+    }
+#pragma unroll
+    for (int j = 0; j < PER; ++j) {
+        float sum = v[0][j];
+#pragma unroll
+        for (int c = 1; c < SP; ++c) sum += v[c][j];
+        finish<FUSED>(p, sum, bias, res[j], m + rank * PER + j, m_end, n, valid, lane);
+    }
+}
+
+template <int NTOK, int TILES, bool FUSED, bool SPLIT>
+__global__ void __launch_bounds__(TLayout<NTOK, TILES>::THREADS, 1)
     w4a16_gemv_tc_kernel(const __grid_constant__ CUtensorMap tmap_x,
                          const __grid_constant__ CUtensorMap tmap_w, const GemvParams p) {
-    using L = TLayout<NTOK>;
-    constexpr int S = L::S, SA = L::SA;
+    using L = TLayout<NTOK, TILES>;
+    constexpr int S = L::S, SA = L::SA, SUB = L::SUB;
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw = smem_u32(smem_raw);
     const uint32_t sbase = (raw + 1023u) & ~1023u;
@@ -138,8 +209,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     const uint32_t bars = sbase + L::BAR_OFF;
     auto full_tma = [&](int s) { return bars + 8u * s; };
     auto empty_smem = [&](int s) { return bars + 8u * (S + s); };
-    auto x_ready = [&](int s) { return bars + 8u * (2 * S + s); };
-    auto tile_bar = [&](int t, int i) { return bars + 8u * (3 * S + t * L::TILE_BARS + i); };
+    auto tile_bar = [&](int t, int i) { return bars + 8u * (2 * S + t * L::TILE_BARS + i); };
     auto full_a = [&](int t, int a) { return tile_bar(t, a); };
     auto empty_a = [&](int t, int a) { return tile_bar(t, SA + a); };
     auto d_full = [&](int t) { return tile_bar(t, 2 * SA); };
@@ -151,18 +221,16 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (threadIdx.x == 0) {
         for (int s = 0; s < S; ++s) {
             mbar_init(full_tma(s), 1);
-            // every row warp of the p.nt tiles in use has read W, and every
-            // such tile's MMAs have read x
-            mbar_init(empty_smem(s), 5 * p.nt);
-            mbar_init(x_ready(s), 1);
+            mbar_init(empty_smem(s), p.nt);  // every tile's MMAs
         }
-        for (int t = 0; t < L::TILES; ++t) {
+        for (int t = 0; t < p.nt; ++t) {
+            const int warps = (RB - 128 * t + 31) / 32 < 4 ? (RB - 128 * t + 31) / 32 : 4;
             for (int a = 0; a < SA; ++a) {
-                mbar_init(full_a(t, a), 4);  // the tile's four row warps
+                mbar_init(full_a(t, a), warps);  // the row warps of the stage's group
                 mbar_init(empty_a(t, a), 1);
             }
             mbar_init(d_full(t), 1);
-            mbar_init(d_empty(t), 4);
+            mbar_init(d_empty(t), warps);
             mbar_init(drain(t), 1);
         }
         *abort_flag = 0;
@@ -179,24 +247,40 @@ __global__ void __launch_bounds__(kThreads, 1)
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
 
-    const int KS = p.K / kGroupK;  // scale groups = stages per chunk
-    // Each CTA walks K from its own starting group, so that the CTAs read
+    // The CTA's stages: all of K, or its slice of it among the CTAs of the
+    // cluster; walked from a starting point of its own, so that the CTAs read
     // different x slices from L2 at any moment.
-    const int rot = static_cast<int>(static_cast<int64_t>(blockIdx.x) * KS / gridDim.x);
+    const int KS = (p.K + kGroupK - 1) / kGroupK;
+    const int rank = SPLIT ? static_cast<int>(cluster_ctarank()) : 0;
+    const int k_first = SPLIT ? static_cast<int>(static_cast<int64_t>(KS) * rank / p.split) : 0;
+    const int k_count =
+        (SPLIT ? static_cast<int>(static_cast<int64_t>(KS) * (rank + 1) / p.split) : KS) - k_first;
+    const int chunk0 = SPLIT ? static_cast<int>(blockIdx.x) / p.split : static_cast<int>(blockIdx.x);
+    const int chunk_step = SPLIT ? p.num_chunks : static_cast<int>(gridDim.x);
+    const int rot = k_first + static_cast<int>(static_cast<int64_t>(chunk0) * k_count / chunk_step);
+    const int k_end = k_first + k_count;
+
+    const int row_tile = (warp - kFirstRowWarp) >> 2;             // row warps: MMA tile
+    // warps wholly past the chunk's rows do nothing
+    const bool row_warp = warp >= kFirstRowWarp && row_tile * 128 + (warp & 3) * 32 < RB;
+    const int sub = warp & 3;                                     // TMEM sub-partition
+    const int r = row_tile * 128 + sub * 32 + lane;               // local row
+    const uint32_t lane_base = tmem + (static_cast<uint32_t>(sub * 32) << 16);
+    bool ok = true;
 
     if (warp == 0) {
         // ------------------------------------------------------------ TMA producer
         if (lane == 0) {
             const uint32_t tx = L::X_BYTES + static_cast<uint32_t>(RB) * (kGroupK / 2);
             uint32_t it = 0;
-            bool ok = true;
-            for (int chunk = blockIdx.x; ok && chunk < p.num_chunks; chunk += gridDim.x) {
-                const int row0 = chunk * RB;
+            for (int chunk = chunk0; ok && chunk < p.num_chunks; chunk += chunk_step) {
+                const int tt = chunk / p.row_chunks;
+                const int row0 = (chunk - tt * p.row_chunks) * RB, m0 = tt * NTOK;
                 int kk = rot;
-                for (int g = 0; g < KS; ++g, ++it) {
+                for (int g = 0; g < k_count; ++g, ++it) {
                     const int s = it % S;
-                    if (!wait_one(empty_smem(s), ((it / S) & 1u) ^ 1u, abort_flag, p.status,
-                                  p.wait_ns)) {
+                    if (!wait_one<false, 64>(empty_smem(s), ((it / S) & 1u) ^ 1u, abort_flag,
+                                             p.status, p.wait_ns)) {
                         ok = false;
                         break;
                     }
@@ -207,8 +291,8 @@ __global__ void __launch_bounds__(kThreads, 1)
                                       tma_box_ok(st + L::X_BOX, L::X_BOX, 1024, sbase, end,
                                                  kk * kGroupK + 64, 2),
                                   p.status)) {
-                        tma_load_2d(st, &tmap_x, full_tma(s), kk * kGroupK, 0);
-                        tma_load_2d(st + L::X_BOX, &tmap_x, full_tma(s), kk * kGroupK + 64, 0);
+                        tma_load_2d(st, &tmap_x, full_tma(s), kk * kGroupK, m0);
+                        tma_load_2d(st + L::X_BOX, &tmap_x, full_tma(s), kk * kGroupK + 64, m0);
                     }
                     const uint32_t wbox = static_cast<uint32_t>(RB / 2) * (kGroupK / 2);
                     if (dbg_check(wbox <= L::W_HALF &&
@@ -222,249 +306,285 @@ __global__ void __launch_bounds__(kThreads, 1)
                         tma_load_2d(st + L::X_BYTES + L::W_HALF, &tmap_w, full_tma(s),
                                     kk * (kGroupK / 2), row0 + RB / 2);
                     }
-                    if (++kk == KS) kk = 0;
+                    if (it == 0 &&
+                        !short_limit_ok(full_tma(0), 0, abort_flag, p.status, p.wait_ns)) {
+                        ok = false;
+                        ++it;
+                        break;
+                    }
+                    if (++kk == k_end) kk = k_first;
                 }
             }
             // every load this thread issued has landed before exit
             const uint32_t last = it < static_cast<uint32_t>(S) ? it : S;
             for (uint32_t i = it - last; i < it; ++i) settle(full_tma(i % S), (i / S) & 1u);
         }
-    } else if (issuer_tile(warp) >= 0) {
+    } else if (warp < kFirstRowWarp) {
         // ------------------------------------------------------------ MMA issuers
-        // (tiles past the chunk's rows, t >= p.nt, are not computed)
-        const int t = issuer_tile(warp);
-        if (lane == 0 && t < p.nt && t < L::TILES) {
+        // one thread per tile; tiles past the chunk's rows, t >= p.nt, are not computed
+        // (whole warps run the loops, so that the operands stay in uniform registers)
+        const int t = warp - 1;
+        if (t < p.nt) {
             constexpr uint32_t idesc = idesc_bf16_f32(128, NTOK);
-            uint32_t it = 0, ia = 0, nchunk = 0;
-            bool ok = true, issued = false;
-            for (int chunk = blockIdx.x; ok && chunk < p.num_chunks;
-                 chunk += gridDim.x, ++nchunk) {
+            int s = 0, a = 0;
+            uint32_t pa = 0, nchunk = 0;
+            bool issued = false;
+            for (int chunk = chunk0; ok && chunk < p.num_chunks; chunk += chunk_step, ++nchunk) {
                 // the epilogue has read the previous chunk's accumulators
                 if (nchunk > 0 &&
-                    !wait_one(d_empty(t), (nchunk - 1u) & 1u, abort_flag, p.status, p.wait_ns)) {
+                    !wait_warp(d_empty(t), (nchunk - 1u) & 1u, abort_flag, p.status, p.wait_ns)) {
                     ok = false;
                     break;
                 }
-                tc_fence_after();
-                for (int g = 0; ok && g < KS; ++g, ++it) {
-                    const int s = it % S;
-                    if (!wait_one(x_ready(s), (it / S) & 1u, abort_flag, p.status, p.wait_ns)) {
-                        ok = false;
-                        break;
-                    }
-                    tc_fence_after();
+                for (int g = 0; ok && g < k_count; ++g) {
                     const uint64_t bdesc = sdesc_kmajor_sw128(sbase + s * L::STAGE);
-                    for (int h = 0; h < kGroupK / L::AK; ++h, ++ia) {
-                        const int a = ia % SA;
-                        if (!wait_one(full_a(t, a), (ia / SA) & 1u, abort_flag, p.status,
-                                      p.wait_ns)) {
+#pragma unroll
+                    for (int h = 0; h < SUB; ++h) {
+
+                        // the A stage is written; its row warps waited for the
+                        // stage's copies, so x has landed too
+                        if (!wait_warp(full_a(t, a), pa, abort_flag, p.status, p.wait_ns)) {
                             ok = false;
                             break;
                         }
                         tc_fence_after();
+                        const uint32_t a_tm = tmem + L::A_COL + a * L::A_COLS + t * (L::AK / 2);
+                        if (elect_one()) {
 #pragma unroll
-                        for (int ks = 0; ks < L::AK / 16; ++ks) {
-                            // k offset in the group -> x box (64 k) and 32-byte step
-                            // in it; the descriptor's start address is in 16-byte units
-                            const int kg = h * L::AK + ks * 16;
-                            tc_mma_ts(tmem + t * NTOK,
-                                      tmem + L::A_COL + a * L::A_COLS + t * (L::AK / 2) + ks * 8,
-                                      bdesc + static_cast<uint64_t>(
-                                                  ((kg >> 6) * L::X_BOX + (kg & 63) * 2) >> 4),
-                                      idesc, (g | h | ks) != 0);
+                            for (int ks = 0; ks < L::AK / 16; ++ks) {
+                                // k offset in the group -> x box (64 k) and 32-byte step
+                                // in it; the descriptor's start address is in 16-byte units
+                                const int kg = h * L::AK + ks * 16;
+                                tc_mma_ts(tmem + t * NTOK, a_tm + ks * 8,
+                                          bdesc + static_cast<uint64_t>(
+                                                      ((kg >> 6) * L::X_BOX + (kg & 63) * 2) >> 4),
+                                          idesc, (g | h | ks) != 0);
+                            }
+                            tc_commit(empty_a(t, a));
+                            // the stage's x and, before it, its weights are read
+                            if (h == SUB - 1) tc_commit(empty_smem(s));
                         }
+                        __syncwarp();
                         issued = true;
-                        tc_commit(empty_a(t, a));
+                        if (++a == SA) a = 0, pa ^= 1u;
                     }
-                    if (!ok) break;
-                    tc_commit(empty_smem(s));
+                    if (++s == S) s = 0;
                 }
                 if (!ok) break;
-                tc_commit(d_full(t));  // the chunk's accumulators of tile t are final
+                if (elect_one()) tc_commit(d_full(t));  // the chunk's accumulators of tile t are final
+                __syncwarp();
             }
             if (issued) {
                 // every MMA issued has completed before tensor memory is freed
-                tc_commit(drain(t));
-                settle(drain(t), 0);
-            }
-        }
-    } else if (warp == 2) {
-        // ------------------------------------------------------------ x reorder
-        // Every 16-byte chunk (x0..x7) of the stage's x boxes becomes
-        // (x0,x4),(x1,x5),(x2,x6),(x3,x7): the pair order of codes_signed.
-        constexpr int kChunks = L::X_BYTES / 16;
-        static_assert(kChunks % 32 == 0, "whole chunks per lane");
-        uint32_t it = 0;
-        bool ok = true;
-        for (int chunk = blockIdx.x; ok && chunk < p.num_chunks; chunk += gridDim.x) {
-            for (int g = 0; g < KS; ++g, ++it) {
-                const int s = it % S;
-                if (!wait_warp(full_tma(s), (it / S) & 1u, abort_flag, p.status, p.wait_ns)) {
-                    ok = false;
-                    break;
+                if (elect_one()) {
+                    tc_commit(drain(t));
+                    settle(drain(t), 0);
                 }
-                uint4* xs = reinterpret_cast<uint4*>(smem + s * L::STAGE);
-#pragma unroll
-                for (int i = 0; i < kChunks / 32; ++i)
-                    xs[lane + 32 * i] = interleave_chunk(xs[lane + 32 * i]);
-                // these generic writes precede the MMAs' async-proxy reads
-                fence_proxy_async_smem();
                 __syncwarp();
-                if (lane == 0) mbar_arrive(x_ready(s));
             }
         }
-    } else if (warp >= kFirstRowWarp && warp < kLastIssuerWarp &&
-               (warp - kFirstRowWarp) / 4 < p.nt && (warp - kFirstRowWarp) / 4 < L::TILES) {
+    } else if (row_warp) {
         // ------------------------------------------------------------ dequant + epilogue
-        const int t = (warp - kFirstRowWarp) >> 2;  // MMA tile
-        const int sub = warp & 3;                   // TMEM sub-partition
-        const int r = t * 128 + sub * 32 + lane;    // local row
-        const uint32_t lane_base = tmem + (static_cast<uint32_t>(sub * 32) << 16);
-        // the row's four 16-byte chunks in a stage (64-byte swizzle)
+        const int t = row_tile;
+        // the row's four 16-byte chunks in a stage (64-byte swizzle: chunk j of row rr
+        // sits at j ^ ((rr >> 1) & 3))
         const bool in_range = r < RB;
         const int bx = r >= RB / 2 ? 1 : 0;
         const int rr = in_range ? r - bx * (RB / 2) : 0;
-        const uint32_t row_off = L::X_BYTES + bx * L::W_HALF + rr * (kGroupK / 2);
-        const uint32_t swz = static_cast<uint32_t>((rr >> 1) & 3);
-        uint32_t it = 0, ia = 0, nchunk = 0;
-        bool ok = true;
-        for (int chunk = blockIdx.x; ok && chunk < p.num_chunks; chunk += gridDim.x, ++nchunk) {
-            const int n = chunk * RB + r;
+        const uint32_t w_first = sbase + L::X_BYTES + bx * L::W_HALF + rr * (kGroupK / 2);
+        uint32_t c_off[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) c_off[i] = 16u * (static_cast<uint32_t>(i) ^ ((rr >> 1) & 3));
+        const int KG = p.K / p.g;      // scales per row
+        const int upg = p.g >> 6;      // 64-k halves of a stage per scale group
+        // running stage and A slots (addresses that advance by a constant and wrap)
+        uint32_t w_at = w_first, full_at = full_tma(0), ph = 0;
+        uint32_t empty_at = empty_a(t, 0), a_at = lane_base + L::A_COL + t * (L::AK / 2), pa = 1;
+        uint32_t nchunk = 0;
+        for (int chunk = chunk0; ok && chunk < p.num_chunks; chunk += chunk_step, ++nchunk) {
+            const int tt = chunk / p.row_chunks;
+            const int n = (chunk - tt * p.row_chunks) * RB + r;
             const bool valid = in_range && n < p.N;
-            // the row's scales in the rotated group order, one group ahead
-            const uint16_t* srow = p.scales + static_cast<int64_t>(valid ? n : 0) * KS;
+            // the row's scales of a stage's two 64-k halves (equal when g is a
+            // multiple of 128), loaded a stage ahead; rows past the range
+            // compute on other rows' data, their sums are never stored
+            const uint16_t* srow = p.scales + static_cast<int64_t>(valid ? n : 0) * KG;
             int kk = rot;
-            uint16_t s_next = __ldg(srow + kk);
-            for (int g = 0; ok && g < KS; ++g, ++it) {
-                const int s = it % S;
-                const uint32_t s2 = valid ? splat_bf16(s_next) : 0u;
-                if (++kk == KS) kk = 0;
-                if (g + 1 < KS) s_next = __ldg(srow + kk);
-                if (!wait_warp(full_tma(s), (it / S) & 1u, abort_flag, p.status, p.wait_ns)) {
+            uint16_t n_lo, n_hi;
+            auto load_scales = [&]() {
+                if (upg == 2) {
+                    n_lo = __ldg(srow + kk);
+                } else {
+                    const int lo = 2 * kk / upg, hi = (2 * kk + 1) / upg;
+                    n_lo = __ldg(srow + lo);
+                    // K ends in the middle of the stage: its second half is zero
+                    n_hi = hi < KG ? __ldg(srow + hi) : static_cast<uint16_t>(0);
+                }
+                if (++kk == k_end) kk = k_first;
+            };
+            load_scales();
+            for (int left = k_count; left > 0; --left) {
+                uint32_t s2_lo = splat_bf16(n_lo), s2_hi = s2_lo;
+                ScaleFma f_lo = scale_fma(s2_lo), f_hi = f_lo;
+                bool w_scale = scale_is_wide(n_lo);
+                if (upg != 2) {
+                    s2_hi = splat_bf16(n_hi);
+                    f_hi = scale_fma(s2_hi);
+                    w_scale = w_scale || scale_is_wide(n_hi);
+                }
+                load_scales();
+                const bool wide = __any_sync(0xffffffffu, w_scale);
+                if (!wait_warp(full_at, ph, abort_flag, p.status, p.wait_ns)) {
                     ok = false;
                     break;
                 }
-                const uint32_t wrow = sbase + s * L::STAGE + row_off;
-                for (int h = 0; h < kGroupK / L::AK; ++h, ++ia) {
-                    const int a = ia % SA;
-                    // code 8 everywhere: rows past the range are zero
+#pragma unroll
+                for (int h = 0; h < SUB; ++h) {
                     uint4 c[L::CHUNKS];
 #pragma unroll
-                    for (int i = 0; i < L::CHUNKS; ++i) {
-                        c[i] = make_uint4(0x88888888u, 0x88888888u, 0x88888888u, 0x88888888u);
-                        if (valid)
-                            c[i] = lds128(wrow + 16u * (static_cast<uint32_t>(L::CHUNKS * h + i) ^ swz));
-                    }
-                    if (!wait_warp(empty_a(t, a), ((ia / SA) & 1u) ^ 1u, abort_flag, p.status,
-                                   p.wait_ns)) {
-                        ok = false;
-                        break;
-                    }
-                    tc_fence_after();
-                    // per 32 codes: exact q - 8 pairs, then wd = RNE_bf16((q - 8) * s)
-                    // (one rounding), stored as 32 x 16 bf16 pairs of the row's lane
-                    const bool st_ok =
-                        dbg_check(L::A_COL + a * L::A_COLS + (t + 1) * (L::AK / 2) <= L::TMEM_COLS,
-                                  p.status);
-                    if constexpr (L::CHUNKS == 1) {
-                        uint32_t v[16];
-                        codes_signed(c[0].x, v + 0);
-                        codes_signed(c[0].y, v + 4);
-                        codes_signed(c[0].z, v + 8);
-                        codes_signed(c[0].w, v + 12);
+                    for (int i = 0; i < L::CHUNKS; ++i) c[i] = lds128(w_at + c_off[L::CHUNKS * h + i]);
+                    const bool st_ok = dbg_check(
+                        (a_at & 0xFFFFu) + L::AK / 2 <= (tmem & 0xFFFFu) + L::TMEM_COLS, p.status);
+                    // wd = RNE_bf16((q - 8) * s), as bf16 pairs of the row's lane
+                    constexpr int CS = L::CHUNKS == 1 ? 1 : 2;  // chunks per store
 #pragma unroll
-                        for (int j = 0; j < 16; ++j) v[j] = bf16x2_mul(v[j], s2);
-                        if (st_ok)
-                            tmem_st_32x32b_x16(lane_base + L::A_COL + a * L::A_COLS + t * (L::AK / 2),
-                                               v);
-                    } else {
+                    for (int i = 0; i < L::CHUNKS; i += CS) {
+                        const bool hi_half = L::CHUNKS * h + i >= 2;
+                        const ScaleFma& f = hi_half ? f_hi : f_lo;
+                        const uint32_t s2 = hi_half ? s2_hi : s2_lo;
+                        uint32_t v[16 * CS];
+                        if (!wide) {
 #pragma unroll
-                        for (int i = 0; i < L::CHUNKS; i += 2) {
-                            uint32_t v[32];
-                            codes_signed(c[i].x, v + 0);
-                            codes_signed(c[i].y, v + 4);
-                            codes_signed(c[i].z, v + 8);
-                            codes_signed(c[i].w, v + 12);
-                            codes_signed(c[i + 1].x, v + 16);
-                            codes_signed(c[i + 1].y, v + 20);
-                            codes_signed(c[i + 1].z, v + 24);
-                            codes_signed(c[i + 1].w, v + 28);
+                            for (int q = 0; q < CS; ++q) {
+                                dequant_word_fma(c[i + q].x, f, v + 16 * q);
+                                dequant_word_fma(c[i + q].y, f, v + 16 * q + 4);
+                                dequant_word_fma(c[i + q].z, f, v + 16 * q + 8);
+                                dequant_word_fma(c[i + q].w, f, v + 16 * q + 12);
+                            }
+                        } else {
 #pragma unroll
-                            for (int j = 0; j < 32; ++j) v[j] = bf16x2_mul(v[j], s2);
-                            if (st_ok)
-                                tmem_st_32x32b_x32(lane_base + L::A_COL + a * L::A_COLS +
-                                                       t * (L::AK / 2) + i * 16,
-                                                   v);
+                            for (int q = 0; q < CS; ++q) {
+                                dequant_word(c[i + q].x, s2, v + 16 * q);
+                                dequant_word(c[i + q].y, s2, v + 16 * q + 4);
+                                dequant_word(c[i + q].z, s2, v + 16 * q + 8);
+                                dequant_word(c[i + q].w, s2, v + 16 * q + 12);
+                            }
+                        }
+                        if (i == 0) {
+                            // the slot's previous MMAs are done
+                            if (!wait_warp(empty_at, pa, abort_flag, p.status, p.wait_ns)) {
+                                ok = false;
+                                break;
+                            }
+                            tc_fence_after();
+                        }
+                        if (st_ok) {
+                            if constexpr (CS == 1)
+                                tmem_st_32x32b_x16(a_at, v);
+                            else
+                                tmem_st_32x32b_x32(a_at + i * 16, v);
                         }
                     }
+                    if (!ok) break;
                     tmem_st_wait();
                     tc_fence_before();
                     __syncwarp();
-                    if (lane == 0) mbar_arrive(full_a(t, a));
+                    if (lane == 0) mbar_arrive(empty_at - 8u * SA);  // full_a of the slot
+                    empty_at += 8u;
+                    a_at += L::A_COLS;
+                    if (empty_at == empty_a(t, SA)) {
+                        empty_at -= 8u * SA;
+                        a_at -= L::A_COLS * SA;
+                        pa ^= 1u;
+                    }
                 }
                 if (!ok) break;
-                __syncwarp();
-                if (lane == 0) mbar_arrive(empty_smem(s));  // this warp's weight reads are done
+                w_at += L::STAGE;
+                full_at += 8u;
+                if (full_at == full_tma(S)) {
+                    full_at = full_tma(0);
+                    w_at = w_first;
+                    ph ^= 1u;
+                }
             }
             if (!ok) break;
-            // ---- epilogue: the row's NTOK accumulators, tokens 0 .. M - 1
+            // the row's NTOK accumulators
             if (!wait_warp(d_full(t), nchunk & 1u, abort_flag, p.status, p.wait_ns)) {
                 ok = false;
                 break;
             }
             tc_fence_after();
-            // the row's accumulators in slices of EC tokens (registers), then
-            // the (fused) epilogue of each slice
-            constexpr int EC = NTOK < 32 ? NTOK : 32;
-            const Epilogue& ep = p.epi;
-            // SwiGLU pairs rows (n, n ^ 1) = (gate, up): RB is even, so n has
-            // the parity of its lane and the partner is lane ^ 1
-            const float bias =
-                (FUSED && ep.bias != nullptr && valid) ? bf16_to_f32(ep.bias[n]) : 0.0f;
+            if constexpr (!SPLIT) {
+                const float bias = (FUSED && p.epi.bias != nullptr && valid)
+                                       ? bf16_to_f32(p.epi.bias[n]) : 0.0f;
+                const int mt = tt * NTOK, m_end = mt + NTOK < p.M ? mt + NTOK : p.M;
 #pragma unroll 1
-            for (int m0 = 0; m0 < NTOK; m0 += EC) {
-                float acc[EC];
+                for (int m0 = 0; mt + m0 < m_end; m0 += L::EC) {
+                    uint32_t d[32];
+                    float res[L::EC];
+                    tmem_ld_32x32b_x32(lane_base + t * NTOK + m0, d);
 #pragma unroll
-                for (int half = 0; half < EC / 16; ++half) {
-                    uint32_t d[16];
-                    tmem_ld_32x32b_x16(lane_base + t * NTOK + m0 + half * 16, d);
-                    tmem_ld_wait_x16(d);
+                    for (int j = 0; j < L::EC; ++j)
+                        res[j] = residual_at<FUSED>(p, mt + m0 + j, m_end, n, valid, lane);
+                    tmem_ld_wait(d);
 #pragma unroll
-                    for (int j = 0; j < 16; ++j) acc[half * 16 + j] = __uint_as_float(d[j]);
+                    for (int j = 0; j < L::EC; ++j)
+                        finish<FUSED>(p, __uint_as_float(d[j]), bias, res[j], mt + m0 + j, m_end, n,
+                                      valid, lane);
                 }
-                if constexpr (!FUSED) {
-#pragma unroll
-                    for (int j = 0; j < EC; ++j) {
-                        const int m = m0 + j;
-                        if (valid && m < p.M)
-                            p.out[static_cast<int64_t>(m) * p.N + n] = f32_to_bf16_rn(acc[j]);
-                    }
-                } else {
-#pragma unroll
-                    for (int j = 0; j < EC; ++j) {
-                        const int m = m0 + j;
-                        const float z = acc[j] + bias;
-                        if (ep.act == kActSwiGLU) {
-                            const float up = __shfl_xor_sync(0xffffffffu, z, 1);
-                            if ((lane & 1) == 0 && valid && m < p.M) {
-                                const int64_t o = static_cast<int64_t>(m) * ep.n_out + (n >> 1);
-                                float h = silu_f32(z) * up;
-                                if (ep.residual != nullptr) h += bf16_to_f32(ep.residual[o]);
-                                p.out[o] = f32_to_bf16_rn(h);
-                            }
-                        } else if (valid && m < p.M) {
-                            const int64_t o = static_cast<int64_t>(m) * ep.n_out + n;
-                            float h = ep.act == kActGELU ? gelu_f32(z) : z;
-                            if (ep.residual != nullptr) h += bf16_to_f32(ep.residual[o]);
-                            p.out[o] = f32_to_bf16_rn(h);
-                        }
-                    }
-                }
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(d_empty(t));  // the next chunk's MMAs may overwrite D
             }
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(d_empty(t));  // the next chunk's MMAs may overwrite D
         }
+    }
+
+    if constexpr (SPLIT) {
+        // ------------------------------------------------------------ sum over the cluster
+        // One chunk per cluster; each CTA holds its K slice's sums.  Per slice
+        // of EC tokens every CTA writes its partial sums to shared memory
+        // (over the consumed stages), and CTA `rank` adds up and finishes its
+        // EC / split tokens, always in the order of the ranks.  The stages
+        // are free once every role of the CTA is done with them.
+        tc_fence_before();
+        __syncthreads();
+        tc_fence_after();
+        const int tt = chunk0 / p.row_chunks;
+        const int n = (chunk0 - tt * p.row_chunks) * RB + r;
+        const bool valid = row_warp && r < RB && n < p.N;
+        const float bias =
+            (FUSED && p.epi.bias != nullptr && valid) ? bf16_to_f32(p.epi.bias[n]) : 0.0f;
+        const int mt = tt * NTOK, m_end = mt + NTOK < p.M ? mt + NTOK : p.M;
+        uint32_t part = sbase;
+#pragma unroll 1
+        for (int m0 = 0; mt + m0 < m_end; m0 += L::EC) {
+            // a CTA that gave up leaves the sums unwritten: its output is incomplete
+            if (row_warp && ok) {
+                uint32_t d[32];
+                tmem_ld_32x32b_x32(lane_base + row_tile * NTOK + m0, d);
+                tmem_ld_wait(d);
+#pragma unroll
+                for (int j = 0; j < L::EC; ++j)
+                    asm volatile("st.shared.u32 [%0], %1;" ::"r"(part + 4u * (j * L::ROWS_MAX + r)),
+                                 "r"(d[j]) : "memory");
+            }
+            __syncwarp();
+            cluster_sync();
+            if (row_warp && ok) {
+                if (p.split == 2)
+                    reduce_slice<2, FUSED>(p, part, L::ROWS_MAX, rank, r, bias, mt + m0, m_end, n,
+                                           valid, lane);
+                else if (p.split == 4)
+                    reduce_slice<4, FUSED>(p, part, L::ROWS_MAX, rank, r, bias, mt + m0, m_end, n,
+                                           valid, lane);
+                else
+                    reduce_slice<8, FUSED>(p, part, L::ROWS_MAX, rank, r, bias, mt + m0, m_end, n,
+                                           valid, lane);
+            }
+            __syncwarp();
+            part = part == sbase ? sbase + L::PART : sbase;
+        }
+        cluster_sync();  // no CTA leaves while another reads its sums
     }
 
     __syncwarp();
@@ -474,39 +594,144 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (warp == 1) tmem_dealloc(tmem, L::TMEM_COLS);
 }
 
-template <int NTOK>
+template <int NTOK, int TILES, bool SPLIT>
 cudaError_t launch_tc_variant(const CUtensorMap* tx, const CUtensorMap* tw, const GemvParams& p,
                               int grid, cudaStream_t stream) {
-    using L = TLayout<NTOK>;
+    using L = TLayout<NTOK, TILES>;
     const bool fused =
         p.epi.bias != nullptr || p.epi.residual != nullptr || p.epi.act != kActNone;
-    auto kern = fused ? w4a16_gemv_tc_kernel<NTOK, true> : w4a16_gemv_tc_kernel<NTOK, false>;
+    auto kern = fused ? w4a16_gemv_tc_kernel<NTOK, TILES, true, SPLIT>
+                      : w4a16_gemv_tc_kernel<NTOK, TILES, false, SPLIT>;
     cudaError_t e =
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, L::SMEM_BYTES);
     if (e != cudaSuccess) return e;
-    kern<<<grid, kThreads, L::SMEM_BYTES, stream>>>(*tx, *tw, p);
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1];
+    cfg.gridDim = dim3(static_cast<unsigned>(grid));
+    cfg.blockDim = dim3(L::THREADS);
+    cfg.dynamicSmemBytes = L::SMEM_BYTES;
+    cfg.stream = stream;
+    if constexpr (SPLIT) {
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = static_cast<unsigned>(p.split);
+        attr[0].val.clusterDim.y = 1;
+        attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+    }
+    e = cudaLaunchKernelEx(&cfg, kern, *tx, *tw, p);
+    if (e != cudaSuccess) return e;
     return cudaGetLastError();
+}
+
+template <int NTOK, int TILES>
+cudaError_t launch_tc_split(const CUtensorMap* tx, const CUtensorMap* tw, const GemvParams& p,
+                            int sm_count, cudaStream_t stream) {
+    if (p.split > 1)
+        return launch_tc_variant<NTOK, TILES, true>(tx, tw, p, p.num_chunks * p.split, stream);
+    const int grid = p.num_chunks < sm_count ? p.num_chunks : sm_count;
+    return launch_tc_variant<NTOK, TILES, false>(tx, tw, p, grid, stream);
+}
+
+// Clusters of `split` CTAs that can be resident at once; cached per device.
+int cluster_slots(int split, int sm_count) {
+    if (split == 1) return sm_count;
+    constexpr int kMaxDev = 64;
+    static std::atomic<int> cache[kMaxDev][4] = {};
+    const int slot = split == 2 ? 0 : split == 4 ? 1 : 2;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDev) return 0;
+    int n = cache[dev][slot].load(std::memory_order_relaxed);
+    if (n != 0) return n;
+    using L = TLayout<128, 3>;
+    auto kern = w4a16_gemv_tc_kernel<128, 3, false, true>;
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, L::SMEM_BYTES) ==
+        cudaSuccess) {
+        cudaLaunchConfig_t cfg = {};
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = static_cast<unsigned>(split);
+        attr[0].val.clusterDim.y = 1;
+        attr[0].val.clusterDim.z = 1;
+        cfg.gridDim = dim3(static_cast<unsigned>(sm_count / split * split));
+        cfg.blockDim = dim3(L::THREADS);
+        cfg.dynamicSmemBytes = L::SMEM_BYTES;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess) n = 0;
+    }
+    cudaGetLastError();  // a failed query leaves no sticky error for the next launch
+    if (n <= 0) n = -1;  // none: no split
+    cache[dev][slot].store(n, std::memory_order_relaxed);
+    return n;
 }
 
 }  // namespace
 
-int gemv_tc_rows_per_cta(int64_t N, int sm_count) {
-    int64_t per = (N + sm_count - 1) / sm_count;
-    per = (per + 1) / 2 * 2;
-    if (per > 128 * kTilesMax) per = 128 * kTilesMax;
-    if (per < 2) per = 2;
-    return static_cast<int>(per);
+GemvTcPlan gemv_tc_plan(int64_t M, int64_t N, int64_t K, int sm_count) {
+    // us per 128-k stage of a CTA that holds 1, 2 or 3 tiles of 128 rows, by token
+    // columns 32, 64, 96, 112, 128 (K = 12288, N = 36864 and 49152, less 4 us: 60.6 / 62.2
+    // / 66.5 / 69.9 / 74.6 and 74.4 / 80.6 / 88.1 / 106.4 / 111.8 us in all)
+    static constexpr double kStageUs[3][5] = {{0.45, 0.45, 0.46, 0.47, 0.48},
+                                              {0.60, 0.61, 0.65, 0.69, 0.73},
+                                              {0.73, 0.80, 0.88, 1.07, 1.13}};
+    GemvTcPlan best{};
+    // equal tiles of at most 128 tokens
+    const int64_t tok_tiles = (M + 127) / 128;
+    const int64_t per = (M + tok_tiles - 1) / tok_tiles;
+    best.tokens = per <= 32 ? 32 : per <= 64 ? 64 : per <= 96 ? 96 : per <= 112 ? 112 : 128;
+    const int tok = best.tokens == 32 ? 0 : best.tokens == 64 ? 1 : (best.tokens - 64) / 16;
+    const int64_t KS = (K + kGroupK - 1) / kGroupK;
+    for (int split = 1; split <= 8; split *= 2) {
+        const int64_t slots = cluster_slots(split, sm_count);
+        if (split > 1 && (slots < tok_tiles || split > KS)) continue;
+        // rows: spread evenly over as few waves of the slots as hold them (a
+        // cluster takes one chunk); even, SwiGLU pairs rows 2j, 2j + 1
+        int64_t waves = (N * tok_tiles + slots * 128 * kTilesMax - 1) / (slots * 128 * kTilesMax);
+        if (split > 1 && waves > 1) continue;
+        int64_t rb = 0;
+        for (;; ++waves) {
+            const int64_t chunks = slots * waves / tok_tiles;
+            if (chunks < 1) continue;
+            rb = ((N + chunks - 1) / chunks + 1) / 2 * 2;
+            if (rb <= 128 * kTilesMax || split > 1) break;
+        }
+        if (rb > 128 * kTilesMax) continue;
+        const int nt = static_cast<int>((rb + 127) / 128);
+        const double stages = static_cast<double>(waves) * static_cast<double>((KS + split - 1) / split);
+        const double cost = 4.0 + stages * kStageUs[nt - 1][tok] +
+                            (split > 1 ? 1.5 + 0.04 * best.tokens : 0.0);
+        if (best.cost_us == 0.0 || cost < best.cost_us) {
+            best.cost_us = cost;
+            best.split = split;
+            best.rows_per_cta = static_cast<int>(rb);
+            best.row_chunks = static_cast<int>((N + rb - 1) / rb);
+            best.num_chunks = static_cast<int>(best.row_chunks * tok_tiles);
+        }
+    }
+    return best;
 }
 
-int gemv_tc_tokens(int64_t M) { return M <= 16 ? 16 : M <= 32 ? 32 : M <= 64 ? 64 : 128; }
-
 cudaError_t gemv_tc_launch(const CUtensorMap* tx, const CUtensorMap* tw, const GemvParams& p,
-                           int sm_count, cudaStream_t stream) {
-    const int grid = p.num_chunks < sm_count ? p.num_chunks : sm_count;
-    if (p.M <= 16) return launch_tc_variant<16>(tx, tw, p, grid, stream);
-    if (p.M <= 32) return launch_tc_variant<32>(tx, tw, p, grid, stream);
-    if (p.M <= 64) return launch_tc_variant<64>(tx, tw, p, grid, stream);
-    return launch_tc_variant<128>(tx, tw, p, grid, stream);
+                           int tokens, int sm_count, cudaStream_t stream) {
+    const bool two = p.nt <= 2;
+    switch (tokens) {
+        case 32:
+            return two ? launch_tc_split<32, 2>(tx, tw, p, sm_count, stream)
+                       : launch_tc_split<32, 3>(tx, tw, p, sm_count, stream);
+        case 64:
+            return two ? launch_tc_split<64, 2>(tx, tw, p, sm_count, stream)
+                       : launch_tc_split<64, 3>(tx, tw, p, sm_count, stream);
+        case 96:
+            return two ? launch_tc_split<96, 2>(tx, tw, p, sm_count, stream)
+                       : launch_tc_split<96, 3>(tx, tw, p, sm_count, stream);
+        case 112:
+            return two ? launch_tc_split<112, 2>(tx, tw, p, sm_count, stream)
+                       : launch_tc_split<112, 3>(tx, tw, p, sm_count, stream);
+        default:
+            return two ? launch_tc_split<128, 2>(tx, tw, p, sm_count, stream)
+                       : launch_tc_split<128, 3>(tx, tw, p, sm_count, stream);
+    }
 }
 
 }  // namespace w4a16

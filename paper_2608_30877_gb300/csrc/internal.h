@@ -33,13 +33,12 @@ struct TsParams {
     uint64_t wait_ns;        // limit of every barrier wait (kWaitLimitNs unless a test lowers it)
 };
 
-// Kernel variants of the fused kernel.  Both take 128 weight rows per tile
-// (the MMA's M) and 64 k per pipeline stage.
+// Kernel variants of the fused kernel.  All take 128 weight rows per tile
+// (the MMA's M) and 64 k per pipeline stage, and run on a persistent grid.
 enum class TsVariant : int {
-    kGemm256 = 0,   // 256 tokens per tile, persistent grid (large M)
-    kGemv32 = 1,    // 32 tokens per tile, one tile per CTA (M <= 32)
-    kGemmPair = 2,  // 256 tokens x 256 weight rows per CTA pair (cta_group::2), persistent
-    kGemmPairWide = 3,  // 384 tokens (two 192-column accumulators) x 256 rows per CTA pair
+    kGemm256 = 0,   // 256 tokens per tile
+    kGemmPair = 1,  // 256 tokens x 256 weight rows per CTA pair (cta_group::2)
+    kGemmPairWide = 2,  // 384 tokens (two 192-column accumulators) x 256 rows per CTA pair
 };
 
 int ts_tokens_per_tile(TsVariant v);
@@ -50,35 +49,48 @@ int ts_grid(TsVariant v, const TsParams& p, int sm_count);
 // Whether the 384-token CTA-pair tiles take fewer unit-costs per pair than the
 // 256-token ones for an M x N product (tile padding and the last wave).
 bool ts_prefer_wide(int64_t M, int64_t N, int sm_count);
+// Modelled time of the better of the two, in us.
+double ts_cost_us(int64_t M, int64_t N, int64_t K, int sm_count);
 cudaError_t ts_launch(TsVariant v, const CUtensorMap* tmap_x, const CUtensorMap* tmap_w,
                       const TsParams& p, int grid, cudaStream_t stream);
 
-// Parameters of the small-M streaming kernels (gemv_rows.cu, gemv_tc.cu).
+// Parameters of the streaming kernels (gemv_rows.cu, gemv_tc.cu).
 struct GemvParams {
     const uint16_t* scales;  // bf16 bits [N, K/g]
     uint16_t* out;           // bf16 bits [M, N]
     int* status;
     int M, N, K, g;
     int rows_per_cta;        // RB: weight rows per CTA chunk, even, <= 352 (<= 384 tcgen05)
-    int num_chunks;          // ceil(N / RB)
+    int num_chunks;          // ceil(N / RB), times the token tiles in the tcgen05 kernel
     int nt;                  // tcgen05 kernel: 128-row MMA tiles per chunk, ceil(RB / 128)
+    int row_chunks;          // tcgen05 kernel: ceil(N / RB)
+    int split;               // tcgen05 kernel: CTAs of a cluster that split K
     Epilogue epi;
     uint64_t wait_ns;
 };
 
-// RB for N rows spread over the SMs; tokens per tile for M.
+// The warp-level kernel, M <= 16 and g = 128 (gemv_rows.cu): RB for N rows spread over
+// the SMs, tokens per x box for M, modelled time.
 int gemv_rows_per_cta(int64_t N, int sm_count);
 int gemv_tokens_per_tile(int64_t M);
+double gemv_cost_us(int64_t M, int64_t N, int64_t K, int sm_count);
 cudaError_t gemv_launch(const CUtensorMap* tmap_x, const CUtensorMap* tmap_w,
                         const GemvParams& p, int sm_count, cudaStream_t stream);
 
-// The tensor-core streaming kernel for the same regime (gemv_tc.cu): RB even,
-// at most 384; x boxes of gemv_tc_tokens(M) rows x 64 k (128-byte swizzle),
-// weight boxes of RB/2 rows x 64 bytes (64-byte swizzle).
-int gemv_tc_rows_per_cta(int64_t N, int sm_count);
-int gemv_tc_tokens(int64_t M);
+// The tensor-core streaming kernel (gemv_tc.cu): RB even, at most 384; x boxes
+// of `tokens` rows x 64 k (128-byte swizzle), weight boxes of RB/2 rows x 64
+// bytes (64-byte swizzle).
+struct GemvTcPlan {
+    int tokens;        // token columns per tile: 32, 64 or 128
+    int split;         // CTAs (one cluster) sharing a chunk, each a slice of K
+    int rows_per_cta;  // RB
+    int row_chunks;    // ceil(N / RB)
+    int num_chunks;    // row_chunks x token tiles
+    double cost_us;    // modelled time (the dispatch compares it with ts_cost_us)
+};
+GemvTcPlan gemv_tc_plan(int64_t M, int64_t N, int64_t K, int sm_count);
 cudaError_t gemv_tc_launch(const CUtensorMap* tmap_x, const CUtensorMap* tmap_w,
-                           const GemvParams& p, int sm_count, cudaStream_t stream);
+                           const GemvParams& p, int tokens, int sm_count, cudaStream_t stream);
 
 // Attention prefill over packed sequences (attention.cu).
 struct AttnParams {

@@ -713,10 +713,6 @@ constexpr int kPairSS = W4A16_PAIR_STAGES, kPairST = W4A16_PAIR_STAGES;
 #define W4A16_WIDE_SS 4
 #endif
 constexpr int kWideT = 384, kWideSS = W4A16_WIDE_SS, kWideST = 4;
-// Small M: 32 tokens per tile, 8 shared-memory stages of 8 KB, 3 A stages;
-// 128 tensor-memory columns so that three CTAs share an SM.
-constexpr int kGemvT = 32, kGemvSS = 8, kGemvST = 3, kGemvDQ = 1, kGemvEP = 1;
-
 // CTA pairs that can be resident at once (SMs left over in a GPC cannot
 // take one); cached per device.
 int pair_slots(int sm_count) {
@@ -752,7 +748,7 @@ int pair_slots(int sm_count) {
 }  // namespace
 
 int ts_tokens_per_tile(TsVariant v) {
-    return v == TsVariant::kGemv32 ? kGemvT : v == TsVariant::kGemmPairWide ? kWideT : kGemmT;
+    return v == TsVariant::kGemmPairWide ? kWideT : kGemmT;
 }
 
 int ts_x_box_tokens(TsVariant v) {
@@ -761,26 +757,35 @@ int ts_x_box_tokens(TsVariant v) {
     return ts_tokens_per_tile(v);
 }
 
-bool ts_prefer_wide(int64_t M, int64_t N, int sm_count) {
-    // Each CTA pair walks ceil(units / pairs) units of (token tile, 256 weight
-    // rows); a unit of the 384-token tiles costs ~1.37 of a 256-token one
-    // (measured: 1.35-1.37 on the 4096- and 8192-token projections, 1.39 for
-    // one tile of each).  The tiles that give the fewer unit-costs per pair win.
+namespace {
+// Units of (token tile, 256 weight rows) that each CTA pair walks.
+int64_t units_per_pair(int64_t M, int64_t N, int tokens, int sm_count) {
     const int64_t pairs = pair_slots(sm_count);
-    const int64_t per_tile = (N + 255) / 256;
-    const int64_t w256 = ((M + kGemmT - 1) / kGemmT * per_tile + pairs - 1) / pairs;
-    const int64_t w384 = ((M + kWideT - 1) / kWideT * per_tile + pairs - 1) / pairs;
-    return w384 * 137 < w256 * 100;
+    return ((M + tokens - 1) / tokens * ((N + 255) / 256) + pairs - 1) / pairs;
+}
+}  // namespace
+
+bool ts_prefer_wide(int64_t M, int64_t N, int sm_count) {
+    // A unit of the 384-token tiles costs ~1.37 of a 256-token one (measured:
+    // 1.35-1.37 on the 4096- and 8192-token projections, 1.39 for one tile of
+    // each).  The tiles that give the fewer unit-costs per pair win.
+    return units_per_pair(M, N, kWideT, sm_count) * 137 <
+           units_per_pair(M, N, kGemmT, sm_count) * 100;
+}
+
+double ts_cost_us(int64_t M, int64_t N, int64_t K, int sm_count) {
+    // a 256-token unit takes 0.344 us per 64-k stage (12288 x 12288 at 256
+    // tokens: 70 us for one unit per pair, 146 us for two at N = 36864)
+    const double narrow = static_cast<double>(units_per_pair(M, N, kGemmT, sm_count));
+    const double wide = 1.37 * static_cast<double>(units_per_pair(M, N, kWideT, sm_count));
+    return 4.0 + 0.344 * static_cast<double>(K / kBK) * (wide < narrow ? wide : narrow);
 }
 
 int ts_grid(TsVariant v, const TsParams& p, int sm_count) {
     if (v == TsVariant::kGemm256) return p.num_tiles < sm_count ? p.num_tiles : sm_count;
-    if (v == TsVariant::kGemmPair || v == TsVariant::kGemmPairWide) {
-        const int units = p.num_t_tiles * ((p.num_w_tiles + 1) / 2);
-        const int slots = pair_slots(sm_count);
-        return 2 * (units < slots ? units : slots);
-    }
-    return p.num_tiles;
+    const int units = p.num_t_tiles * ((p.num_w_tiles + 1) / 2);
+    const int slots = pair_slots(sm_count);
+    return 2 * (units < slots ? units : slots);
 }
 
 cudaError_t ts_launch(TsVariant v, const CUtensorMap* tx, const CUtensorMap* tw,
@@ -791,11 +796,8 @@ cudaError_t ts_launch(TsVariant v, const CUtensorMap* tx, const CUtensorMap* tw,
     if (v == TsVariant::kGemmPair)
         return launch_variant<kGemmT, kPairSS, kPairST, kGemmDQ, kGemmEP, 1, true>(tx, tw, p,
                                                                                   grid, stream);
-    if (v == TsVariant::kGemmPairWide)
-        return launch_variant<kWideT, kWideSS, kWideST, kGemmDQ, kGemmEP, 1, true, 2>(
-            tx, tw, p, grid, stream);
-    return launch_variant<kGemvT, kGemvSS, kGemvST, kGemvDQ, kGemvEP, 3, false>(tx, tw, p, grid,
-                                                                               stream);
+    return launch_variant<kWideT, kWideSS, kWideST, kGemmDQ, kGemmEP, 1, true, 2>(tx, tw, p, grid,
+                                                                                 stream);
 }
 
 }  // namespace w4a16
