@@ -281,6 +281,16 @@ int launch_gemv_tc(const DeviceState& st, const GemvTcPlan& plan, const void* x,
 int launch_linear(const DeviceState& st, const void* x, const void* w, const void* s, void* out,
                   int64_t M, int64_t N, int64_t K, int64_t g, const Epilogue& epi,
                   cudaStream_t stream) {
+    // a few rows: tokens over CTAs, unless so many tokens that the GEMM's one wave of
+    // tiles is cheaper (12288 x 2: M = 64 4.9 us against 68, 65536 242 against 316;
+    // 12288 x 8: M = 1000 17 against 74, 65536 824 against 318)
+    if (N <= kHeadRows &&
+        (M <= 128 || head_cost_us(M, N, K) < ts_cost_us(M, N, K, st.sm_count))) {
+        const HeadParams p{static_cast<const uint16_t*>(s), static_cast<uint16_t*>(out),
+                           static_cast<int>(M), static_cast<int>(N), static_cast<int>(K),
+                           static_cast<int>(g), epi};
+        return launch_head(x, w, p, st.sm_count, stream) == cudaSuccess ? W4A16_OK : W4A16_ERR_CUDA;
+    }
     // Up to 128 tokens the weights stream once per call on the streaming kernels
     // (12288 x 49152: M = 64 81 us there against 212 on the 256-token GEMM tiles,
     // M = 128 112 against 214).  M <= 16: the warp-level kernel has the higher rate

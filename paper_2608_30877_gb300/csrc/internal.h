@@ -92,6 +92,18 @@ GemvTcPlan gemv_tc_plan(int64_t M, int64_t N, int64_t K, int sm_count);
 cudaError_t gemv_tc_launch(const CUtensorMap* tmap_x, const CUtensorMap* tmap_w,
                            const GemvParams& p, int tokens, int sm_count, cudaStream_t stream);
 
+// Linear layers of at most kHeadRows weight rows (head.cu).
+constexpr int kHeadRows = 8;
+struct HeadParams {
+    const uint16_t* scales;
+    uint16_t* out;
+    int M, N, K, g;
+    Epilogue epi;
+};
+double head_cost_us(int64_t M, int64_t N, int64_t K);  // modelled time
+cudaError_t launch_head(const void* x, const void* w, const HeadParams& p, int sm_count,
+                        cudaStream_t stream);
+
 // Attention prefill over packed sequences (attention.cu).
 struct AttnParams {
     const int32_t* seq_start;  // device [nseq + 1]

@@ -236,24 +236,35 @@ __global__ void __cluster_dims__(kTopkCtas, 1, 1) __launch_bounds__(kTopkThreads
     }
 }
 
-__global__ void gather_rows_kernel(const uint16_t* __restrict__ src, int64_t src_rows,
-                                   int64_t D, const int32_t* __restrict__ idx, int64_t P,
-                                   uint16_t* __restrict__ dst, int* status) {
+// A CTA copies one kGatherChunk-element piece of a row at a time (blockIdx.y
+// and on): 64 rows of 24 KB on one CTA each were a serial chain of six loads
+// and stores per thread.
+constexpr int kGatherThreads = 256;
+constexpr int kGatherChunk = 8 * kGatherThreads;
+
+__global__ void __launch_bounds__(kGatherThreads)
+    gather_rows_kernel(const uint16_t* __restrict__ src, int64_t src_rows, int64_t D,
+                       const int32_t* __restrict__ idx, int64_t P, uint16_t* __restrict__ dst,
+                       int* status) {
+    const int64_t j_step = static_cast<int64_t>(gridDim.y) * kGatherChunk;
     for (int64_t p = blockIdx.x; p < P; p += gridDim.x) {
         const int32_t r = idx[p];
+        const bool ok = r >= 0 && r < src_rows;
+        if (!ok && threadIdx.x == 0 && blockIdx.y == 0)
+            atomicCAS(status, 0, 1 /* W4A16_ERR_INVALID_ARG; the first error is kept */);
+        const uint16_t* s = src + (ok ? static_cast<int64_t>(r) : 0) * D;
         uint16_t* d = dst + p * D;
-        if (r < 0 || r >= src_rows) {
-            for (int64_t j = threadIdx.x; j < D; j += blockDim.x) d[j] = 0;
-            if (threadIdx.x == 0) atomicCAS(status, 0, 1 /* W4A16_ERR_INVALID_ARG; the first error is kept */);
-            continue;
-        }
-        const uint16_t* s = src + static_cast<int64_t>(r) * D;
-        if ((D & 7) == 0) {  // rows of whole 16-byte chunks (bases are 16-byte aligned)
-            const uint4* s4 = reinterpret_cast<const uint4*>(s);
-            uint4* d4 = reinterpret_cast<uint4*>(d);
-            for (int64_t j = threadIdx.x; j < D / 8; j += blockDim.x) d4[j] = s4[j];
-        } else {
-            for (int64_t j = threadIdx.x; j < D; j += blockDim.x) d[j] = s[j];
+        for (int64_t j0 = static_cast<int64_t>(blockIdx.y) * kGatherChunk; j0 < D; j0 += j_step) {
+            if ((D & 7) == 0) {  // rows of whole 16-byte chunks (bases are 16-byte aligned)
+                const int64_t j = j0 + 8 * threadIdx.x;
+                if (j < D)
+                    *reinterpret_cast<uint4*>(d + j) =
+                        ok ? __ldg(reinterpret_cast<const uint4*>(s + j)) : make_uint4(0, 0, 0, 0);
+            } else {
+                const int64_t end = j0 + kGatherChunk < D ? j0 + kGatherChunk : D;
+                for (int64_t j = j0 + threadIdx.x; j < end; j += kGatherThreads)
+                    d[j] = ok ? s[j] : static_cast<uint16_t>(0);
+            }
         }
     }
 }
@@ -274,9 +285,13 @@ cudaError_t launch_topk_smallest(const void* scores, bool bf16, int64_t n, int k
 cudaError_t launch_gather_rows(const uint16_t* src, int64_t src_rows, int64_t D,
                                const int32_t* idx, int64_t P, uint16_t* dst, int* status,
                                int sm_count, cudaStream_t stream) {
-    const int64_t blocks = P < 4 * sm_count ? P : 4 * sm_count;
-    gather_rows_kernel<<<static_cast<int>(blocks), 256, 0, stream>>>(src, src_rows, D, idx, P,
-                                                                     dst, status);
+    // pieces of rows until the CTAs fill the SMs eight times over
+    const int64_t pieces = (D + kGatherChunk - 1) / kGatherChunk;
+    const int64_t want = 8 * static_cast<int64_t>(sm_count);
+    const int64_t bx = P < want ? P : want;
+    const int64_t by = pieces < (want + bx - 1) / bx ? pieces : (want + bx - 1) / bx;
+    gather_rows_kernel<<<dim3(static_cast<unsigned>(bx), static_cast<unsigned>(by)), kGatherThreads,
+                         0, stream>>>(src, src_rows, D, idx, P, dst, status);
     return cudaGetLastError();
 }
 
