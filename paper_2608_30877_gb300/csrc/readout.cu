@@ -6,20 +6,28 @@
 //   topk_smallest the k smallest scores (best binders: lowest free energy),
 //                 ascending by IEEE totalOrder with NaN last, ties by index.
 //
-// Top-k, GB300-first: one thread-block cluster of 8 CTAs (1024 threads each)
-// does a most-significant-digit-first radix select over order-preserving
-// 32-bit keys.  Each CTA histograms one contiguous eighth of the scores; CTA 0
-// sums the eight histograms through distributed shared memory and picks the
-// digit, four passes of 8 bits.  The selected (key, index) pairs are then
-// written straight into CTA 0's shared memory -- equal keys taken in index
-// order by an ordered block scan -- and CTA 0 sorts them (bitonic) and stores
-// the result.  Nothing goes through global scratch memory, and the cluster
-// barriers are hardware barriers among co-scheduled CTAs.
+// Top-k, GB300-first: one thread-block cluster of 8 CTAs (1024 threads each; 16 CTAs
+// beyond 320000 scores) reads the scores once and does a radix select, most
+// significant digit first, over (order-preserving 32-bit key, index) pairs.  Each CTA
+// keeps the keys of its contiguous slice in shared memory (up to 40000; longer slices
+// are read again) and histograms them, the first digit into four copies by
+// lane, as most scores share a few exponents.  Every CTA adds up all histograms
+// through distributed shared memory and finds the digit itself: one cluster
+// barrier a digit of 11 bits.  The search ends with the first bin that is wanted
+// whole; the digits of the index only matter where equal keys straddle the k-th.
+// The selected pairs are gathered by every CTA, which ranks its share of them by
+// counting smaller pairs, and stores them.  Nothing goes through global memory.
+// Bound by latency (about five cluster barriers) and the first digit's atomics:
+// 200000 scores, k = 1000 62 -> 20 us; 10000, k = 100 28.8 -> 10.8; 2000000, k = 1024
+// 295 -> 67 (before: seven passes over the scores by scalar loads, a digit search by one
+// thread and 55 sorting steps on one CTA).
 #include "internal.h"
 
+#include <atomic>
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
 #include <cstdint>
+#include <utility>
 
 namespace cg = cooperative_groups;
 
@@ -27,9 +35,11 @@ namespace w4a16 {
 
 namespace {
 
-constexpr int kTopkCtas = 8;
 constexpr int kTopkThreads = 1024;
 constexpr int kTopkWarps = kTopkThreads / 32;
+constexpr int kTopkBins = 2048;         // 11-bit digits
+constexpr int kTopkCopies = 4;          // histograms of the first digit, by lane
+constexpr int kTopkCache = 40 * 1000;   // keys a CTA keeps in shared memory
 
 // Keys whose unsigned order is totalOrder on the scores; every NaN maps to
 // the largest key.
@@ -40,42 +50,18 @@ __device__ __forceinline__ uint32_t order_key_f32(float f) {
 }
 
 struct TopkShared {
-    uint32_t hist[256];
-    uint32_t total[256];
+    uint32_t keys[kTopkCache];
+    // (the copies of one bin lie on different banks)
+    uint32_t priv[kTopkCopies][kTopkBins + 32 / kTopkCopies];
+    // this CTA's histogram of a pass, read by the other CTAs; a pass's buffer
+    // is written again two passes on, two cluster barriers after the last read
+    uint32_t hist[2][kTopkBins];
+    unsigned long long list[kTopkMaxK];   // this CTA's selected (key << 32 | index)
+    unsigned long long all[kTopkMaxK];    // every CTA's
     uint32_t warp_sum[kTopkWarps];
-    uint32_t round_total;                 // block total of the last block_rank
-    uint32_t digit, need;                 // written by CTA 0 each pass
-    uint32_t count_lt, count_eq;          // this CTA's
-    uint32_t lt_off, eq_off, eq_take;     // written by CTA 0 for this CTA
-    uint32_t lt_cursor;
-    unsigned long long sel[kTopkMaxK];    // CTA 0: selected (key << 32 | index)
+    uint32_t digit, before, bin;          // of the current pass
+    uint32_t count;
 };
-
-// Block-wide exclusive scan of one flag per thread, in thread order;
-// returns this thread's position; the block total is left in *total (shared
-// memory), valid for every thread on return.
-__device__ __forceinline__ uint32_t block_rank(bool flag, uint32_t* warp_sum, uint32_t* total) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const uint32_t ballot = __ballot_sync(0xffffffffu, flag);
-    const uint32_t in_warp = __popc(ballot & ((1u << lane) - 1u));
-    if (lane == 0) warp_sum[warp] = __popc(ballot);
-    __syncthreads();
-    if (warp == 0) {
-        const uint32_t v = lane < kTopkWarps ? warp_sum[lane] : 0u;
-        uint32_t incl = v;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl += t;
-        }
-        if (lane < kTopkWarps) warp_sum[lane] = incl - v;  // exclusive
-        if (lane == 31) *total = incl;
-    }
-    __syncthreads();
-    const uint32_t r = warp_sum[warp] + in_warp;
-    __syncthreads();
-    return r;
-}
 
 // Scores are fp32, or bf16 (widened exactly: its bits are the top half of
 // the fp32's).
@@ -92,148 +78,171 @@ __device__ __forceinline__ uint32_t order_key(const void* scores, int64_t i) {
     return order_key_f32(score_at<BF16>(scores, i));
 }
 
-template <bool BF16>
-__global__ void __cluster_dims__(kTopkCtas, 1, 1) __launch_bounds__(kTopkThreads, 1)
+template <bool BF16, int kTopkCtas>
+__global__ void __launch_bounds__(kTopkThreads, 1)
     topk_smallest_kernel(const void* __restrict__ scores, int64_t n, int k,
                          int32_t* __restrict__ out_idx, float* __restrict__ out_val) {
-    __shared__ TopkShared sh;
+    extern __shared__ __align__(16) uint8_t topk_smem[];
+    TopkShared& sh = *reinterpret_cast<TopkShared*>(topk_smem);
     cg::cluster_group cluster = cg::this_cluster();
     const int rank = static_cast<int>(cluster.block_rank());
-    const int tid = threadIdx.x;
-    TopkShared* root = cluster.map_shared_rank(&sh, 0);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
 
-    const int64_t lo = n * rank / kTopkCtas, hi = n * (rank + 1) / kTopkCtas;
-    uint32_t prefix = 0, mask = 0, need = static_cast<uint32_t>(k);
+    // the CTA's slice, starting on a 16-byte boundary of the scores
+    constexpr int V = BF16 ? 8 : 4;
+    const int64_t per = (n + kTopkCtas * V - 1) / (kTopkCtas * V) * V;
+    const int64_t lo = per * rank < n ? per * rank : n;
+    const int count = static_cast<int>((lo + per < n ? lo + per : n) - lo);
+    const bool cached = per <= kTopkCache;
 
-    // ---- radix select: the k-th smallest key, four digits of 8 bits
-    for (int pass = 0; pass < 4; ++pass) {
-        const int shift = 24 - 8 * pass;
-        if (tid < 256) sh.hist[tid] = 0;
-        __syncthreads();
-        for (int64_t i = lo + tid; i < hi; i += kTopkThreads) {
-            const uint32_t key = order_key<BF16>(scores, i);
-            if ((key & mask) == prefix) atomicAdd(&sh.hist[(key >> shift) & 255u], 1u);
+    for (int i = tid; i < static_cast<int>(sizeof(sh.priv) / 4); i += kTopkThreads)
+        (&sh.priv[0][0])[i] = 0;
+    if (tid == 0) sh.count = 0;
+    __syncthreads();
+    // ---- one read of the scores: keys, and the histogram of their first digit
+    uint32_t* mine = sh.priv[lane % kTopkCopies];
+    auto first = [&](int i, uint32_t key) {
+        if (cached) sh.keys[i] = key;
+        atomicAdd(&mine[key >> 21], 1u);
+    };
+    const int whole = count / V * V;
+    constexpr int kLoads = 4;  // 16-byte loads in flight per thread
+    for (int i0 = tid * V; i0 < whole; i0 += kLoads * kTopkThreads * V) {
+        uint4 c[kLoads];
+#pragma unroll
+        for (int u = 0; u < kLoads; ++u) {
+            const int i = i0 + u * kTopkThreads * V;
+            if (i < whole)
+                c[u] = __ldg(reinterpret_cast<const uint4*>(static_cast<const uint8_t*>(scores) +
+                                                            (lo + i) * (BF16 ? 2 : 4)));
         }
-        cluster.sync();
-        if (rank == 0) {
-            if (tid < 256) {
-                uint32_t s = 0;
-                for (int r = 0; r < kTopkCtas; ++r) s += cluster.map_shared_rank(&sh, r)->hist[tid];
-                sh.total[tid] = s;
+#pragma unroll
+        for (int u = 0; u < kLoads; ++u) {
+            const int i = i0 + u * kTopkThreads * V;
+            if (i >= whole) break;
+            const uint32_t h[4] = {c[u].x, c[u].y, c[u].z, c[u].w};
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                if constexpr (BF16) {
+                    first(i + 2 * e, order_key_f32(__uint_as_float(h[e] << 16)));
+                    first(i + 2 * e + 1, order_key_f32(__uint_as_float(h[e] & 0xFFFF0000u)));
+                } else {
+                    first(i + e, order_key_f32(__uint_as_float(h[e])));
+                }
             }
+        }
+    }
+    for (int i = whole + tid; i < count; i += kTopkThreads) first(i, order_key<BF16>(scores, lo + i));
+    __syncthreads();
+    auto key_at = [&](int i) { return cached ? sh.keys[i] : order_key<BF16>(scores, lo + i); };
+
+    // ---- radix select over (key, index): the k-th smallest pair, 11 bits at a
+    // time, the digits of the index only where equal keys straddle the k-th.  A
+    // pass ends the search as soon as a whole bin is wanted.  `top` holds the
+    // digits found, `low` the bits below them.
+    unsigned long long top = 0;
+    int low = 64;
+    uint32_t need = static_cast<uint32_t>(k);
+    for (int pass = 0;; ++pass) {
+        const int bits = pass % 3 == 2 ? 10 : 11;
+        uint32_t* hist = sh.hist[pass & 1];
+        const int b0 = 2 * tid;  // this thread's bins
+        if (pass == 0) {
+            uint32_t s0 = 0, s1 = 0;
+#pragma unroll
+            for (int c = 0; c < kTopkCopies; ++c) {
+                s0 += sh.priv[c][b0];
+                s1 += sh.priv[c][b0 + 1];
+            }
+            hist[b0] = s0;
+            hist[b0 + 1] = s1;
+        } else {
+            hist[b0] = hist[b0 + 1] = 0;
             __syncthreads();
-            if (tid == 0) {
-                uint32_t before = 0, d = 0;
-                for (; d < 255; ++d) {
-                    if (before + sh.total[d] >= need) break;
-                    before += sh.total[d];
-                }
-                sh.digit = d;
-                sh.need = need - before;
+            for (int i = tid; i < count; i += kTopkThreads) {
+                const unsigned long long pair =
+                    (static_cast<unsigned long long>(key_at(i)) << 32) | static_cast<uint32_t>(lo + i);
+                if (pair >> low == top)
+                    atomicAdd(&hist[static_cast<uint32_t>(pair >> (low - bits)) & ((1u << bits) - 1u)], 1u);
             }
         }
         cluster.sync();
-        const uint32_t d = root->digit;
-        need = root->need;
-        prefix |= d << shift;
-        mask |= 255u << shift;
-    }
-    const uint32_t thr = prefix;        // the k-th smallest key
-    const uint32_t need_eq = need;      // how many keys equal to it are taken
-
-    // ---- per-CTA counts of keys below and equal to the threshold
-    uint32_t lt = 0, eq = 0;
-    for (int64_t i = lo + tid; i < hi; i += kTopkThreads) {
-        const uint32_t key = order_key<BF16>(scores, i);
-        lt += key < thr;
-        eq += key == thr;
-    }
-    lt = __reduce_add_sync(0xffffffffu, lt);
-    eq = __reduce_add_sync(0xffffffffu, eq);
-    if ((tid & 31) == 0) sh.warp_sum[tid >> 5] = lt;
-    __syncthreads();
-    if (tid == 0) {
-        uint32_t s = 0;
-        for (int w = 0; w < kTopkWarps; ++w) s += sh.warp_sum[w];
-        sh.count_lt = s;
-    }
-    __syncthreads();
-    if ((tid & 31) == 0) sh.warp_sum[tid >> 5] = eq;
-    __syncthreads();
-    if (tid == 0) {
-        uint32_t s = 0;
-        for (int w = 0; w < kTopkWarps; ++w) s += sh.warp_sum[w];
-        sh.count_eq = s;
-        sh.lt_cursor = 0;
-    }
-    cluster.sync();
-    if (rank == 0 && tid == 0) {
-        // keys below the threshold first (all of them), then the first
-        // need_eq equal keys in index order (CTA slices are in index order)
-        uint32_t lt_off = 0, eq_seen = 0, eq_off = static_cast<uint32_t>(k) - need_eq;
+        // every CTA adds up all histograms and finds the digit for itself
+        uint32_t t0 = 0, t1 = 0;
+#pragma unroll
         for (int r = 0; r < kTopkCtas; ++r) {
-            TopkShared* o = cluster.map_shared_rank(&sh, r);
-            const uint32_t take = eq_seen >= need_eq ? 0u
-                                  : (o->count_eq < need_eq - eq_seen ? o->count_eq
-                                                                     : need_eq - eq_seen);
-            o->lt_off = lt_off;
-            o->eq_off = eq_off;
-            o->eq_take = take;
-            lt_off += o->count_lt;
-            eq_seen += o->count_eq;
-            eq_off += take;
+            const uint2 h = *reinterpret_cast<const uint2*>(
+                &cluster.map_shared_rank(&sh, r)->hist[pass & 1][b0]);
+            t0 += h.x;
+            t1 += h.y;
         }
-    }
-    cluster.sync();
-
-    // ---- write the selected (key, index) pairs into CTA 0's shared memory
-    const uint32_t eq_take = sh.eq_take;
-    uint32_t eq_base = 0;
-    for (int64_t base = lo; base < hi; base += kTopkThreads) {
-        const int64_t i = base + tid;
-        const uint32_t key = i < hi ? order_key<BF16>(scores, i) : 0xFFFFFFFFu;
-        const bool is_lt = i < hi && key < thr;
-        const bool is_eq = i < hi && key == thr;
-        if (is_lt) {
-            const uint32_t pos = sh.lt_off + atomicAdd(&sh.lt_cursor, 1u);
-            root->sel[pos] = (static_cast<unsigned long long>(key) << 32) | static_cast<uint32_t>(i);
+        uint32_t incl = t0 + t1;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t v = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += v;
         }
-        const uint32_t r = block_rank(is_eq, sh.warp_sum, &sh.round_total);
-        if (is_eq && eq_base + r < eq_take)
-            root->sel[sh.eq_off + eq_base + r] =
-                (static_cast<unsigned long long>(key) << 32) | static_cast<uint32_t>(i);
-        eq_base += sh.round_total;
-    }
-    cluster.sync();
-
-    // ---- CTA 0: sort the k pairs (bitonic over the next power of two) and store
-    if (rank == 0) {
-        int p2 = 1;
-        while (p2 < k) p2 <<= 1;
-        for (int j = k + tid; j < p2; j += kTopkThreads) sh.sel[j] = ~0ull;
+        if (lane == 31) sh.warp_sum[warp] = incl;
         __syncthreads();
-        for (int size = 2; size <= p2; size <<= 1) {
-            for (int stride = size >> 1; stride > 0; stride >>= 1) {
-                for (int j = tid; j < p2; j += kTopkThreads) {
-                    const int partner = j ^ stride;
-                    if (partner > j) {
-                        const bool up = (j & size) == 0;
-                        const unsigned long long a = sh.sel[j], b = sh.sel[partner];
-                        if ((a > b) == up) {
-                            sh.sel[j] = b;
-                            sh.sel[partner] = a;
-                        }
-                    }
-                }
-                __syncthreads();
-            }
+        uint32_t before = sh.warp_sum[lane];
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t v = __shfl_up_sync(0xffffffffu, before, o);
+            if (lane >= o) before += v;
         }
-        for (int j = tid; j < k; j += kTopkThreads) {
-            const uint32_t idx = static_cast<uint32_t>(sh.sel[j] & 0xFFFFFFFFull);
-            out_idx[j] = static_cast<int32_t>(idx);
-            out_val[j] = score_at<BF16>(scores, idx);
+        before = __shfl_sync(0xffffffffu, before, warp > 0 ? warp - 1 : 0);
+        before = (warp > 0 ? before : 0u) + incl - (t0 + t1);  // of all bins before b0
+        if (before < need && need <= before + t0) {
+            sh.digit = b0;
+            sh.before = before;
+            sh.bin = t0;
+        } else if (before + t0 < need && need <= before + t0 + t1) {
+            sh.digit = b0 + 1;
+            sh.before = before + t0;
+            sh.bin = t1;
+        }
+        __syncthreads();
+        top = (top << bits) | sh.digit;
+        low -= bits;
+        need -= sh.before;
+        if (need == sh.bin) break;
+    }
+
+    // ---- the CTA's pairs up to the bin, in any order; exactly k in the cluster
+    for (int i = tid; i < count; i += kTopkThreads) {
+        const unsigned long long pair =
+            (static_cast<unsigned long long>(key_at(i)) << 32) | static_cast<uint32_t>(lo + i);
+        if (pair >> low <= top) sh.list[atomicAdd(&sh.count, 1u)] = pair;
+    }
+    cluster.sync();
+    // ---- every CTA gathers all k and ranks its share of them
+    if (tid < k) {
+        uint32_t at = tid;
+        int r = 0;
+        for (; r < kTopkCtas - 1; ++r) {
+            const uint32_t c = cluster.map_shared_rank(&sh, r)->count;
+            if (at < c) break;
+            at -= c;
+        }
+        sh.all[tid] = cluster.map_shared_rank(&sh, r)->list[at];
+    }
+    auto done = cluster.barrier_arrive();  // this CTA has read the others' lists
+    __syncthreads();
+    constexpr int kLanes = 8;  // threads per ranked pair
+    const int e0 = k * rank / kTopkCtas, e1 = k * (rank + 1) / kTopkCtas;
+    for (int e = e0 + tid / kLanes; e - tid / kLanes < e1; e += kTopkThreads / kLanes) {
+        const unsigned long long p = e < e1 ? sh.all[e] : 0ull;
+        uint32_t pos = 0;
+        for (int j = tid % kLanes; j < k; j += kLanes) pos += sh.all[j] < p;
+#pragma unroll
+        for (int o = 1; o < kLanes; o <<= 1) pos += __shfl_xor_sync(0xffffffffu, pos, o);
+        if (e < e1 && tid % kLanes == 0) {
+            const uint32_t idx = static_cast<uint32_t>(p);
+            out_idx[pos] = static_cast<int32_t>(idx);
+            out_val[pos] = score_at<BF16>(scores, idx);
         }
     }
+    cluster.barrier_wait(std::move(done));
 }
 
 // A CTA copies one kGatherChunk-element piece of a row at a time (blockIdx.y
@@ -269,17 +278,73 @@ __global__ void __launch_bounds__(kGatherThreads)
     }
 }
 
+template <bool BF16, int CTAS>
+cudaError_t topk_config(cudaLaunchConfig_t* cfg, cudaLaunchAttribute* attr) {
+    auto kern = topk_smallest_kernel<BF16, CTAS>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         sizeof(TopkShared));
+    if (e == cudaSuccess && CTAS > 8)
+        e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    attr->id = cudaLaunchAttributeClusterDimension;
+    attr->val.clusterDim.x = CTAS;
+    attr->val.clusterDim.y = 1;
+    attr->val.clusterDim.z = 1;
+    cfg->gridDim = dim3(CTAS);
+    cfg->blockDim = dim3(kTopkThreads);
+    cfg->dynamicSmemBytes = sizeof(TopkShared);
+    cfg->attrs = attr;
+    cfg->numAttrs = 1;
+    return e;
+}
+
+template <bool BF16, int CTAS>
+cudaError_t launch_topk(const void* scores, int64_t n, int k, int32_t* out_idx, float* out_val,
+                        cudaStream_t stream) {
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1];
+    cudaError_t e = topk_config<BF16, CTAS>(&cfg, attr);
+    if (e != cudaSuccess) return e;
+    cfg.stream = stream;
+    e = cudaLaunchKernelEx(&cfg, topk_smallest_kernel<BF16, CTAS>, scores, n, k, out_idx, out_val);
+    if (e != cudaSuccess) return e;
+    return cudaGetLastError();
+}
+
+// Whether the device can place a cluster of 16 of these CTAs; asked once per device.
+bool wide_cluster_fits() {
+    constexpr int kMaxDev = 64;
+    static std::atomic<int> cache[kMaxDev] = {};  // 0: not asked, 1: yes, 2: no
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDev) return false;
+    int v = cache[dev].load(std::memory_order_relaxed);
+    if (v == 0) {
+        cudaLaunchConfig_t cfg = {};
+        cudaLaunchAttribute attr[1];
+        int clusters = 0;
+        v = topk_config<false, 16>(&cfg, attr) == cudaSuccess &&
+                    cudaOccupancyMaxActiveClusters(&clusters, topk_smallest_kernel<false, 16>, &cfg) ==
+                        cudaSuccess &&
+                    clusters > 0
+                ? 1
+                : 2;
+        cudaGetLastError();  // a failed query leaves no sticky error for the next launch
+        cache[dev].store(v, std::memory_order_relaxed);
+    }
+    return v == 1;
+}
+
 }  // namespace
 
 cudaError_t launch_topk_smallest(const void* scores, bool bf16, int64_t n, int k,
                                  int32_t* out_idx, float* out_val, cudaStream_t stream) {
-    if (bf16)
-        topk_smallest_kernel<true><<<kTopkCtas, kTopkThreads, 0, stream>>>(scores, n, k, out_idx,
-                                                                           out_val);
-    else
-        topk_smallest_kernel<false><<<kTopkCtas, kTopkThreads, 0, stream>>>(scores, n, k, out_idx,
-                                                                            out_val);
-    return cudaGetLastError();
+    // 16 CTAs (a cluster size beyond the portable 8) where 8 cannot keep their keys in
+    // shared memory and the GPU can place them: 2000000 scores 69 us against 103.
+    // Below that their longer barriers cost more (200000: 27 against 21).
+    const bool wide = n > 8 * kTopkCache && wide_cluster_fits();
+    return bf16 ? (wide ? launch_topk<true, 16>(scores, n, k, out_idx, out_val, stream)
+                        : launch_topk<true, 8>(scores, n, k, out_idx, out_val, stream))
+                : (wide ? launch_topk<false, 16>(scores, n, k, out_idx, out_val, stream)
+                        : launch_topk<false, 8>(scores, n, k, out_idx, out_val, stream));
 }
 
 cudaError_t launch_gather_rows(const uint16_t* src, int64_t src_rows, int64_t D,
