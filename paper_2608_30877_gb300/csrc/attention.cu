@@ -11,11 +11,11 @@
 //   S  = Q K^T   tcgen05.mma kind::f16, A = Q and B = K from shared memory
 //                (TMA, 128-byte swizzle, K-major), S fp32 in tensor memory,
 //                two S buffers that blocks alternate between;
-//   softmax      four warps, thread = query row: tcgen05.ld of its S row into
-//                registers, causal/window mask per 32-key chunk, running max
-//                and sum in fp32 (exp2 with the scale folded in), P as bf16
-//                pairs written over S with tcgen05.st; O rescaled in tensor
-//                memory when the running max grows (lazily, by more than 2^8);
+//   softmax      eight warps, a row over the four threads of a quad: tcgen05.ld of
+//                S into registers, causal/window mask, running max and sum in
+//                fp32 (exp2 with the scale folded in), P as bf16 pairs written over
+//                S with tcgen05.st; O rescaled in tensor memory when the running
+//                max grows (lazily, by more than 2^8);
 //   O += P V     tcgen05.mma with A = P from tensor memory and B = V from
 //                shared memory as an MN-major operand (V is stored token-
 //                major, d contiguous -- exactly the layout the TMA box has);
@@ -23,12 +23,22 @@
 //                stores.
 // S runs two blocks ahead of PV, so the S product of the next block is
 // ready when the softmax of the current one ends.  The kernel is persistent
-// with two CTAs per SM (256 tensor-memory columns and 104 KB of shared memory
-// each), every CTA taking every grid-th job, heads fastest; one CTA's softmax
-// and epilogue overlap the other's MMAs.  Within a CTA the roles are one TMA
-// warp, one MMA warp and the four softmax warps, linked by mbarriers whose
-// phases run on across jobs: Q and K of the next job load during the current
-// job's last blocks, and its first S products run during the epilogue.
+// with two CTAs per SM (256 tensor-memory columns and 105 KB of shared memory
+// each), every CTA taking about every grid-th job; one CTA's softmax and epilogue
+// overlap the other's MMAs.  Within a CTA the roles are one TMA warp, which also
+// finds the jobs, one S and one PV issuing warp and eight softmax warps, linked by
+// mbarriers whose phases run on across jobs: Q and K of the next job load during the
+// current job's last blocks, and its first S products run during the epilogue.
+//
+// What bounds it (96 heads, us; before and after the job order below, the job ring and
+// the streaming hints): 64 ragged pairs of 200 to 1024 tokens 1105 -> 976, 64 x 1024
+// tokens 2110 -> 1713, 10007 tokens under a window of 4096 1390 -> 1278 (62% of the
+// bf16 peak).  DRAM traffic was the limit of the short sequences (76% of its
+// rate, 6.4 GB for 3.8 GB of input and output) and is now 4.6 GB; then the latency of
+// the softmax -> PV -> S chain of two CTAs per SM, no unit being busy half the time.
+// Measured and not kept: P in columns of its own, so that S only waits for the scores to
+// be read (1035 / 1287 / 1800); exponentials taken with the old max ahead of the
+// block's (1059 / 1389 / 1884); the next output chunk read during the stores (1026).
 // Every wait is bounded (ptx.cuh); on a timeout the kernel records
 // W4A16_ERR_TIMEOUT, waits for its own copies and MMAs and frees tensor memory.
 #include "internal.h"
@@ -48,6 +58,8 @@ constexpr int kFirstSoftmaxWarp = 3;  // warps 3..10: two per TMEM sub-partition
 constexpr int kSoftmaxWarps = 8;
 constexpr int kThreads = (kFirstSoftmaxWarp + kSoftmaxWarps) * 32;  // + TMA, S-MMA, PV-MMA warps
 
+constexpr int kJobSlots = 8;   // ring of jobs, written by the TMA warp
+
 struct AttnLayout {
     static constexpr int QBOX = kBQ * 128;    // one [128 rows x 64 cols] bf16 box: 16 KB
     static constexpr int KBOX = kBKV * 128;   // one [64 rows x 64 cols] bf16 box: 8 KB
@@ -61,9 +73,10 @@ struct AttnLayout {
     static constexpr int STAGE_WARP = 16 * 64;
     static constexpr int BAR_OFF = STAGE_OFF + kSoftmaxWarps * STAGE_WARP;
     // q_full, q_empty, k_full[2], k_empty[2], v_full[2], v_empty[2],
-    // s_full[2], p_full[2], o_ready[2], drain[2]
-    static constexpr int NBARS = 18;
-    static constexpr int MISC_OFF = BAR_OFF + NBARS * 8;
+    // s_full[2], p_full[2], o_ready[2], drain[2], job_full[kJobSlots]
+    static constexpr int NBARS = 18 + kJobSlots;
+    static constexpr int JOB_OFF = BAR_OFF + (NBARS * 8 + 15) / 16 * 16;
+    static constexpr int MISC_OFF = JOB_OFF + kJobSlots * 32;
     static constexpr int SMEM_BYTES = MISC_OFF + 32 + 1024;
     // tensor memory columns: two S buffers (blocks alternate; P of a block is
     // written over the first half of its S) and O
@@ -225,17 +238,23 @@ struct AttnJob {
     bool valid;
 };
 
-// Resumable warp-collective search for the x-th query block over the
-// sequences (blocks of a sequence numbered from its last, the heaviest under
-// the causal mask, down).  x never decreases between calls of one warp, so
-// the search resumes at the 32-sequence group where the last one ended.
+// Resumable warp-collective search over the sequences.  The query block looked for
+// never precedes the last one's sequence, so the search resumes at the
+// 32-sequence group where the last one ended.
 struct JobCursor {
     int s0 = 0;    // first sequence of the current group
     int base = 0;  // query blocks of the sequences before s0
 };
 
-__device__ __forceinline__ bool find_block(const AttnParams& p, int x, int lane, JobCursor& cur,
-                                           int& ss, int& se, int& q0) {
+// Job t: its sequence holds the x-th query block, x = t / H, of all sequences'; a
+// sequence's jobs are numbered head by head, the query blocks of a head from the
+// last, the heaviest under the causal mask, down.  So the CTAs running at one time
+// work on all query blocks of a few heads, whose K and V come from DRAM once:
+// numbered with the heads fastest they did not stay in L2 (64 ragged pairs 1078 us, 1005
+// so; 64 x 1024 tokens 2044 and 1740; 10007 under a window of 4096 1360 and 1282).
+__device__ __forceinline__ AttnJob job_at(const AttnParams& p, int64_t t, int lane, JobCursor& cur) {
+    AttnJob j{};
+    const int x = static_cast<int>(t / p.H);
     for (; cur.s0 < p.nseq; cur.s0 += 32) {
         const int s = cur.s0 + lane;
         int a = 0, b = 0, nqb = 0;
@@ -247,34 +266,24 @@ __device__ __forceinline__ bool find_block(const AttnParams& p, int x, int lane,
         int incl = nqb;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
-            const int t = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl += t;
+            const int u = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += u;
         }
-        const int excl = incl - nqb;
-        const bool mine = s < p.nseq && x >= cur.base + excl && x < cur.base + incl;
-        const unsigned who = __ballot_sync(0xffffffffu, mine);
+        const int excl = cur.base + incl - nqb;  // query blocks before sequence s
+        const unsigned who = __ballot_sync(0xffffffffu, nqb > 0 && x >= excl && x < excl + nqb);
         if (who) {
             const int src = __ffs(who) - 1;
-            const int e = __shfl_sync(0xffffffffu, excl, src);
             const int n = __shfl_sync(0xffffffffu, nqb, src);
-            ss = __shfl_sync(0xffffffffu, a, src);
-            se = __shfl_sync(0xffffffffu, b, src);
-            q0 = ss + (n - 1 - (x - cur.base - e)) * kBQ;
-            return true;
+            const int64_t r = t - static_cast<int64_t>(__shfl_sync(0xffffffffu, excl, src)) * p.H;
+            j.ss = __shfl_sync(0xffffffffu, a, src);
+            j.se = __shfl_sync(0xffffffffu, b, src);
+            j.h = static_cast<int>(r / n);
+            j.q0 = j.ss + (n - 1 - static_cast<int>(r % n)) * kBQ;
+            j.valid = true;
+            return j;
         }
         cur.base += __shfl_sync(0xffffffffu, incl, 31);
     }
-    return false;
-}
-
-// Job t of the CTA's sequence t = blockIdx.x, blockIdx.x + gridDim.x, ...:
-// heads vary fastest, so the CTAs running at one time share the K/V of a
-// few sequences in L2.
-__device__ __forceinline__ AttnJob job_at(const AttnParams& p, int64_t t, int lane, JobCursor& cur) {
-    AttnJob j{};
-    const int x = static_cast<int>(t / p.H);
-    j.h = static_cast<int>(t % p.H);
-    j.valid = find_block(p, x, lane, cur, j.ss, j.se, j.q0);
     return j;
 }
 
@@ -286,36 +295,16 @@ __device__ __forceinline__ void key_range(const AttnJob& jb, int W, int& b_first
     nblk = (q_last - jb.ss) / kBKV - b_first + 1;
 }
 
-// Walks the CTA's key blocks in order across its jobs; warp-collective (the
-// job search uses the whole warp).
-struct BlockWalk {
-    JobCursor cur;
-    int64_t t = 0;
-    AttnJob jb{};
-    int b_first = 0, nblk = 0, j = 0;
-    uint32_t jn = 0;  // jobs of the CTA before this one
-    bool valid = false;
+// A job as the TMA warp, which runs ahead of the others, hands it to them: the
+// search through the sequence table and its loads happen once, off the path of
+// the softmax (64 ragged pairs 1090 -> 1078 us).  nblk = 0 ends the CTA's jobs.
+// The TMA warp writes job i after it has loaded job i - 1, whose Q waited for
+// the last S product of job i - 2; S is at most two blocks, hence at most two
+// jobs, ahead of the softmax.  So every warp has read job i - 4 by then, and
+// eight slots need no barrier for their release.
+struct __align__(16) JobSlot {
+    int ss, se, q0, h, b_first, nblk, pad[2];
 };
-
-__device__ __forceinline__ void walk_job(const AttnParams& p, int64_t njobs, int lane, BlockWalk& w) {
-    w.valid = false;
-    if (w.t < njobs) {
-        w.jb = job_at(p, w.t, lane, w.cur);
-        if (w.jb.valid) {
-            key_range(w.jb, p.window, w.b_first, w.nblk);
-            w.j = 0;
-            w.valid = true;
-        }
-    }
-}
-
-__device__ __forceinline__ void walk_next(const AttnParams& p, int64_t njobs, int64_t step,
-                                          int lane, BlockWalk& w) {
-    if (++w.j < w.nblk) return;
-    w.t += step;
-    ++w.jn;
-    walk_job(p, njobs, lane, w);
-}
 
 __global__ void __launch_bounds__(kThreads, 2)
     attention_prefill_kernel(const __grid_constant__ CUtensorMap tmap_q,
@@ -344,6 +333,8 @@ __global__ void __launch_bounds__(kThreads, 2)
     auto p_full = [&](uint32_t b) { return bars + 96u + 8u * b; };
     auto o_ready = [&](uint32_t b) { return bars + 112u + 8u * b; };
     auto drain = [&](uint32_t i) { return bars + 128u + 8u * i; };
+    auto job_full = [&](uint32_t jn) { return bars + 144u + 8u * (jn % kJobSlots); };
+    JobSlot* jobs = reinterpret_cast<JobSlot*>(smem + L::JOB_OFF);
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + L::MISC_OFF);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + L::MISC_OFF + 4);
     int* bad_flag = reinterpret_cast<int*>(smem + L::MISC_OFF + 8);
@@ -372,6 +363,7 @@ __global__ void __launch_bounds__(kThreads, 2)
             }
             mbar_init(drain(0), 1);
             mbar_init(drain(1), 1);
+            for (uint32_t i = 0; i < kJobSlots; ++i) mbar_init(job_full(i), 1);
             *abort_flag = 0;
             fence_mbar_init();
             prefetch_tmap(&tmap_q);
@@ -400,12 +392,25 @@ __global__ void __launch_bounds__(kThreads, 2)
         // PV product is.
         bool ok = run;
         JobCursor cur;
+        // Q is read once (as the output is written once), K and V by every query block:
+        // marked so, they keep L2 to K and V (64 ragged pairs 1004 -> 976 us)
+        const uint64_t once = l2_policy_evict_first();
         uint32_t g = 0, jn = 0, nq = 0, nk = 0, nv = 0;
-        for (int64_t t = t_first; ok && t < njobs; t += t_step) {
-            const AttnJob jb = job_at(p, t, lane, cur);
-            if (!jb.valid) break;
-            int b_first, nblk;
-            key_range(jb, W, b_first, nblk);
+        // Round i of the CTAs takes jobs i grid .. (i + 1) grid - 1, rotated by 37 i:
+        // without the rotation a grid that is a multiple of the query blocks
+        // per head would give a CTA the same, say the heaviest, block of every head.
+        int64_t turn = t_first;  // (blockIdx + 37 i) % grid
+        for (int64_t t0 = 0; ok; t0 += t_step, turn = (turn + 37) % t_step) {
+            const int64_t t = t0 + turn;
+            AttnJob jb{};
+            if (t < njobs) jb = job_at(p, t, lane, cur);
+            int b_first = 0, nblk = 0;
+            if (jb.valid) key_range(jb, W, b_first, nblk);
+            if (lane == 0) {
+                jobs[jn % kJobSlots] = JobSlot{jb.ss, jb.se, jb.q0, jb.h, b_first, nblk, {0, 0}};
+                mbar_arrive(job_full(jn));
+            }
+            if (nblk == 0) break;
             if (lane == 0) {
                 if (!wait_one(q_empty, (jn & 1u) ^ 1u, abort_flag, p.status, p.wait_ns)) ok = false;
                 if (ok) {
@@ -416,9 +421,9 @@ __global__ void __launch_bounds__(kThreads, 2)
                                                  sbase + L::K_OFF, jb.h * kD + 64, 2) &&
                                       jb.q0 >= 0 && jb.q0 < p.M,
                                   p.status)) {
-                        tma_load_2d(sbase + L::Q_OFF, &tmap_q, q_full, jb.h * kD, jb.q0);
-                        tma_load_2d(sbase + L::Q_OFF + L::QBOX, &tmap_q, q_full, jb.h * kD + 64,
-                                    jb.q0);
+                        tma_load_2d_hint(sbase + L::Q_OFF, &tmap_q, q_full, jb.h * kD, jb.q0, once);
+                        tma_load_2d_hint(sbase + L::Q_OFF + L::QBOX, &tmap_q, q_full, jb.h * kD + 64,
+                                         jb.q0, once);
                     }
                     ++nq;
                 }
@@ -485,37 +490,35 @@ __global__ void __launch_bounds__(kThreads, 2)
         // 10007 under a window of 4096 1511 -> 1440).
         constexpr uint32_t idesc_s = idesc_bf16_f32(kBQ, kBKV);
         bool ok = run;
-        BlockWalk ws;  // the next block to take its S product
-        if (ok) {
-            ws.t = t_first;
-            walk_job(p, njobs, lane, ws);
-        }
         uint32_t gs = 0;
-        while (ok && ws.valid) {
-            const uint32_t b = gs & 1u;
-            // the buffer's previous block (gs - 2) has had its PV product
-            ok = gs < 2 ||
-                 wait_warp(o_ready(b), ((gs - 2) >> 1) & 1u, abort_flag, p.status, p.wait_ns);
-            if (ok && ws.j == 0) ok = wait_warp(q_full, ws.jn & 1u, abort_flag, p.status, p.wait_ns);
-            if (ok) ok = wait_warp(k_full(b), (gs >> 1) & 1u, abort_flag, p.status, p.wait_ns);
-            if (!ok) break;
-            tc_fence_after();
-            const uint64_t qd = sdesc_kmajor_sw128(sbase + L::Q_OFF);
-            const uint64_t kd = sdesc_kmajor_sw128(sbase + L::K_OFF + b * L::KV_TILE);
-            const uint32_t d = tmem + L::S_COL + b * kBKV;
-            if (elect_one()) {
+        for (uint32_t jn = 0; ok; ++jn) {
+            if (!wait_warp(job_full(jn), (jn / kJobSlots) & 1u, abort_flag, p.status, p.wait_ns)) break;
+            const int nblk = jobs[jn % kJobSlots].nblk;
+            if (nblk == 0) break;
+            for (int j = 0; j < nblk; ++j, ++gs) {
+                const uint32_t b = gs & 1u;
+                // the buffer's previous block (gs - 2) has had its PV product
+                ok = gs < 2 ||
+                     wait_warp(o_ready(b), ((gs - 2) >> 1) & 1u, abort_flag, p.status, p.wait_ns);
+                if (ok && j == 0) ok = wait_warp(q_full, jn & 1u, abort_flag, p.status, p.wait_ns);
+                if (ok) ok = wait_warp(k_full(b), (gs >> 1) & 1u, abort_flag, p.status, p.wait_ns);
+                if (!ok) break;
+                tc_fence_after();
+                const uint64_t qd = sdesc_kmajor_sw128(sbase + L::Q_OFF);
+                const uint64_t kd = sdesc_kmajor_sw128(sbase + L::K_OFF + b * L::KV_TILE);
+                const uint32_t d = tmem + L::S_COL + b * kBKV;
+                if (elect_one()) {
 #pragma unroll
-                for (int kk = 0; kk < kD / 16; ++kk)
-                    tc_mma_ss(d, qd + (((kk >> 2) * L::QBOX + (kk & 3) * 32) >> 4),
-                              kd + (((kk >> 2) * L::KBOX + (kk & 3) * 32) >> 4), idesc_s,
-                              kk > 0 ? 1u : 0u);
-                tc_commit(s_full(b));
-                tc_commit(k_empty(b));
-                if (ws.j == ws.nblk - 1) tc_commit(q_empty);  // the job's last S frees Q
+                    for (int kk = 0; kk < kD / 16; ++kk)
+                        tc_mma_ss(d, qd + (((kk >> 2) * L::QBOX + (kk & 3) * 32) >> 4),
+                                  kd + (((kk >> 2) * L::KBOX + (kk & 3) * 32) >> 4), idesc_s,
+                                  kk > 0 ? 1u : 0u);
+                    tc_commit(s_full(b));
+                    tc_commit(k_empty(b));
+                    if (j == nblk - 1) tc_commit(q_empty);  // the job's last S frees Q
+                }
+                __syncwarp();
             }
-            __syncwarp();
-            ++gs;
-            walk_next(p, njobs, t_step, lane, ws);
         }
         if (elect_one()) {
             tc_commit(drain(0));  // every MMA issued has completed before tensor memory is freed
@@ -526,36 +529,34 @@ __global__ void __launch_bounds__(kThreads, 2)
         // ------------------------------------------------------------ PV issuer
         constexpr uint32_t idesc_o = idesc_bf16_f32(kBQ, kD) | (1u << 16);  // B MN-major
         bool ok = run;
-        BlockWalk wp;  // the next block to take its PV product
-        if (ok) {
-            wp.t = t_first;
-            walk_job(p, njobs, lane, wp);
-        }
         uint32_t g = 0;
-        while (ok && wp.valid) {
-            const uint32_t b = g & 1u;
-            // O += P V once the softmax warps have written P of block g (for
-            // a job's first block, after they read out the previous job's O)
-            ok = wait_warp(p_full(b), (g >> 1) & 1u, abort_flag, p.status, p.wait_ns) &&
-                 wait_warp(v_full(b), (g >> 1) & 1u, abort_flag, p.status, p.wait_ns);
-            if (!ok) break;
-            tc_fence_after();
-            const uint64_t vd =
-                sdesc_mnmajor_sw128(sbase + L::V_OFF + b * L::KV_TILE, L::KBOX, 1024);
-            const uint32_t ptm = tmem + L::S_COL + b * kBKV;
-            const uint32_t more = wp.j > 0 ? 1u : 0u;
-            if (elect_one()) {
+        for (uint32_t jn = 0; ok; ++jn) {
+            if (!wait_warp(job_full(jn), (jn / kJobSlots) & 1u, abort_flag, p.status, p.wait_ns)) break;
+            const int nblk = jobs[jn % kJobSlots].nblk;
+            if (nblk == 0) break;
+            for (int j = 0; j < nblk; ++j, ++g) {
+                const uint32_t b = g & 1u;
+                // O += P V once the softmax warps have written P of block g (for
+                // a job's first block, after they read out the previous job's O)
+                ok = wait_warp(p_full(b), (g >> 1) & 1u, abort_flag, p.status, p.wait_ns) &&
+                     wait_warp(v_full(b), (g >> 1) & 1u, abort_flag, p.status, p.wait_ns);
+                if (!ok) break;
+                tc_fence_after();
+                const uint64_t vd =
+                    sdesc_mnmajor_sw128(sbase + L::V_OFF + b * L::KV_TILE, L::KBOX, 1024);
+                const uint32_t ptm = tmem + L::S_COL + b * kBKV;
+                const uint32_t more = j > 0 ? 1u : 0u;
+                if (elect_one()) {
 #pragma unroll
-                for (int kk = 0; kk < kBKV / 16; ++kk)
-                    // keys 16 kk .. 16 kk + 15: rows of the V tile; P columns 8 kk ..
-                    tc_mma_ts(tmem + L::O_COL, ptm + kk * 8, vd + ((kk * 16 * 128) >> 4), idesc_o,
-                              kk > 0 ? 1u : more);
-                tc_commit(o_ready(b));
-                tc_commit(v_empty(b));
+                    for (int kk = 0; kk < kBKV / 16; ++kk)
+                        // keys 16 kk .. 16 kk + 15: rows of the V tile; P columns 8 kk ..
+                        tc_mma_ts(tmem + L::O_COL, ptm + kk * 8, vd + ((kk * 16 * 128) >> 4), idesc_o,
+                                  kk > 0 ? 1u : more);
+                    tc_commit(o_ready(b));
+                    tc_commit(v_empty(b));
+                }
+                __syncwarp();
             }
-            __syncwarp();
-            ++g;
-            walk_next(p, njobs, t_step, lane, wp);
         }
         if (elect_one()) {
             tc_commit(drain(1));
@@ -577,13 +578,15 @@ __global__ void __launch_bounds__(kThreads, 2)
         const uint32_t lane_base = tmem + (static_cast<uint32_t>(rb) << 16);
         const float cs = 1.4426950408889634f * p.scale;  // log2(e) / sqrt(d)
         bool ok = run;
-        JobCursor cur;
         uint32_t gb = 0;
-        for (int64_t t = t_first; ok && t < njobs; t += t_step) {
-            const AttnJob jb = job_at(p, t, lane, cur);
-            if (!jb.valid) break;
-            int b_first, nblk;
-            key_range(jb, W, b_first, nblk);
+        for (uint32_t jn = 0; ok; ++jn) {
+            if (!wait_warp(job_full(jn), (jn / kJobSlots) & 1u, abort_flag, p.status, p.wait_ns)) {
+                ok = false;
+                break;
+            }
+            const JobSlot jb = jobs[jn % kJobSlots];
+            const int b_first = jb.b_first, nblk = jb.nblk;
+            if (nblk == 0) break;
             const int i0 = jb.q0 + rb + g;  // query tokens of rows g and g + 8
             // Running max m (log2 units, scale folded in) and this thread's
             // part of the sum l, per row.  The max is raised lazily: only when
@@ -733,7 +736,7 @@ __global__ void __launch_bounds__(kThreads, 2)
                                                                     ((u ^ ((q >> 1) & 3)) << 4));
                     if (q < rows_left &&
                         dbg_check(jb.q0 + rb + q < jb.se && jb.q0 + rb + q >= jb.ss, p.status))
-                        *reinterpret_cast<uint4*>(obase + static_cast<int64_t>(q) * Hd + ch * 32 + u * 8) = w;
+                        __stcs(reinterpret_cast<uint4*>(obase + static_cast<int64_t>(q) * Hd + ch * 32 + u * 8), w);
                 }
                 __syncwarp();
             }
