@@ -222,6 +222,16 @@ int w4a16_attention_prefill(const void* qkv_bf16, const void* seq_start_i32, int
                             void* stream);
 
 /*
+ * Zeroes the rows of out that w4a16_attention_prefill leaves untouched: tokens
+ * outside every sequence, or all of them if the table is bad (nothing is
+ * recorded here).  With both calls on one stream, in either order, every row of
+ * out is written, without a pass over the rows attention writes anyway.
+ * Arguments and checks as there (H * d columns).
+ */
+int w4a16_attention_zero_outside(const void* seq_start_i32, int64_t nseq, int64_t M, int64_t H,
+                                 int64_t d, void* out_bf16, void* stream);
+
+/*
  * Scoring readout, the last modules of the screening pipeline (Sec. 3.3):
  * the affinity head reads one hidden state per pair of the packed batch
  * (w4a16_gather_rows, then w4a16_linear_fused with the head's weights and

@@ -562,6 +562,25 @@ extern "C" int w4a16_attention_prefill(const void* qkv_bf16, const void* seq_sta
                : W4A16_ERR_CUDA;
 }
 
+extern "C" int w4a16_attention_zero_outside(const void* seq_start_i32, int64_t nseq, int64_t M,
+                                            int64_t H, int64_t d, void* out_bf16, void* stream) {
+    if (seq_start_i32 == nullptr || out_bf16 == nullptr) return W4A16_ERR_INVALID_ARG;
+    if (nseq <= 0 || M <= 0 || H <= 0 || d <= 0) return W4A16_ERR_INVALID_ARG;
+    if (d != attention_head_dim()) return W4A16_ERR_UNSUPPORTED;
+    if (M > kMaxDim || nseq > kMaxDim / 2 || H > 65535) return W4A16_ERR_UNSUPPORTED;
+    if (!aligned16(seq_start_i32) || !aligned16(out_bf16)) return W4A16_ERR_ALIGNMENT;
+    if (overlaps(out_bf16, M * H * d * 2, seq_start_i32, (nseq + 1) * 4))
+        return W4A16_ERR_INVALID_ARG;
+    DeviceState* st = nullptr;
+    const int rc = device_state(&st);
+    if (rc != W4A16_OK) return rc;
+    return launch_zero_outside(static_cast<const int32_t*>(seq_start_i32), static_cast<int>(nseq), M,
+                               H * d, static_cast<uint16_t*>(out_bf16), st->sm_count,
+                               static_cast<cudaStream_t>(stream)) == cudaSuccess
+               ? W4A16_OK
+               : W4A16_ERR_CUDA;
+}
+
 extern "C" int w4a16_gather_rows(const void* src_bf16, int64_t src_rows, int64_t D,
                                  const void* index_i32, int64_t P, void* dst_bf16,
                                  void* stream) {

@@ -750,7 +750,34 @@ __global__ void __launch_bounds__(kThreads, 2)
     if (warp == 1) tmem_dealloc(tmem, L::TMEM_COLS);
 }
 
+// Zeroes the output rows that attention_prefill_kernel leaves untouched: the
+// tokens before the first sequence and after the last (sequences lie back to
+// back), or every row if the table is bad.
+__global__ void __launch_bounds__(256)
+    zero_outside_kernel(const int32_t* __restrict__ seq_start, int nseq, int64_t M,
+                        int64_t row_chunks, uint4* __restrict__ out) {
+    int bad = 0;
+    for (int s = threadIdx.x; s < nseq; s += blockDim.x) {
+        const int a = seq_start[s], b = seq_start[s + 1];
+        if (a < 0 || b < a || b > M) bad = 1;
+    }
+    bad = __syncthreads_or(bad);
+    const int64_t head = (bad ? M : seq_start[0]) * row_chunks;
+    const int64_t tail = (bad ? M : seq_start[nseq]) * row_chunks, end = M * row_chunks;
+    const int64_t first = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
+    const int64_t step = static_cast<int64_t>(gridDim.x) * blockDim.x;
+    for (int64_t i = first; i < head; i += step) out[i] = make_uint4(0, 0, 0, 0);
+    for (int64_t i = tail + first; i < end; i += step) out[i] = make_uint4(0, 0, 0, 0);
+}
+
 }  // namespace
+
+cudaError_t launch_zero_outside(const int32_t* seq_start, int nseq, int64_t M, int64_t row_elems,
+                                uint16_t* out, int sm_count, cudaStream_t stream) {
+    zero_outside_kernel<<<2 * sm_count, 256, 0, stream>>>(seq_start, nseq, M, row_elems / 8,
+                                                          reinterpret_cast<uint4*>(out));
+    return cudaGetLastError();
+}
 
 cudaError_t launch_attention_prefill(const CUtensorMap* tmap_q, const CUtensorMap* tmap_kv,
                                      const AttnParams& p, cudaStream_t stream) {

@@ -121,6 +121,10 @@ int attention_key_block();
 cudaError_t launch_attention_prefill(const CUtensorMap* tmap_q, const CUtensorMap* tmap_kv,
                                      const AttnParams& p, cudaStream_t stream);
 
+// Zeroes the rows of out [M, row_elems] outside every sequence.
+cudaError_t launch_zero_outside(const int32_t* seq_start, int nseq, int64_t M, int64_t row_elems,
+                                uint16_t* out, int sm_count, cudaStream_t stream);
+
 // Scoring readout (readout.cu).
 constexpr int kTopkMaxK = 1024;  // largest k of the top-k
 cudaError_t launch_topk_smallest(const void* scores, bool bf16, int64_t n, int k,

@@ -61,6 +61,7 @@ def lib() -> ctypes.CDLL:
         L.w4a16_stack_graph_destroy.argtypes = [p]
         L.w4a16_gather_rows.argtypes = [p, i64, i64, p, i64, p, p]
         L.w4a16_attention_prefill.argtypes = [p, p, i64, i64, i64, i64, i64, p, p]
+        L.w4a16_attention_zero_outside.argtypes = [p, i64, i64, i64, i64, p, p]
         L.w4a16_topk_smallest.argtypes = [p, ctypes.c_int, i64, i64, p, p, p]
         L.w4a16_quantize.argtypes = [p, p, p, i64, i64, i64, p]
         L.w4a16_get_device_error.argtypes = [p]
@@ -71,7 +72,7 @@ def lib() -> ctypes.CDLL:
         L.w4a16_version.restype = ctypes.c_int
         for f in ("w4a16_linear", "w4a16_linear_fused", "w4a16_linear_stack",
                   "w4a16_gather_rows", "w4a16_topk_smallest", "w4a16_attention_prefill",
-                  "w4a16_stack_graph_create", "w4a16_stack_graph_launch",
+                  "w4a16_attention_zero_outside", "w4a16_stack_graph_create", "w4a16_stack_graph_launch",
                   "w4a16_stack_graph_destroy", "w4a16_dequant", "w4a16_quantize",
                   "w4a16_get_device_error", "w4a16_selftest_wait_timeout",
                   "w4a16_selftest_set_wait_limit"):
@@ -201,13 +202,17 @@ def attention_prefill(qkv: torch.Tensor, seq_start: torch.Tensor, H: int, window
     qkv bf16 [M, 3 H 128], seq_start int32 [nseq + 1] -> out bf16 [M, H 128]."""
     M = qkv.shape[0]
     d = qkv.shape[1] // (3 * H)
-    if out is None:
-        out = torch.zeros((M, H * d), dtype=torch.bfloat16, device=qkv.device)
+    fresh = out is None
+    if fresh:
+        out = torch.empty((M, H * d), dtype=torch.bfloat16, device=qkv.device)
     _need_cuda(qkv, seq_start, out)
     assert qkv.dtype == torch.bfloat16 and seq_start.dtype == torch.int32
     _check("w4a16_attention_prefill", lib().w4a16_attention_prefill(
         qkv.data_ptr(), seq_start.data_ptr(), seq_start.shape[0] - 1, M, H, d, int(window),
         out.data_ptr(), _stream(stream)))
+    if fresh:  # tokens outside every sequence are zero
+        _check("w4a16_attention_zero_outside", lib().w4a16_attention_zero_outside(
+            seq_start.data_ptr(), seq_start.shape[0] - 1, M, H, d, out.data_ptr(), _stream(stream)))
     return out
 
 
