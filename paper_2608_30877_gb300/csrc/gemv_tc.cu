@@ -127,43 +127,6 @@ __device__ __forceinline__ float ld_shared_cluster_f32(uint32_t addr) {
     return v;
 }
 
-// Residual of one row (lane) and token m of the fused epilogue, 0 where there is none.
-// Read for a whole slice before any of its outputs is stored: the residual may be
-// the output, so the compiler keeps loads and stores in order, and one at a time they
-// are a chain of memory latencies (333 x 12288 x 12288 with a residual 117 us, 93 so).
-template <bool FUSED>
-__device__ __forceinline__ float residual_at(const GemvParams& p, int m, int m_end, int n,
-                                             bool valid, int lane) {
-    const Epilogue& ep = p.epi;
-    const bool glu = ep.act == kActSwiGLU;
-    if (!FUSED || ep.residual == nullptr || !valid || m >= m_end || (glu && (lane & 1) != 0))
-        return 0.0f;
-    return bf16_to_f32(ep.residual[static_cast<int64_t>(m) * ep.n_out + (glu ? n >> 1 : n)]);
-}
-
-// Output of one row (lane) and token m (if below m_end) from the finished sum, with
-// the fused epilogue.  SwiGLU pairs rows (n, n ^ 1) = (gate, up): RB is even, so n
-// has the parity of its lane and the partner is lane ^ 1 (all lanes call).
-template <bool FUSED>
-__device__ __forceinline__ void finish(const GemvParams& p, float acc, float bias, float residual,
-                                       int m, int m_end, int n, bool valid, int lane) {
-    const Epilogue& ep = p.epi;
-    if constexpr (!FUSED) {
-        if (valid && m < m_end) p.out[static_cast<int64_t>(m) * p.N + n] = f32_to_bf16_rn(acc);
-    } else {
-        const float z = acc + bias;
-        if (ep.act == kActSwiGLU) {
-            const float up = __shfl_xor_sync(0xffffffffu, z, 1);
-            if ((lane & 1) == 0 && valid && m < m_end)
-                p.out[static_cast<int64_t>(m) * ep.n_out + (n >> 1)] =
-                    f32_to_bf16_rn(silu_f32(z) * up + residual);
-        } else if (valid && m < m_end) {
-            const float h = ep.act == kActGELU ? gelu_f32(z) : z;
-            p.out[static_cast<int64_t>(m) * ep.n_out + n] = f32_to_bf16_rn(h + residual);
-        }
-    }
-}
-
 // Sums of one row over the SP CTAs of the cluster, in the order of the ranks,
 // and their output: the tokens [rank 32 / SP, ..) of a slice of 32.  All the
 // remote loads are issued before the first sum (one round trip per slice).
@@ -172,23 +135,21 @@ __device__ __forceinline__ void reduce_slice(const GemvParams& p, uint32_t part,
                                              int r, float bias, int m, int m_end, int n, bool valid,
                                              int lane) {
     constexpr int PER = 32 / SP;
-    float v[SP][PER], res[PER];
-#pragma unroll
-    for (int j = 0; j < PER; ++j)
-        res[j] = residual_at<FUSED>(p, m + rank * PER + j, m_end, n, valid, lane);
+    float v[SP][PER];
 #pragma unroll
     for (int c = 0; c < SP; ++c) {
         const uint32_t at = mapa_shared(part + 4u * (rank * PER * pitch + r), c);
 #pragma unroll
         for (int j = 0; j < PER; ++j) v[c][j] = ld_shared_cluster_f32(at + 4u * j * pitch);
     }
+    float sum[PER];
 #pragma unroll
     for (int j = 0; j < PER; ++j) {
-        float sum = v[0][j];
+        sum[j] = v[0][j];
 #pragma unroll
-        for (int c = 1; c < SP; ++c) sum += v[c][j];
-        finish<FUSED>(p, sum, bias, res[j], m + rank * PER + j, m_end, n, valid, lane);
+        for (int c = 1; c < SP; ++c) sum[j] += v[c][j];
     }
+    store_tokens<FUSED, PER>(p.epi, p.out, sum, m + rank * PER, m_end, n, valid, bias, lane);
 }
 
 template <int NTOK, int TILES, bool FUSED, bool SPLIT>
@@ -521,16 +482,12 @@ __global__ void __launch_bounds__(TLayout<NTOK, TILES>::THREADS, 1)
 #pragma unroll 1
                 for (int m0 = 0; mt + m0 < m_end; m0 += L::EC) {
                     uint32_t d[32];
-                    float res[L::EC];
+                    float v[L::EC];
                     tmem_ld_32x32b_x32(lane_base + t * NTOK + m0, d);
-#pragma unroll
-                    for (int j = 0; j < L::EC; ++j)
-                        res[j] = residual_at<FUSED>(p, mt + m0 + j, m_end, n, valid, lane);
                     tmem_ld_wait(d);
 #pragma unroll
-                    for (int j = 0; j < L::EC; ++j)
-                        finish<FUSED>(p, __uint_as_float(d[j]), bias, res[j], mt + m0 + j, m_end, n,
-                                      valid, lane);
+                    for (int j = 0; j < L::EC; ++j) v[j] = __uint_as_float(d[j]);
+                    store_tokens<FUSED, L::EC>(p.epi, p.out, v, mt + m0, m_end, n, valid, bias, lane);
                 }
                 tc_fence_before();
                 __syncwarp();

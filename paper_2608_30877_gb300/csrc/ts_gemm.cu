@@ -24,7 +24,8 @@
 //               32-token chunks: tcgen05.ld of the accumulator, the fused
 //               epilogue if any (bias, activation, residual), fp32 -> bf16,
 //               stores to out.  The next tile's MMAs wait until the
-//               accumulator is drained, so two groups halve that wait.
+//               accumulator is drained, so two groups halve that wait (four
+//               with a fused epilogue, whose arithmetic is the longer part).
 // A warp may only touch the 32 TMEM lanes of its sub-partition (warp % 4), so
 // each group of four warps covers all 128 lanes.
 //
@@ -46,6 +47,10 @@ constexpr int kRows = 128;  // weight rows per tile (MMA M)
 #endif
 constexpr uint32_t kEpilogueSleepNs = W4A16_EPI_SLEEP_NS;
 constexpr int kBK = 64;     // k per stage (one 128-byte swizzle row of bf16)
+// Epilogue groups of four warps.  Fused, four against two: 8192 x 49152 x 12288
+// SwiGLU 11.46 against 11.57 ms, 200 x 36864 x 12288 residual 124.5 against 127.5 us;
+// plain, four lose (1024 x 12288 x 12288 192 against 188 us).
+constexpr int kPlainEP = 2, kFusedEP = 4;
 
 // PAIR: a CTA pair (cta_group::2) computes 2 x 128 weight rows x T tokens;
 // each CTA stages T/2 tokens of x and its own 128 weight rows.  NB: the tile's
@@ -122,149 +127,39 @@ __device__ __forceinline__ void unit_tile(int unit, const TsParams& p, int rank,
     wt = wu * CW + rank;
 }
 
-__device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
-    uint32_t r;
-    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
-    return r;
-}
-
-// Fused epilogue of one tile for the epilogue thread that owns weight row n
-// (TMEM lane `lane` of its sub-partition): the 32-token chunks c0, c0 + cs,
-// ... of the T tokens from TMEM column d_col.  Residuals of a chunk are read
-// before any of its outputs is written (the residual may be the output).
-// SwiGLU pairs rows (n, n ^ 1) = (gate, up) of output column n / 2 across
-// neighbouring lanes: the even lane finishes the even tokens, the odd lane
-// the odd ones.  Otherwise neighbouring lanes swap values so that each store
-// writes the outputs (n, n+1) of one token as a 32-bit word (even n_out).
-template <int T>
-__device__ __forceinline__ void fused_epilogue_tile(const TsParams& p, uint32_t d_col, int m0,
-                                                    int n, int lane, int c0, int cs) {
-    const Epilogue& e = p.epi;
-    const bool n_ok = n < p.N;
-    const bool has_res = e.residual != nullptr;
-    const float b = (e.bias != nullptr && n_ok) ? bf16_to_f32(e.bias[n]) : 0.0f;
-    const bool odd = (lane & 1) != 0;
+// Epilogue of one tile for the epilogue thread that owns weight row n (TMEM lane
+// `lane` of its sub-partition): the 32-token chunks c0, c0 + cs, ... of the T tokens
+// from TMEM column d_col; fused, 16 tokens at a time (32 spill next to the residuals;
+// plain, 16 at a time are slower: 200 x 36864 x 12288 131 against 118 us).
+template <int T, bool FUSED>
+__device__ __forceinline__ void epilogue_tile(const TsParams& p, uint32_t d_col, int m0, int n,
+                                              int lane, int c0, int cs) {
+    const bool n_ok =
+        n < p.N && dbg_check(m0 >= 0 && ((p.N & 1) != 0 || (n | 1) < p.N), p.status);
+    const float bias =
+        FUSED && p.epi.bias != nullptr && n_ok ? bf16_to_f32(p.epi.bias[n]) : 0.0f;
 #pragma unroll 1
     for (int c = c0; c < T / 32; c += cs) {
-        uint32_t v[32];
-        tmem_ld_32x32b_x32(d_col + c * 32, v);
-        tmem_ld_wait(v);
-        const int mbase = m0 + c * 32;
-        if (e.act == kActSwiGLU) {
-            const int col = n >> 1;
-            float r[16];
-#pragma unroll
-            for (int j = 0; j < 16; ++j) {
-                const int m = mbase + 2 * j + (odd ? 1 : 0);
-                r[j] = (has_res && m < p.M && n_ok)
-                           ? bf16_to_f32(e.residual[static_cast<int64_t>(m) * e.n_out + col])
-                           : 0.0f;
-            }
-#pragma unroll
-            for (int j = 0; j < 16; ++j) {
-                const float z0 = __uint_as_float(v[2 * j]) + b;
-                const float z1 = __uint_as_float(v[2 * j + 1]) + b;
-                const float other = __shfl_xor_sync(0xffffffffu, odd ? z0 : z1, 1);
-                const int m = mbase + 2 * j + (odd ? 1 : 0);
-                const float h = (odd ? silu_f32(other) * z1 : silu_f32(z0) * other) + r[j];
-                if (m < p.M && n_ok) p.out[static_cast<int64_t>(m) * e.n_out + col] = f32_to_bf16_rn(h);
-            }
-        } else if ((e.n_out & 1) == 0) {
-            // even lane: token 2j, columns (n, n+1); odd lane: token 2j+1, (n-1, n)
-            const int col = odd ? n - 1 : n;
-            uint32_t rw[16];
-#pragma unroll
-            for (int j = 0; j < 16; ++j) {
-                const int m = mbase + 2 * j + (odd ? 1 : 0);
-                rw[j] = (has_res && m < p.M && n_ok)
-                            ? *reinterpret_cast<const uint32_t*>(
-                                  e.residual + static_cast<int64_t>(m) * e.n_out + col)
-                            : 0u;
-            }
-#pragma unroll
-            for (int j = 0; j < 16; ++j) {
-                float h0 = __uint_as_float(v[2 * j]) + b, h1 = __uint_as_float(v[2 * j + 1]) + b;
-                if (e.act == kActGELU) {
-                    h0 = gelu_f32(h0);
-                    h1 = gelu_f32(h1);
-                }
-                const float other = __shfl_xor_sync(0xffffffffu, odd ? h0 : h1, 1);
-                const int m = mbase + 2 * j + (odd ? 1 : 0);
-                // (lo, hi) = outputs (col, col + 1) of token m
-                float lo = odd ? other : h0, hi = odd ? h1 : other;
-                lo += __uint_as_float(rw[j] << 16);
-                hi += __uint_as_float(rw[j] & 0xFFFF0000u);
-                if (m < p.M && n_ok)
-                    *reinterpret_cast<uint32_t*>(p.out + static_cast<int64_t>(m) * e.n_out + col) =
-                        pack_bf16x2(lo, hi);
-            }
-        } else {
-            float r[32];
-#pragma unroll
-            for (int j = 0; j < 32; ++j) {
-                const int m = mbase + j;
-                r[j] = (has_res && m < p.M && n_ok)
-                           ? bf16_to_f32(e.residual[static_cast<int64_t>(m) * e.n_out + n])
-                           : 0.0f;
-            }
-#pragma unroll
-            for (int j = 0; j < 32; ++j) {
-                const int m = mbase + j;
-                const float z = __uint_as_float(v[j]) + b;
-                const float h = (e.act == kActGELU ? gelu_f32(z) : z) + r[j];
-                if (m < p.M && n_ok) p.out[static_cast<int64_t>(m) * e.n_out + n] = f32_to_bf16_rn(h);
-            }
-        }
-    }
-}
-
-// Plain epilogue of one tile: bf16 stores of the accumulators; for even N
-// neighbouring lanes pair up so that each store writes two adjacent outputs
-// (n, n+1) of one token as a 32-bit word.
-template <int T>
-__device__ __forceinline__ void plain_epilogue_tile(const TsParams& p, uint32_t d_col, int m0,
-                                                    int n, int lane, bool n_even, int c0, int cs) {
+        if constexpr (FUSED) {
 #pragma unroll 1
-    for (int c = c0; c < T / 32; c += cs) {
-        uint32_t v[32];
-        tmem_ld_32x32b_x32(d_col + c * 32, v);
-        tmem_ld_wait(v);
-        const int mbase = m0 + c * 32;
-        if (n_even) {
-            // Pair neighbouring lanes so that each store writes two
-            // adjacent outputs (n, n+1) of one token as a 32-bit word.
+            for (int h = 0; h < 2; ++h) {
+                uint32_t d[16];
+                float v[16];
+                tmem_ld_32x32b_x16(d_col + c * 32 + h * 16, d);
+                tmem_ld_wait_x16(d);
 #pragma unroll
-            for (int j = 0; j < 16; ++j) {
-                const float f0 = __uint_as_float(v[2 * j]);
-                const float f1 = __uint_as_float(v[2 * j + 1]);
-                const float send = (lane & 1) ? f0 : f1;
-                const float other = __shfl_xor_sync(0xffffffffu, send, 1);
-                int m, col;
-                uint32_t word;
-                if ((lane & 1) == 0) {
-                    m = mbase + 2 * j;
-                    col = n;
-                    word = pack_bf16x2(f0, other);
-                } else {
-                    m = mbase + 2 * j + 1;
-                    col = n - 1;
-                    word = pack_bf16x2(other, f1);
-                }
-                if (m < p.M && col < p.N &&
-                    dbg_check((col & 1) == 0 && col + 1 < p.N && m >= 0 && col >= 0, p.status))
-                    *reinterpret_cast<uint32_t*>(p.out + static_cast<int64_t>(m) * p.N +
-                                                 col) = word;
+                for (int j = 0; j < 16; ++j) v[j] = __uint_as_float(d[j]);
+                store_tokens<true, 16>(p.epi, p.out, v, m0 + c * 32 + h * 16, p.M, n, n_ok, bias,
+                                       lane);
             }
         } else {
+            uint32_t d[32];
+            float v[32];
+            tmem_ld_32x32b_x32(d_col + c * 32, d);
+            tmem_ld_wait(d);
 #pragma unroll
-            for (int j = 0; j < 32; ++j) {
-                const int m = mbase + j;
-                if (m < p.M && n < p.N) {
-                    const uint32_t word = pack_bf16x2(__uint_as_float(v[j]), 0.0f);
-                    p.out[static_cast<int64_t>(m) * p.N + n] =
-                        static_cast<uint16_t>(word & 0xFFFFu);
-                }
-            }
+            for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(d[j]);
+            store_tokens<false, 32>(p.epi, p.out, v, m0 + c * 32, p.M, n, n_ok, 0.0f, lane);
         }
     }
 }
@@ -594,7 +489,6 @@ __global__ void __launch_bounds__(threads_for<DQ, EP>(), MIN_BLOCKS)
         const int sub = warp & 3;
         const int eg = (warp - (2 + 4 * DQ)) >> 2;
         const uint32_t lane_base = tmem + (static_cast<uint32_t>(sub * 32) << 16);
-        const bool n_even = (p.N & 1) == 0;
         uint32_t tcount = 0;
         for (int unit = unit_first<CW>(); unit < unit_count<CW>(p); unit += unit_stride<CW>(), ++tcount) {
             int tt, wt;
@@ -603,10 +497,7 @@ __global__ void __launch_bounds__(threads_for<DQ, EP>(), MIN_BLOCKS)
                 break;
             tc_fence_after();
             const int n = wt * kRows + sub * 32 + lane;
-            if constexpr (FUSED)
-                fused_epilogue_tile<T>(p, lane_base + L::D_COL, tt * T, n, lane, eg, EP);
-            else
-                plain_epilogue_tile<T>(p, lane_base + L::D_COL, tt * T, n, lane, n_even, eg, EP);
+            epilogue_tile<T, FUSED>(p, lane_base + L::D_COL, tt * T, n, lane, eg, EP);
             tc_fence_before();
             __syncwarp();
             if (lane == 0) {
@@ -652,15 +543,12 @@ __global__ void __launch_bounds__(threads_for<DQ, EP>(), MIN_BLOCKS)
     }
 }
 
-template <int T, int S_SMEM, int S_TMEM, int DQ, int EP, int MIN_BLOCKS, bool PAIR, int NB = 1>
-cudaError_t launch_variant(const CUtensorMap* tx, const CUtensorMap* tw, const TsParams& p,
-                           int grid, cudaStream_t stream) {
+template <int T, int S_SMEM, int S_TMEM, int DQ, int MIN_BLOCKS, bool FUSED, bool PAIR, int NB>
+cudaError_t launch_epilogue(const CUtensorMap* tx, const CUtensorMap* tw, const TsParams& p,
+                            int grid, cudaStream_t stream) {
     using L = Layout<T, S_SMEM, S_TMEM, PAIR, NB>;
-    // the plain variant carries none of the fused epilogue's code or registers
-    const bool fused =
-        p.epi.bias != nullptr || p.epi.residual != nullptr || p.epi.act != kActNone;
-    auto kern = fused ? w4a16_ts_kernel<T, S_SMEM, S_TMEM, DQ, EP, MIN_BLOCKS, true, PAIR, NB>
-                      : w4a16_ts_kernel<T, S_SMEM, S_TMEM, DQ, EP, MIN_BLOCKS, false, PAIR, NB>;
+    constexpr int EP = FUSED ? kFusedEP : kPlainEP;
+    auto kern = w4a16_ts_kernel<T, S_SMEM, S_TMEM, DQ, EP, MIN_BLOCKS, FUSED, PAIR, NB>;
     // Idempotent; cheap enough to repeat per launch and per device.
     cudaError_t e =
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, L::SMEM_BYTES);
@@ -686,6 +574,17 @@ cudaError_t launch_variant(const CUtensorMap* tx, const CUtensorMap* tw, const T
     return cudaGetLastError();
 }
 
+template <int T, int S_SMEM, int S_TMEM, int DQ, int MIN_BLOCKS, bool PAIR, int NB = 1>
+cudaError_t launch_variant(const CUtensorMap* tx, const CUtensorMap* tw, const TsParams& p,
+                           int grid, cudaStream_t stream) {
+    // the plain variant carries none of the fused epilogue's code or registers
+    if (p.epi.bias != nullptr || p.epi.residual != nullptr || p.epi.act != kActNone)
+        return launch_epilogue<T, S_SMEM, S_TMEM, DQ, MIN_BLOCKS, true, PAIR, NB>(tx, tw, p, grid,
+                                                                                stream);
+    return launch_epilogue<T, S_SMEM, S_TMEM, DQ, MIN_BLOCKS, false, PAIR, NB>(tx, tw, p, grid,
+                                                                             stream);
+}
+
 // Large M: 256 tokens per tile, 6 stages of (32 KB x + 4 KB packed weights),
 // tensor memory = 256 accumulator columns + 6 x 32 A columns.
 #ifndef W4A16_GEMM_DQ
@@ -694,11 +593,7 @@ cudaError_t launch_variant(const CUtensorMap* tx, const CUtensorMap* tw, const T
 #ifndef W4A16_GEMM_SS
 #define W4A16_GEMM_SS 6
 #endif
-#ifndef W4A16_GEMM_EP
-#define W4A16_GEMM_EP 2
-#endif
-constexpr int kGemmT = 256, kGemmSS = W4A16_GEMM_SS, kGemmST = 6, kGemmDQ = W4A16_GEMM_DQ,
-              kGemmEP = W4A16_GEMM_EP;
+constexpr int kGemmT = 256, kGemmSS = W4A16_GEMM_SS, kGemmST = 6, kGemmDQ = W4A16_GEMM_DQ;
 // CTA pairs: 256 tokens per tile, each CTA a ring of 8 stages of (16 KB x +
 // 4 KB packed weights) and 8 tensor-memory A stages: 256 accumulator + 8 x 32
 // A columns fill the 512 columns.
@@ -722,7 +617,7 @@ int pair_slots(int sm_count) {
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDev) return sm_count / 2;
     if (cache[dev] > 0) return cache[dev];
     using L = Layout<kGemmT, kPairSS, kPairST, true>;
-    auto kern = w4a16_ts_kernel<kGemmT, kPairSS, kPairST, kGemmDQ, kGemmEP, 1, false, true, 1>;
+    auto kern = w4a16_ts_kernel<kGemmT, kPairSS, kPairST, kGemmDQ, kPlainEP, 1, false, true, 1>;
     int n = 0;
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, L::SMEM_BYTES) ==
         cudaSuccess) {
@@ -733,7 +628,7 @@ int pair_slots(int sm_count) {
         attr[0].val.clusterDim.y = 1;
         attr[0].val.clusterDim.z = 1;
         cfg.gridDim = dim3(static_cast<unsigned>(sm_count / 2 * 2));
-        cfg.blockDim = dim3(threads_for<kGemmDQ, kGemmEP>());
+        cfg.blockDim = dim3(threads_for<kGemmDQ, kPlainEP>());
         cfg.dynamicSmemBytes = L::SMEM_BYTES;
         cfg.attrs = attr;
         cfg.numAttrs = 1;
@@ -791,13 +686,10 @@ int ts_grid(TsVariant v, const TsParams& p, int sm_count) {
 cudaError_t ts_launch(TsVariant v, const CUtensorMap* tx, const CUtensorMap* tw,
                       const TsParams& p, int grid, cudaStream_t stream) {
     if (v == TsVariant::kGemm256)
-        return launch_variant<kGemmT, kGemmSS, kGemmST, kGemmDQ, kGemmEP, 1, false>(tx, tw, p,
-                                                                                   grid, stream);
+        return launch_variant<kGemmT, kGemmSS, kGemmST, kGemmDQ, 1, false>(tx, tw, p, grid, stream);
     if (v == TsVariant::kGemmPair)
-        return launch_variant<kGemmT, kPairSS, kPairST, kGemmDQ, kGemmEP, 1, true>(tx, tw, p,
-                                                                                  grid, stream);
-    return launch_variant<kWideT, kWideSS, kWideST, kGemmDQ, kGemmEP, 1, true, 2>(tx, tw, p, grid,
-                                                                                 stream);
+        return launch_variant<kGemmT, kPairSS, kPairST, kGemmDQ, 1, true>(tx, tw, p, grid, stream);
+    return launch_variant<kWideT, kWideSS, kWideST, kGemmDQ, 1, true, 2>(tx, tw, p, grid, stream);
 }
 
 }  // namespace w4a16
