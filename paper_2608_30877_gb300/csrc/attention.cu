@@ -30,15 +30,23 @@
 // mbarriers whose phases run on across jobs: Q and K of the next job load during the
 // current job's last blocks, and its first S products run during the epilogue.
 //
-// What bounds it (96 heads, us; before and after the job order below, the job ring and
-// the streaming hints): 64 ragged pairs of 200 to 1024 tokens 1105 -> 976, 64 x 1024
-// tokens 2110 -> 1713, 10007 tokens under a window of 4096 1390 -> 1278 (62% of the
-// bf16 peak).  DRAM traffic was the limit of the short sequences (76% of its
-// rate, 6.4 GB for 3.8 GB of input and output) and is now 4.6 GB; then the latency of
-// the softmax -> PV -> S chain of two CTAs per SM, no unit being busy half the time.
+// What bounds it (96 heads, us; before and after the job order below, the job ring,
+// the streaming hints and the order of the issuers' waits): 64 ragged pairs of 200 to
+// 1024 tokens 1105 -> 973, 64 x 1024 tokens 2110 -> 1684, 10007 tokens under a window of
+// 4096 1390 -> 1247 (64% of the bf16 peak).  DRAM traffic was the limit of the short
+// sequences (76% of its rate, 6.4 GB for 3.8 GB of input and output) and is now 4.6 GB.
+// In the steady state a block takes ~1560 clocks per CTA: 8 MMAs of S (N = 64, whose 6 KB
+// of operands from shared memory take longer than their math) and 4 of PV of each of the
+// two CTAs fill most of them, and the chain of a block is softmax 1050, P to the PV issuer
+// 210, PV 600, its completion to the S issuer 280, S 1100.  With parts left out the last
+// two shapes fall to 1587 and 1164 us without the softmax's arithmetic, 1533 and 1081 with
+// half the MMAs, 1666 and 1263 without loads of K and V, so no one of them bounds it alone.
 // Measured and not kept: P in columns of its own, so that S only waits for the scores to
 // be read (1035 / 1287 / 1800); exponentials taken with the old max ahead of the
-// block's (1059 / 1389 / 1884); the next output chunk read during the stores (1026).
+// block's (1059 / 1389 / 1884); the next output chunk read during the stores (1026); S and
+// PV issued in turn by one warp, S right behind the PV product before it (1085 / 1333 /
+// 1848); blocks of 128 keys, their S one product of N = 128 (1142 / 1510 / 2035); the
+// search for a job during the loads of the one before (970 / 1254 / 1682).
 // Every wait is bounded (ptx.cuh); on a timeout the kernel records
 // W4A16_ERR_TIMEOUT, waits for its own copies and MMAs and frees tensor memory.
 #include "internal.h"
@@ -110,17 +118,6 @@ __device__ __forceinline__ uint64_t sdesc_mnmajor_sw128(uint32_t saddr, uint32_t
     d |= static_cast<uint64_t>(1) << 46;
     d |= static_cast<uint64_t>(2) << 61;
     return d;
-}
-
-// 32 lanes x 16 columns of 32 bits (see tmem_st_32x32b_x32).
-__device__ __forceinline__ void tmem_st_32x32b_x16(uint32_t taddr, const uint32_t (&v)[16]) {
-    asm volatile(
-        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], "
-        "{%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16};" ::"r"(taddr),
-        "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]),
-        "r"(v[8]), "r"(v[9]), "r"(v[10]), "r"(v[11]), "r"(v[12]), "r"(v[13]), "r"(v[14]),
-        "r"(v[15])
-        : "memory");
 }
 
 // 16-lane tensor-memory shapes (the warp covers 16 lanes from the address's
@@ -497,11 +494,14 @@ __global__ void __launch_bounds__(kThreads, 2)
             if (nblk == 0) break;
             for (int j = 0; j < nblk; ++j, ++gs) {
                 const uint32_t b = gs & 1u;
-                // the buffer's previous block (gs - 2) has had its PV product
-                ok = gs < 2 ||
-                     wait_warp(o_ready(b), ((gs - 2) >> 1) & 1u, abort_flag, p.status, p.wait_ns);
-                if (ok && j == 0) ok = wait_warp(q_full, jn & 1u, abort_flag, p.status, p.wait_ns);
-                if (ok) ok = wait_warp(k_full(b), (gs >> 1) & 1u, abort_flag, p.status, p.wait_ns);
+                ok = (j > 0 || wait_warp(q_full, jn & 1u, abort_flag, p.status, p.wait_ns)) &&
+                     wait_warp(k_full(b), (gs >> 1) & 1u, abort_flag, p.status, p.wait_ns);
+                // last, because it comes last (a poll that succeeds takes ~150 clocks,
+                // here and for PV; with these two orders turned round 983 -> 973 us,
+                // 1287 -> 1247, 1716 -> 1684): the buffer's previous block (gs - 2) has
+                // had its PV product
+                if (ok && gs >= 2)
+                    ok = wait_warp(o_ready(b), ((gs - 2) >> 1) & 1u, abort_flag, p.status, p.wait_ns);
                 if (!ok) break;
                 tc_fence_after();
                 const uint64_t qd = sdesc_kmajor_sw128(sbase + L::Q_OFF);
@@ -538,8 +538,8 @@ __global__ void __launch_bounds__(kThreads, 2)
                 const uint32_t b = g & 1u;
                 // O += P V once the softmax warps have written P of block g (for
                 // a job's first block, after they read out the previous job's O)
-                ok = wait_warp(p_full(b), (g >> 1) & 1u, abort_flag, p.status, p.wait_ns) &&
-                     wait_warp(v_full(b), (g >> 1) & 1u, abort_flag, p.status, p.wait_ns);
+                ok = wait_warp(v_full(b), (g >> 1) & 1u, abort_flag, p.status, p.wait_ns) &&
+                     wait_warp(p_full(b), (g >> 1) & 1u, abort_flag, p.status, p.wait_ns);
                 if (!ok) break;
                 tc_fence_after();
                 const uint64_t vd =
