@@ -292,12 +292,13 @@ int launch_linear(const DeviceState& st, const void* x, const void* w, const voi
         return launch_head(x, w, p, st.sm_count, stream) == cudaSuccess ? W4A16_OK : W4A16_ERR_CUDA;
     }
     // Up to 128 tokens the weights stream once per call on the streaming kernels
-    // (12288 x 49152: M = 64 81 us there against 212 on the 256-token GEMM tiles,
-    // M = 128 112 against 214).  M <= 16: the warp-level kernel has the higher rate
-    // where every SM has many rows (M = 8: N = 49152 65 us against 73, 36864 53
-    // against 61), the tcgen05 one on narrow layers, whose K it splits (24576 47
-    // against 39, 12288 34 against 24, K = 49152 126 against 73) and from 9 tokens
-    // on (M = 16: N = 49152 81 against 74, 36864 65 against 61).
+    // (12288 x 49152: M = 64 78 us there against 212 on the 256-token GEMM tiles,
+    // M = 128 104 against 214).  M <= 16: the warp-level kernel has the higher rate
+    // between about 25000 and 36000 rows (M = 8: N = 30000 49.7 us against 51.4; 36864
+    // 52.3 against 52.5) and on the shortest K; the tcgen05 one elsewhere (49152 65.8
+    // against 63.2, 60000 124 against 99, and, its K split, 24576 46 against 37, 12288
+    // 35 against 23, K = 49152 132 against 66) and from 9 tokens on (M = 16: N = 30000
+    // 61 against 51, 49152 82 against 63).
     if (M <= 128) {
         const GemvTcPlan plan = gemv_tc_plan(M, N, K, st.sm_count);
         const bool rows = M <= 16 && g == 128 &&

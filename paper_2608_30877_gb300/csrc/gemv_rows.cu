@@ -1,8 +1,8 @@
 // Small-M (M <= 16, g = 128) int4-dequant + matmul for sm_103a: the bandwidth-bound
 // regime where the whole packed weight matrix streams from HBM once per call, for
-// layers with enough rows to give every SM some 180 and more (below that, and from 9
-// tokens on where the rows are many, gemv_tc.cu's split of K over clusters is faster;
-// gemv_cost_us).
+// layers with enough rows to give every SM some 165 to 235 (with fewer, gemv_tc.cu's
+// split of K over clusters is faster, with more, its three tiles; from 9 tokens on it nearly
+// always is) and for the shortest K; the dispatch compares gemv_cost_us with its plan's.
 //
 // Design, GB300-first:
 //   - persistent grid, one CTA per SM; CTA c owns a contiguous range of RB

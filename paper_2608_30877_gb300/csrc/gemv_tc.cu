@@ -1,5 +1,5 @@
 // Streaming int4-dequant + matmul on the 5th-generation tensor core for few
-// tokens (M = 17..128, every group size, and more tokens in 128-token tiles
+// tokens (M <= 128, every group size, and more tokens in 128-token tiles
 // where the GEMM's CTA pairs would leave SMs idle): the regime where the whole
 // packed weight matrix streams from HBM about once per call.
 //
@@ -34,17 +34,23 @@
 // 56 -> 24 us.
 //
 // What bounds it (K = 12288, 152 SMs): the row warps' latency and issue slots, not the
-// tensor pipe: a stage costs 0.45-0.48, 0.60-0.73, 0.73-1.13 us for one, two, three
-// tiles (N = 49152: 74 us at M <= 32, 81 at 64, 88 at 90, 106 at 100, 112 at 128;
-// before this kernel dequantised in k order, through one FMA, with no x reorder warp,
-// operands in uniform registers and addresses that only advance: 92, 103, 137, 137,
-// 139).  tcgen05.mma with A in tensor memory runs at 18 / 32 / 64 clocks for 32 / 64 /
+// tensor pipe: a stage costs 0.39-0.50, 0.51-0.71, 0.62-1.05 us for one, two, three
+// tiles (N = 49152: 63 us at M <= 32, 78 at 64, 84 at 96, 103 at 112, 104 at 128).  In order,
+// what brought it there from 92, 103, 137, 137 and 139: weights dequantised in k order,
+// with no x reorder warp, through one FMA, operands in uniform registers, addresses that
+// only advance (72, 80, 86, -, 110); then, from stamps of a row warp, whose 1540 clocks
+// per stage were two barrier polls of 190-230 that found their barriers long complete,
+// 310 to read the codes and dequantise half, 340 for the other half, 110 for the stores and 360
+// of scales and votes: the two polls under way together, and the next stage's scales
+// prepared during the stores where a stage is one A stage (in more, smaller A stages that
+// is slower: 64 tokens 82 against 79 us).
+// tcgen05.mma with A in tensor memory runs at 18 / 32 / 64 clocks for 32 / 64 /
 // 128 columns with three independent accumulators, 44 with one (measured alone), so
 // the MMAs need 0.22-0.8 us of a stage.  From 97 tokens on three tiles leave the A ring
-// only two or three slots of a quarter stage.  Measured and not kept: two groups of row
-// warps per tile (M = 24: 99 us: the A ring is too short for them), barrier polls
-// issued ahead of the dequantisation (81), one issuing warp for all tiles (92), a
-// rolled dequant loop (78).
+// only two or three slots of a quarter stage.  Measured and not kept (M <= 32): two groups
+// of row warps per tile (99 us: the A ring is too short for them), the next stage's codes
+// read before this one's stores end (71) or after (66), one issuing warp for all tiles
+// (92), a rolled dequant loop (78), 16 token columns for M <= 16 (67).
 //
 // Every wait is bounded (ptx.cuh); on a timeout the kernel records
 // W4A16_ERR_TIMEOUT, drains its copies and MMAs, frees tensor memory and
@@ -383,10 +389,14 @@ __global__ void __launch_bounds__(TLayout<NTOK, TILES>::THREADS, 1)
                 }
                 if (++kk == k_end) kk = k_first;
             };
-            load_scales();
-            for (int left = k_count; left > 0; --left) {
-                uint32_t s2_lo = splat_bf16(n_lo), s2_hi = s2_lo;
-                ScaleFma f_lo = scale_fma(s2_lo), f_hi = f_lo;
+            // the scales of the next stage to dequantise, and the load for the one after:
+            // with one A stage per stage, while its last stores are under way
+            uint32_t s2_lo = 0, s2_hi = 0;
+            ScaleFma f_lo{}, f_hi{};
+            bool wide = false;
+            auto next_scales = [&]() {
+                s2_lo = s2_hi = splat_bf16(n_lo);
+                f_lo = f_hi = scale_fma(s2_lo);
                 bool w_scale = scale_is_wide(n_lo);
                 if (upg != 2) {
                     s2_hi = splat_bf16(n_hi);
@@ -394,11 +404,18 @@ __global__ void __launch_bounds__(TLayout<NTOK, TILES>::THREADS, 1)
                     w_scale = w_scale || scale_is_wide(n_hi);
                 }
                 load_scales();
-                const bool wide = __any_sync(0xffffffffu, w_scale);
-                if (!wait_warp(full_at, ph, abort_flag, p.status, p.wait_ns)) {
+                wide = __any_sync(0xffffffffu, w_scale);
+            };
+            load_scales();
+            if (SUB == 1) next_scales();
+            for (int left = k_count; left > 0; --left) {
+                if (SUB > 1) next_scales();
+                // the stage has landed, and the previous MMAs of its first A slot are done
+                if (!wait_warp2(full_at, ph, empty_at, pa, abort_flag, p.status, p.wait_ns)) {
                     ok = false;
                     break;
                 }
+                tc_fence_after();
 #pragma unroll
                 for (int h = 0; h < SUB; ++h) {
                     uint4 c[L::CHUNKS];
@@ -431,7 +448,7 @@ __global__ void __launch_bounds__(TLayout<NTOK, TILES>::THREADS, 1)
                                 dequant_word(c[i + q].w, s2, v + 16 * q + 12);
                             }
                         }
-                        if (i == 0) {
+                        if (h > 0 && i == 0) {
                             // the slot's previous MMAs are done
                             if (!wait_warp(empty_at, pa, abort_flag, p.status, p.wait_ns)) {
                                 ok = false;
@@ -447,6 +464,7 @@ __global__ void __launch_bounds__(TLayout<NTOK, TILES>::THREADS, 1)
                         }
                     }
                     if (!ok) break;
+                    if (SUB == 1 && h == SUB - 1) next_scales();
                     tmem_st_wait();
                     tc_fence_before();
                     __syncwarp();
@@ -627,11 +645,12 @@ int cluster_slots(int split, int sm_count) {
 
 GemvTcPlan gemv_tc_plan(int64_t M, int64_t N, int64_t K, int sm_count) {
     // us per 128-k stage of a CTA that holds 1, 2 or 3 tiles of 128 rows, by token
-    // columns 32, 64, 96, 112, 128 (K = 12288, N = 36864 and 49152, less 4 us: 60.6 / 62.2
-    // / 66.5 / 69.9 / 74.6 and 74.4 / 80.6 / 88.1 / 106.4 / 111.8 us in all)
-    static constexpr double kStageUs[3][5] = {{0.45, 0.45, 0.46, 0.47, 0.48},
-                                              {0.60, 0.61, 0.65, 0.69, 0.73},
-                                              {0.73, 0.80, 0.88, 1.07, 1.13}};
+    // columns 32, 64, 96, 112, 128 (K = 12288, N = 19000 without a split, 36864 and 49152,
+    // less 4 us: 41.4 / 45.4 / 46.6 / 48.0 / 52.3, 52.6 / 58.3 / 64 / 67.3 / 72.5 and
+    // 63.2 / 78.2 / 83.6 / 103.3 / 104.2 us in all)
+    static constexpr double kStageUs[3][5] = {{0.39, 0.43, 0.44, 0.46, 0.50},
+                                              {0.51, 0.57, 0.63, 0.66, 0.71},
+                                              {0.62, 0.77, 0.83, 1.03, 1.05}};
     GemvTcPlan best{};
     // equal tiles of at most 128 tokens
     const int64_t tok_tiles = (M + 127) / 128;

@@ -211,6 +211,16 @@ __device__ __forceinline__ bool wait_warp(uint32_t bar, uint32_t parity, volatil
     }
 }
 
+// Wait by a whole warp for two barriers, their polls under way together.
+__device__ __forceinline__ bool wait_warp2(uint32_t bar0, uint32_t parity0, uint32_t bar1,
+                                           uint32_t parity1, volatile int* abort_flag, int* status,
+                                           uint64_t limit_ns) {
+    const bool d0 = mbar_try_wait<false>(bar0, parity0), d1 = mbar_try_wait<false>(bar1, parity1);
+    if (__all_sync(0xffffffffu, d0 && d1)) return true;
+    return wait_warp(bar0, parity0, abort_flag, status, limit_ns) &&
+           wait_warp(bar1, parity1, abort_flag, status, limit_ns);
+}
+
 // Bounded wait used by the drains before exit: gives up silently after
 // kWaitLimitNs (the copy or MMA it waits for was issued by this CTA and
 // completes on its own).
