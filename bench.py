@@ -41,27 +41,25 @@ NCU_TRAFFIC = {
     # mean of one launch per stack shape at M = 16384 (384-token tiles, as in
     # the benched stack), scaled by 4 to M = 65536
     # (profiles/gemm_pair_wide_stack_traffic_m16384.md)
-    ("stack", "ts", "cc26b2d7ce6a2d19"): 7.1208e9 * 4,
+    ("stack", "ts", "18c5e9d80b49e365"): 7.1588e9 * 4,
     # QKV prefill 4096x12288x36864 (384-token CTA pairs), one launch
     # (profiles/gemm_pair_wide_qkv_prefill_4096x12288x36864.md)
-    ("qkv", "ts", "cc26b2d7ce6a2d19"): 1.4663e9 + 0.2894e9,
+    ("qkv", "ts", "18c5e9d80b49e365"): 1.4829e9 + 0.2914e9,
     # MLP up / down at 8192 tokens (384-token CTA pairs), one launch each
     # (DRAM counters only; profiles/gemm_pair_mlp_traffic_8192.md)
-    ("mlp_up", "ts", "cc26b2d7ce6a2d19"): 3.9122e9 + 0.8025e9,
-    ("mlp_down", "ts", "cc26b2d7ce6a2d19"): 4.7823e9 + 0.1976e9,
-    # small-M readout, M = 8 (warp-level kernel), 12288x49152, one launch
-    ("gemv", "gemv", "270f49f687deb1b3"): 0.31859e9 + 0.00380e9,
-    # the same at M = 16 (16 token columns), one launch (DRAM counters only)
-    ("gemv16", "gemv", "270f49f687deb1b3"): 0.31808e9 + 0.00319e9,
-    # small-M readout, M = 32 (tensor-core kernel), 12288x49152, one launch
-    ("gemv32", "gemvtc", "b81ddd27f1e19156"): 0.32655e9 + 0.00362e9,
+    ("mlp_up", "ts", "18c5e9d80b49e365"): 3.9608e9 + 0.8024e9,
+    ("mlp_down", "ts", "18c5e9d80b49e365"): 4.7825e9 + 0.1976e9,
+    # small-M readout, M = 8 and M = 32 (tensor-core streaming kernel, 32 token
+    # columns), 12288x49152, one launch each (profiles/gemv_tc_m32_12288x49152.md)
+    ("gemv", "gemv", "2e8e502e20039969"): 0.32525e9 + 0.00332e9,
+    ("gemv32", "gemvtc", "2e8e502e20039969"): 0.32657e9 + 0.00318e9,
     # attention prefill per 8 pairs of 1024 tokens x 96 heads (full capture of
     # one 8-pair launch); scaled by pairs / 8 for the benched launch
-    ("attention", "attn", "f94e5ad5312cd435"): 0.8716e9 + 0.1923e9,
+    ("attention", "attn", "2c879819e8d835be"): 0.6046e9 + 0.1739e9,
 }
 
 KERNEL_FILES = {"ts": ("ts_gemm.cu", "dequant.cuh", "ptx.cuh"),
-                "gemv": ("gemv_rows.cu", "dequant.cuh", "ptx.cuh"),
+                "gemv": ("gemv_tc.cu", "dequant.cuh", "ptx.cuh"),  # M <= 16 at this width
                 "gemvtc": ("gemv_tc.cu", "dequant.cuh", "ptx.cuh"),
                 "attn": ("attention.cu",)}
 
@@ -82,9 +80,9 @@ def ncu_traffic(config: str, m: int, pairs: int = 8):
         t = NCU_TRAFFIC.get((config, "attn", kernel_source_hash("attn")))
         return None if t is None else t * pairs / 8  # qkv and out grow with the pairs
     if config == "gemv":
-        if 17 <= m <= 32:  # the tensor-core kernel; the capture is of M = 32
+        if 17 <= m <= 32:  # the capture is of M = 32
             return NCU_TRAFFIC.get(("gemv32", "gemvtc", kernel_source_hash("gemvtc")))
-        if m > 8:  # the M = 9..16 instantiation, captured at M = 16
+        if m > 8:  # no capture of M = 9..16
             return NCU_TRAFFIC.get(("gemv16", "gemv", kernel_source_hash("gemv")))
         kind = "gemv"
     else:

@@ -81,7 +81,8 @@ typedef enum {
  * Dispatch, by modelled time (csrc/api.cu): the fused dequant + tcgen05 GEMM for
  * large M; a tcgen05 kernel that streams the weights for M <= 128 and for larger
  * M where the GEMM's tiles would leave SMs idle (few weight rows); a warp-level
- * streaming kernel for M <= 16, g = 128 and many rows.  The tcgen05 kernels multiply
+ * streaming kernel for M <= 16, g = 128 where it is faster; for N <= 8 a kernel that
+ * splits the tokens over the GPU.  All but the warp-level one multiply
  * x by the dequantised weights wd defined above, so they differ from each other
  * only in the fp32 summation order.  The warp-level streaming kernel factors
  * the scale out of each group instead: it sums x * (code - 8) over the group
@@ -259,7 +260,7 @@ int w4a16_gather_rows(const void* src_bf16, int64_t src_rows, int64_t D,
  *                  1 <= n < 2^31; other score_bits: W4A16_ERR_INVALID_ARG
  *   1 <= k <= n, k <= 1024 (larger k: W4A16_ERR_UNSUPPORTED)
  *   out_index_i32  [k] int32, out_score_f32 [k] fp32, device, disjoint
- * One launch of one 8-CTA thread-block cluster; no scratch memory.
+ * One launch of one thread-block cluster of 8 or 16 CTAs; no scratch memory.
  */
 int w4a16_topk_smallest(const void* scores, int score_bits, int64_t n, int64_t k,
                         void* out_index_i32, void* out_score_f32, void* stream);

@@ -81,7 +81,7 @@ cudaError_t gemv_launch(const CUtensorMap* tmap_x, const CUtensorMap* tmap_w,
 // of `tokens` rows x 64 k (128-byte swizzle), weight boxes of RB/2 rows x 64
 // bytes (64-byte swizzle).
 struct GemvTcPlan {
-    int tokens;        // token columns per tile: 32, 64 or 128
+    int tokens;        // token columns per tile: 32, 64, 96, 112 or 128
     int split;         // CTAs (one cluster) sharing a chunk, each a slice of K
     int rows_per_cta;  // RB
     int row_chunks;    // ceil(N / RB)
