@@ -309,8 +309,8 @@ int launch_linear(const DeviceState& st, const void* x, const void* w, const voi
     }
     // Beyond that too, in tiles of up to 128 tokens, where the GEMM's CTA pairs do
     // not fill the GPU (few weight rows, or a nearly empty last wave), by the two
-    // modelled times: 12288 x 12288 at M = 130 49 us against 69, 333 68 against 95,
-    // 512 108 against 136; at 1024 240 against 200, where the GEMM stays.
+    // modelled times: 12288 x 12288 at M = 130 47 us against 69, 333 66 against 95,
+    // 512 104 against 136; at 1024 240 against 190, where the GEMM stays.
     if (g_gemm_pair && g_gemm_wide_from < 0) {
         const GemvTcPlan plan = gemv_tc_plan(M, N, K, st.sm_count);
         if (plan.cost_us < 0.95 * ts_cost_us(M, N, K, st.sm_count))

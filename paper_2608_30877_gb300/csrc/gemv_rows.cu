@@ -168,6 +168,8 @@ __global__ void __launch_bounds__(kMaxThreads, 1)
         prefetch_tmap(&tmap_w);
     }
     __syncthreads();
+    grid_launch_dependents();
+    grid_wait();
 
     const int KS = p.K / kBKS;        // scale groups = real stages per chunk
     const int R = (KS + U - 1) / U;   // rounds per chunk
@@ -503,7 +505,18 @@ cudaError_t launch_gemv_variant(const CUtensorMap* tx, const CUtensorMap* tw,
     if (e != cudaSuccess) return e;
     const int threads =
         32 * (kFirstComputeWarp + (p.rows_per_cta + kRowsPerWarp - 1) / kRowsPerWarp);
-    kern<<<grid, threads, L::SMEM_BYTES, stream>>>(*tx, *tw, p);
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1];
+    cfg.gridDim = dim3(static_cast<unsigned>(grid));
+    cfg.blockDim = dim3(static_cast<unsigned>(threads));
+    cfg.dynamicSmemBytes = L::SMEM_BYTES;
+    cfg.stream = stream;
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // grid_wait
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    e = cudaLaunchKernelEx(&cfg, kern, *tx, *tw, p);
+    if (e != cudaSuccess) return e;
     return cudaGetLastError();
 }
 

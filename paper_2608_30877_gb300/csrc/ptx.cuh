@@ -28,6 +28,22 @@ __device__ __forceinline__ bool elect_one() {
     return p != 0;
 }
 
+// Programmatic launch: a kernel launched with cudaLaunchAttributeProgrammaticStream-
+// Serialization may start when every CTA of the one before it in the stream has called
+// grid_launch_dependents (or ended), and touches global memory only after grid_wait,
+// which returns once that one has completed and its writes are visible.  Its launch, barriers
+// and tensor memory are then under way as the SMs of the one before it fall idle: 0.5 us
+// of a streaming kernel (12288 x 12288, M = 8 23.3 -> 22.8 us; 2048 x 2048, M = 1 7.1 ->
+// 6.5; 36864 x 12288 with g = 64 after other work 66.0 -> 64.2).  A kernel calls
+// grid_launch_dependents before its own grid_wait: the next one waits for all of it.
+__device__ __forceinline__ void grid_launch_dependents() {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+__device__ __forceinline__ void grid_wait() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 // ---------------------------------------------------------------- mbarrier
 
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
