@@ -41,21 +41,21 @@ NCU_TRAFFIC = {
     # mean of one launch per stack shape at M = 16384 (384-token tiles, as in
     # the benched stack), scaled by 4 to M = 65536
     # (profiles/gemm_pair_wide_stack_traffic_m16384.md)
-    ("stack", "ts", "18c5e9d80b49e365"): 7.1588e9 * 4,
+    ("stack", "ts", "96e8156fb430b201"): 7.1506e9 * 4,
     # QKV prefill 4096x12288x36864 (384-token CTA pairs), one launch
     # (profiles/gemm_pair_wide_qkv_prefill_4096x12288x36864.md)
-    ("qkv", "ts", "18c5e9d80b49e365"): 1.4829e9 + 0.2914e9,
+    ("qkv", "ts", "96e8156fb430b201"): 1.4726e9 + 0.2892e9,
     # MLP up / down at 8192 tokens (384-token CTA pairs), one launch each
     # (DRAM counters only; profiles/gemm_pair_mlp_traffic_8192.md)
-    ("mlp_up", "ts", "18c5e9d80b49e365"): 3.9608e9 + 0.8024e9,
-    ("mlp_down", "ts", "18c5e9d80b49e365"): 4.7825e9 + 0.1976e9,
+    ("mlp_up", "ts", "96e8156fb430b201"): 3.9457e9 + 0.8025e9,
+    ("mlp_down", "ts", "96e8156fb430b201"): 4.7834e9 + 0.1975e9,
     # small-M readout, M = 8 and M = 32 (tensor-core streaming kernel, 32 token
     # columns), 12288x49152, one launch each (profiles/gemv_tc_m32_12288x49152.md)
-    ("gemv", "gemv", "2e8e502e20039969"): 0.32525e9 + 0.00332e9,
-    ("gemv32", "gemvtc", "2e8e502e20039969"): 0.32657e9 + 0.00318e9,
+    ("gemv", "gemv", "7dfe2915b3327dfb"): 0.32543e9 + 0.00322e9,
+    ("gemv32", "gemvtc", "7dfe2915b3327dfb"): 0.32668e9 + 0.00322e9,
     # attention prefill per 8 pairs of 1024 tokens x 96 heads (full capture of
     # one 8-pair launch); scaled by pairs / 8 for the benched launch
-    ("attention", "attn", "2c879819e8d835be"): 0.6046e9 + 0.1739e9,
+    ("attention", "attn", "2c879819e8d835be"): 0.6044e9 + 0.1733e9,
 }
 
 KERNEL_FILES = {"ts": ("ts_gemm.cu", "dequant.cuh", "ptx.cuh"),
