@@ -216,7 +216,9 @@ int w4a16_quantize(const void* w_f32, void* w_packed_u8, void* scales_bf16,
  *   d              head dimension, 128 (else W4A16_ERR_UNSUPPORTED)
  *   out_bf16       [M, H*d] bf16, device, must not overlap the inputs
  * The softmax is computed in fp32 with P rounded to bf16 for the PV product
- * (tcgen05), O accumulated in fp32, one bf16 rounding at the store.
+ * (tcgen05), O accumulated in fp32, one bf16 rounding at the store.  Where a
+ * kernel gave up on a wait (W4A16_ERR_TIMEOUT), the sequences' rows that it did
+ * not finish are zero.
  */
 int w4a16_attention_prefill(const void* qkv_bf16, const void* seq_start_i32, int64_t nseq,
                             int64_t M, int64_t H, int64_t d, int64_t window, void* out_bf16,
@@ -292,8 +294,8 @@ int w4a16_get_device_error(void* stream);
  * W4A16_ERR_INVALID_ARG).  A test lowers it so that a real kernel's waits run
  * out and the kernel takes its abort path: it records W4A16_ERR_TIMEOUT,
  * waits for its own copies and MMAs in flight, frees its tensor memory and
- * returns, leaving its output incomplete.  Process-wide and not meant for
- * concurrent use with other launches.
+ * returns, leaving its output incomplete (attention's unfinished rows zero).
+ * Process-wide and not meant for concurrent use with other launches.
  */
 int w4a16_selftest_wait_timeout(int64_t limit_ns, void* stream);
 int w4a16_selftest_set_wait_limit(int64_t limit_ns);

@@ -85,7 +85,7 @@ struct AttnLayout {
     static constexpr int NBARS = 18 + kJobSlots;
     static constexpr int JOB_OFF = BAR_OFF + (NBARS * 8 + 15) / 16 * 16;
     static constexpr int MISC_OFF = JOB_OFF + kJobSlots * 32;
-    static constexpr int SMEM_BYTES = MISC_OFF + 32 + 1024;
+    static constexpr int SMEM_BYTES = MISC_OFF + 16 + 4 * kSoftmaxWarps + 1024;
     // tensor memory columns: two S buffers (blocks alternate; P of a block is
     // written over the first half of its S) and O
     static constexpr int S_COL = 0, O_COL = 2 * kBKV, TMEM_COLS = 256;
@@ -335,6 +335,7 @@ __global__ void __launch_bounds__(kThreads, 2)
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + L::MISC_OFF);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + L::MISC_OFF + 4);
     int* bad_flag = reinterpret_cast<int*>(smem + L::MISC_OFF + 8);
+    int* jobs_done = reinterpret_cast<int*>(smem + L::MISC_OFF + 16);  // per softmax warp
 
     if (warp == 0) {
         // the sequence boundaries must be non-decreasing within [0, M]
@@ -578,8 +579,8 @@ __global__ void __launch_bounds__(kThreads, 2)
         const uint32_t lane_base = tmem + (static_cast<uint32_t>(rb) << 16);
         const float cs = 1.4426950408889634f * p.scale;  // log2(e) / sqrt(d)
         bool ok = run;
-        uint32_t gb = 0;
-        for (uint32_t jn = 0; ok; ++jn) {
+        uint32_t gb = 0, jn = 0;
+        for (; ok; ++jn) {
             if (!wait_warp(job_full(jn), (jn / kJobSlots) & 1u, abort_flag, p.status, p.wait_ns)) {
                 ok = false;
                 break;
@@ -741,6 +742,7 @@ __global__ void __launch_bounds__(kThreads, 2)
                 __syncwarp();
             }
         }
+        if (lane == 0) jobs_done[sw] = static_cast<int>(jn);  // stored jobs
         // a softmax warp that gave up may have tensor-memory stores in flight
         tmem_st_wait();
     }
@@ -748,6 +750,25 @@ __global__ void __launch_bounds__(kThreads, 2)
     __syncthreads();
     tc_fence_after();
     if (warp == 1) tmem_dealloc(tmem, L::TMEM_COLS);
+    // A CTA that gave up: the rows of its jobs that were not stored become zero,
+    // so that an output allocated unfilled holds nothing else (each softmax warp
+    // its 16 rows of a job; the jobs numbered as the TMA warp numbers them).
+    if (run && warp >= kFirstSoftmaxWarp && *abort_flag) {
+        const int sw = warp - kFirstSoftmaxWarp;
+        const int rb = (warp & 3) * 32 + (sw >> 2) * 16;
+        JobCursor cur;
+        int64_t turn = t_first, t0 = 0;
+        for (int i = 0;; ++i, t0 += t_step, turn = (turn + 37) % t_step) {
+            if (i < jobs_done[sw]) continue;
+            AttnJob jb{};
+            if (t0 + turn < njobs) jb = job_at(p, t0 + turn, lane, cur);
+            if (!jb.valid) break;
+            const int end = jb.se < jb.q0 + rb + 16 ? jb.se : jb.q0 + rb + 16;
+            for (int q = jb.q0 + rb + (lane >> 4); q < end; q += 2)
+                reinterpret_cast<uint4*>(p.out + static_cast<int64_t>(q) * Hd + jb.h * kD)[lane & 15] =
+                    make_uint4(0, 0, 0, 0);
+        }
+    }
 }
 
 // Zeroes the output rows that attention_prefill_kernel leaves untouched: the
