@@ -37,6 +37,8 @@
 #include "internal.h"
 #include "ptx.cuh"
 
+#include <atomic>
+
 namespace w4a16 {
 
 namespace {
@@ -612,13 +614,13 @@ constexpr int kWideT = 384, kWideSS = W4A16_WIDE_SS, kWideST = 4;
 // take one); cached per device.
 int pair_slots(int sm_count) {
     constexpr int kMaxDev = 64;
-    static int cache[kMaxDev] = {};
+    static std::atomic<int> cache[kMaxDev] = {};
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDev) return sm_count / 2;
-    if (cache[dev] > 0) return cache[dev];
+    int n = cache[dev].load(std::memory_order_relaxed);
+    if (n > 0) return n;
     using L = Layout<kGemmT, kPairSS, kPairST, true>;
     auto kern = w4a16_ts_kernel<kGemmT, kPairSS, kPairST, kGemmDQ, kPlainEP, 1, false, true, 1>;
-    int n = 0;
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, L::SMEM_BYTES) ==
         cudaSuccess) {
         cudaLaunchConfig_t cfg = {};
@@ -636,7 +638,7 @@ int pair_slots(int sm_count) {
     }
     cudaGetLastError();  // a failed query leaves no sticky error for the next launch
     if (n <= 0) n = sm_count / 2;
-    cache[dev] = n;
+    cache[dev].store(n, std::memory_order_relaxed);
     return n;
 }
 
