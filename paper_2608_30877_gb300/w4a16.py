@@ -89,9 +89,16 @@ def version() -> int:
     return int(lib().w4a16_version())
 
 
+# The current stream's handle alone takes 0.3 us, a Stream object for it 2.9; the
+# function is not public, so a torch without it goes by the object.
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _stream(stream) -> int:
-    if stream is None:  # its handle alone takes 0.3 us, a Stream object for it 2.9
-        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+    if stream is None:
+        if _raw_stream is not None:
+            return _raw_stream(torch.cuda.current_device())
+        stream = torch.cuda.current_stream()
     return int(stream.cuda_stream) if hasattr(stream, "cuda_stream") else int(stream)
 
 

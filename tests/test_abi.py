@@ -129,3 +129,17 @@ def test_debug_build_exports_the_same_symbols():
         assert hasattr(D, name), name
     D.w4a16_status_string.restype = C.c_char_p
     assert b"debug" in D.w4a16_status_string(W.ERR_INDEX)
+
+
+def test_current_stream_without_the_private_handle_function(monkeypatch):
+    """The binding takes the current stream's handle from a torch function that is not
+    public; where a torch lacks it, the public Stream object serves."""
+    import torch
+
+    class FakeStream:
+        cuda_stream = 0x1234
+
+    monkeypatch.setattr(W, "_raw_stream", None, raising=False)
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda *a: FakeStream())
+    assert W._stream(None) == 0x1234
+    assert W._stream(FakeStream()) == 0x1234 and W._stream(7) == 7
