@@ -277,19 +277,22 @@ int launch_gemv_tc(const DeviceState& st, const GemvTcPlan& plan, const void* x,
                : W4A16_ERR_CUDA;
 }
 
-// Validated arguments -> one kernel launch.
-int launch_linear(const DeviceState& st, const void* x, const void* w, const void* s, void* out,
-                  int64_t M, int64_t N, int64_t K, int64_t g, const Epilogue& epi,
-                  cudaStream_t stream) {
+// The kernel that a linear layer runs on.
+struct LinearRoute {
+    enum Kind { kHead = 0, kRows = 1, kStream = 2, kGemm = 3 } kind;
+    GemvTcPlan plan;  // kStream
+    TsVariant gemm;   // kGemm
+};
+
+LinearRoute choose_linear(const DeviceState& st, int64_t M, int64_t N, int64_t K, int64_t g) {
+    LinearRoute r{};
     // a few rows: tokens over CTAs, unless so many tokens that the GEMM's one wave of
     // tiles is cheaper (12288 x 2: M = 64 4.9 us against 68, 65536 242 against 316;
     // 12288 x 8: M = 1000 17 against 74, 65536 824 against 318)
     if (N <= kHeadRows &&
         (M <= 128 || head_cost_us(M, N, K) < ts_cost_us(M, N, K, st.sm_count))) {
-        const HeadParams p{static_cast<const uint16_t*>(s), static_cast<uint16_t*>(out),
-                           static_cast<int>(M), static_cast<int>(N), static_cast<int>(K),
-                           static_cast<int>(g), epi};
-        return launch_head(x, w, p, st.sm_count, stream) == cudaSuccess ? W4A16_OK : W4A16_ERR_CUDA;
+        r.kind = LinearRoute::kHead;
+        return r;
     }
     // Up to 128 tokens the weights stream once per call on the streaming kernels
     // (12288 x 49152: M = 64 78 us there against 212 on the 256-token GEMM tiles,
@@ -300,28 +303,48 @@ int launch_linear(const DeviceState& st, const void* x, const void* w, const voi
     // 35 against 23, K = 49152 132 against 66) and from 9 tokens on (M = 16: N = 30000
     // 61 against 51, 49152 82 against 63).
     if (M <= 128) {
-        const GemvTcPlan plan = gemv_tc_plan(M, N, K, st.sm_count);
+        r.plan = gemv_tc_plan(M, N, K, st.sm_count);
         const bool rows = M <= 16 && g == 128 &&
-                          (g_small_m == 0 ? gemv_cost_us(M, N, K, st.sm_count) < plan.cost_us
+                          (g_small_m == 0 ? gemv_cost_us(M, N, K, st.sm_count) < r.plan.cost_us
                                           : g_small_m == 'm');
-        return rows ? launch_gemv(st, x, w, s, out, M, N, K, g, epi, stream)
-                    : launch_gemv_tc(st, plan, x, w, s, out, M, N, K, g, epi, stream);
+        r.kind = rows ? LinearRoute::kRows : LinearRoute::kStream;
+        return r;
     }
     // Beyond that too, in tiles of up to 128 tokens, where the GEMM's CTA pairs do
     // not fill the GPU (few weight rows, or a nearly empty last wave), by the two
     // modelled times: 12288 x 12288 at M = 130 47 us against 69, 333 66 against 95,
     // 512 104 against 136; at 1024 240 against 190, where the GEMM stays.
     if (g_gemm_pair && g_gemm_wide_from < 0) {
-        const GemvTcPlan plan = gemv_tc_plan(M, N, K, st.sm_count);
-        if (plan.cost_us < 0.95 * ts_cost_us(M, N, K, st.sm_count))
-            return launch_gemv_tc(st, plan, x, w, s, out, M, N, K, g, epi, stream);
+        r.plan = gemv_tc_plan(M, N, K, st.sm_count);
+        if (r.plan.cost_us < 0.95 * ts_cost_us(M, N, K, st.sm_count)) {
+            r.kind = LinearRoute::kStream;
+            return r;
+        }
     }
-    const TsVariant v = g_gemm_pair && (g_gemm_wide_from >= 0
-                                            ? M >= g_gemm_wide_from
-                                            : ts_prefer_wide(M, N, st.sm_count))
-                            ? TsVariant::kGemmPairWide
-                        : g_gemm_pair ? TsVariant::kGemmPair
-                                      : TsVariant::kGemm256;
+    r.kind = LinearRoute::kGemm;
+    r.gemm = g_gemm_pair && (g_gemm_wide_from >= 0 ? M >= g_gemm_wide_from
+                                                   : ts_prefer_wide(M, N, st.sm_count))
+                 ? TsVariant::kGemmPairWide
+             : g_gemm_pair ? TsVariant::kGemmPair
+                           : TsVariant::kGemm256;
+    return r;
+}
+
+// Validated arguments -> one kernel launch.
+int launch_linear(const DeviceState& st, const void* x, const void* w, const void* s, void* out,
+                  int64_t M, int64_t N, int64_t K, int64_t g, const Epilogue& epi,
+                  cudaStream_t stream) {
+    const LinearRoute route = choose_linear(st, M, N, K, g);
+    if (route.kind == LinearRoute::kHead) {
+        const HeadParams p{static_cast<const uint16_t*>(s), static_cast<uint16_t*>(out),
+                           static_cast<int>(M), static_cast<int>(N), static_cast<int>(K),
+                           static_cast<int>(g), epi};
+        return launch_head(x, w, p, st.sm_count, stream) == cudaSuccess ? W4A16_OK : W4A16_ERR_CUDA;
+    }
+    if (route.kind == LinearRoute::kRows) return launch_gemv(st, x, w, s, out, M, N, K, g, epi, stream);
+    if (route.kind == LinearRoute::kStream)
+        return launch_gemv_tc(st, route.plan, x, w, s, out, M, N, K, g, epi, stream);
+    const TsVariant v = route.gemm;
     const int T = ts_tokens_per_tile(v);
     alignas(64) CUtensorMap tx;
     alignas(64) CUtensorMap tw;
@@ -389,6 +412,26 @@ extern "C" int w4a16_linear_fused(const void* x_bf16, const void* w_packed_u8,
                        static_cast<int>(activation == W4A16_ACT_SWIGLU ? N / 2 : N)};
     return launch_linear(*st, x_bf16, w_packed_u8, scales_bf16, out_bf16, M, N, K, g, epi,
                          static_cast<cudaStream_t>(stream));
+}
+
+extern "C" int w4a16_selftest_route(int64_t M, int64_t N, int64_t K, int64_t g, int32_t* route) {
+    if (route == nullptr || M <= 0 || N <= 0 || K <= 0 || g <= 0 || K % g != 0)
+        return W4A16_ERR_INVALID_ARG;
+    if (g % 64 != 0 || M > kMaxDim || N > kMaxDim || K > kMaxDim) return W4A16_ERR_UNSUPPORTED;
+    DeviceState* st = nullptr;
+    const int rc = device_state(&st);
+    if (rc != W4A16_OK) return rc;
+    const LinearRoute r = choose_linear(*st, M, N, K, g);
+    const bool stream = r.kind == LinearRoute::kStream;
+    route[0] = r.kind;
+    route[1] = stream                           ? r.plan.tokens
+               : r.kind == LinearRoute::kGemm ? ts_tokens_per_tile(r.gemm)
+                                              : 0;
+    route[2] = stream                           ? r.plan.split
+               : r.kind == LinearRoute::kGemm ? (r.gemm == TsVariant::kGemm256 ? 1 : 2)
+                                              : 1;
+    route[3] = stream ? r.plan.rows_per_cta : 0;
+    return W4A16_OK;
 }
 
 extern "C" int w4a16_linear_stack(const w4a16_layer* layers, int64_t n_layers, int64_t M,

@@ -67,6 +67,7 @@ def lib() -> ctypes.CDLL:
         L.w4a16_get_device_error.argtypes = [p]
         L.w4a16_selftest_wait_timeout.argtypes = [i64, p]
         L.w4a16_selftest_set_wait_limit.argtypes = [i64]
+        L.w4a16_selftest_route.argtypes = [i64, i64, i64, i64, ctypes.POINTER(ctypes.c_int32)]
         L.w4a16_status_string.argtypes = [ctypes.c_int]
         L.w4a16_status_string.restype = ctypes.c_char_p
         L.w4a16_version.restype = ctypes.c_int
@@ -75,7 +76,7 @@ def lib() -> ctypes.CDLL:
                   "w4a16_attention_zero_outside", "w4a16_stack_graph_create", "w4a16_stack_graph_launch",
                   "w4a16_stack_graph_destroy", "w4a16_dequant", "w4a16_quantize",
                   "w4a16_get_device_error", "w4a16_selftest_wait_timeout",
-                  "w4a16_selftest_set_wait_limit"):
+                  "w4a16_selftest_set_wait_limit", "w4a16_selftest_route"):
             getattr(L, f).restype = ctypes.c_int
         _lib = L
     return _lib
@@ -283,6 +284,17 @@ def set_wait_limit(limit_ns: int) -> None:
     """Wait limit of the kernels launched from now on (0: the default);
     test hook, see include/w4a16.h."""
     _check("w4a16_selftest_set_wait_limit", lib().w4a16_selftest_set_wait_limit(int(limit_ns)))
+
+
+ROUTES = ("head", "rows", "stream", "gemm")
+
+
+def route(M: int, N: int, K: int, g: int = 128):
+    """(kernel of ROUTES, tokens per tile, CTAs per cluster, rows per CTA) that linear runs
+    with these sizes; test hook, see include/w4a16.h."""
+    r = (ctypes.c_int32 * 4)()
+    _check("w4a16_selftest_route", lib().w4a16_selftest_route(M, N, K, g, r))
+    return ROUTES[r[0]], r[1], r[2], r[3]
 
 
 def get_device_error(stream=None) -> int:

@@ -143,3 +143,12 @@ def test_current_stream_without_the_private_handle_function(monkeypatch):
     monkeypatch.setattr(torch.cuda, "current_stream", lambda *a: FakeStream())
     assert W._stream(None) == 0x1234
     assert W._stream(FakeStream()) == 0x1234 and W._stream(7) == 7
+
+
+def test_route_hook_rejects_bad_sizes(L):
+    r = (ctypes.c_int32 * 4)()
+    assert L.w4a16_selftest_route(8, 8, 256, 128, None) == W.ERR_INVALID_ARG
+    assert L.w4a16_selftest_route(0, 8, 256, 128, r) == W.ERR_INVALID_ARG
+    assert L.w4a16_selftest_route(8, 8, 200, 128, r) == W.ERR_INVALID_ARG
+    assert L.w4a16_selftest_route(8, 8, 256, 32, r) == W.ERR_UNSUPPORTED
+    assert L.w4a16_selftest_route(1 << 31, 8, 256, 128, r) == W.ERR_UNSUPPORTED
