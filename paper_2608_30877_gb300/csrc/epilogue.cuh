@@ -45,7 +45,7 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
 // the output, and read one by one after the stores they are a chain of memory latencies
 // (333 x 12288 x 12288 with a residual: 117 us one by one in 16-bit loads, 88 read
 // first, 69 in pairs; with SwiGLU 79 us at 16 bits and no swap, 72 so).
-template <int ACT, int CNT>
+template <int ACT, int CNT, bool PLAIN = false>
 __device__ __forceinline__ void store_tokens_act(const Epilogue& e, uint16_t* out,
                                                  const float (&v)[CNT], int m0, int m_end, int n,
                                                  bool ok, float bias, int lane) {
@@ -54,25 +54,29 @@ __device__ __forceinline__ void store_tokens_act(const Epilogue& e, uint16_t* ou
     const bool odd = (lane & 1) != 0;
     if constexpr (ACT != kActSwiGLU) {
         if ((e.n_out & 1) != 0) {  // rows of odd width: columns cannot pair up
-            const int count = ok ? m_end - m0 : 0;  // tokens to store
-            const int64_t at = static_cast<int64_t>(m0) * e.n_out + n;
+            if constexpr (PLAIN) {
+                // addresses that advance: with a 64-bit product per store 16384 x 64 x 12289
+                // takes 208 us against 125, 1000 x 64 x 36865 45.5 against 30 (fused they gain 10%
+                // in a GEMM with GELU and cost 10 to 25% with a residual and where K is split)
+                const int count = ok ? m_end - m0 : 0;  // tokens to store
+                uint16_t* dst = out + static_cast<int64_t>(m0) * e.n_out + n;
+#pragma unroll
+                for (int j = 0; j < CNT; ++j, dst += e.n_out)
+                    if (j < count) *dst = f32_to_bf16_rn(v[j]);
+                return;
+            }
             float r[CNT];
 #pragma unroll
-            for (int j = 0; j < CNT; ++j) r[j] = 0.0f;
-            if (e.residual != nullptr) {
-                const uint16_t* src = e.residual + at;
+            for (int j = 0; j < CNT; ++j)
+                r[j] = e.residual != nullptr && ok && m0 + j < m_end
+                           ? bf16_to_f32(e.residual[static_cast<int64_t>(m0 + j) * e.n_out + n])
+                           : 0.0f;
 #pragma unroll
-                for (int j = 0; j < CNT; ++j, src += e.n_out)
-                    if (j < count) r[j] = bf16_to_f32(*src);
-            }
-            // (addresses that advance: with a 64-bit product per store 16384 x 64 x 12289
-            // takes 208 us against 125, 1000 x 64 x 36865 45.5 against 30)
-            uint16_t* dst = out + at;
-#pragma unroll
-            for (int j = 0; j < CNT; ++j, dst += e.n_out) {
+            for (int j = 0; j < CNT; ++j) {
                 const float z = v[j] + bias;
                 const float h = (ACT == kActGELU ? gelu_f32(z) : z) + r[j];
-                if (j < count) *dst = f32_to_bf16_rn(h);
+                if (ok && m0 + j < m_end)
+                    out[static_cast<int64_t>(m0 + j) * e.n_out + n] = f32_to_bf16_rn(h);
             }
             return;
         }
@@ -123,7 +127,7 @@ __device__ __forceinline__ void store_tokens(const Epilogue& e, uint16_t* out,
                                              bool ok, float bias, int lane) {
     if constexpr (!FUSED) {
         const Epilogue plain{nullptr, nullptr, kActNone, e.n_out};
-        store_tokens_act<kActNone, CNT>(plain, out, v, m0, m_end, n, ok, 0.0f, lane);
+        store_tokens_act<kActNone, CNT, true>(plain, out, v, m0, m_end, n, ok, 0.0f, lane);
     } else if (e.act == kActSwiGLU) {
         store_tokens_act<kActSwiGLU, CNT>(e, out, v, m0, m_end, n, ok, bias, lane);
     } else if (e.act == kActGELU) {
