@@ -301,15 +301,16 @@ int w4a16_selftest_wait_timeout(int64_t limit_ns, void* stream);
 int w4a16_selftest_set_wait_limit(int64_t limit_ns);
 
 /*
- * Test hook: the kernel that w4a16_linear runs for these sizes on the current device
- * (nothing is launched), so that a test can state which one it exercises.
+ * Test hook: the kernel that w4a16_linear_fused runs for these sizes, activation and with or
+ * without a residual on the current device (w4a16_linear: 0, 0); nothing is launched.
  *   route[0]  0 few weight rows, 1 warp-level streaming, 2 tensor-core streaming,
  *             3 GEMM
  *   route[1]  tokens per tile (2, 3), else 0
  *   route[2]  CTAs of a cluster: those that split K (2), the GEMM's pair (3), else 1
  *   route[3]  weight rows per CTA (2), else 0
  */
-int w4a16_selftest_route(int64_t M, int64_t N, int64_t K, int64_t g, int32_t* route);
+int w4a16_selftest_route(int64_t M, int64_t N, int64_t K, int64_t g, int activation,
+                         int residual, int32_t* route);
 
 /* Static text for a status code; never NULL. */
 const char* w4a16_status_string(int status);

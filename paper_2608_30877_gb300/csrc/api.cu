@@ -284,28 +284,29 @@ struct LinearRoute {
     TsVariant gemm;   // kGemm
 };
 
-LinearRoute choose_linear(const DeviceState& st, int64_t M, int64_t N, int64_t K, int64_t g) {
+LinearRoute choose_linear(const DeviceState& st, int64_t M, int64_t N, int64_t K, int64_t g,
+                          const Epilogue& epi) {
     LinearRoute r{};
     // a few rows: tokens over CTAs, unless so many tokens that the GEMM's one wave of
     // tiles is cheaper (12288 x 2: M = 64 4.9 us against 68, 65536 242 against 316;
     // 12288 x 8: M = 1000 17 against 74, 65536 824 against 318)
     if (N <= kHeadRows &&
-        (M <= 128 || head_cost_us(M, N, K) < ts_cost_us(M, N, K, st.sm_count))) {
+        (M <= 128 || head_cost_us(M, N, K) < ts_cost_us(M, N, K, epi, st.sm_count))) {
         r.kind = LinearRoute::kHead;
         return r;
     }
     // Up to 128 tokens the weights stream once per call on the streaming kernels
     // (12288 x 49152: M = 64 78 us there against 212 on the 256-token GEMM tiles,
-    // M = 128 104 against 214).  M <= 16: the warp-level kernel has the higher rate
-    // between about 25000 and 36000 rows (M = 8: N = 30000 49.7 us against 51.4; 36864
-    // 52.3 against 52.5) and on the shortest K; the tcgen05 one elsewhere (49152 65.8
-    // against 63.2, 60000 124 against 99, and, its K split, 24576 46 against 37, 12288
-    // 35 against 23, K = 49152 132 against 66) and from 9 tokens on (M = 16: N = 30000
-    // 61 against 51, 49152 82 against 63).
+    // M = 128 104 against 214).  M <= 16, g = 128: the warp-level kernel where its modelled
+    // time is lower.  M <= 8, warp-level against tcgen05 (one launch after another, weights
+    // from HBM): K = 12288, N = 12288 34 against 22 us, 25000 45 / 35 (both K split), 30000
+    // 48.5 / 50, 36864 51 / 50.5, 49152 64.5 / 60.5, with SwiGLU 66 / 69; K = 1024, N = 12288 5.0
+    // / 6.2, 49152 9.9 / 10.1, with SwiGLU 10.7 / 13.9; K = 128, 98304 5.9 / 6.5.  M = 9..16: K =
+    // 12288, 30000 60 / 50; K = 1024, 12288 6.2 / 6.2.
     if (M <= 128) {
-        r.plan = gemv_tc_plan(M, N, K, st.sm_count);
+        r.plan = gemv_tc_plan(M, N, K, g, epi, st.sm_count);
         const bool rows = M <= 16 && g == 128 &&
-                          (g_small_m == 0 ? gemv_cost_us(M, N, K, st.sm_count) < r.plan.cost_us
+                          (g_small_m == 0 ? gemv_cost_us(M, N, K, epi, st.sm_count) < r.plan.cost_us
                                           : g_small_m == 'm');
         r.kind = rows ? LinearRoute::kRows : LinearRoute::kStream;
         return r;
@@ -315,8 +316,8 @@ LinearRoute choose_linear(const DeviceState& st, int64_t M, int64_t N, int64_t K
     // modelled times: 12288 x 12288 at M = 130 47 us against 69, 333 66 against 95,
     // 512 104 against 136; at 1024 240 against 190, where the GEMM stays.
     if (g_gemm_pair && g_gemm_wide_from < 0) {
-        r.plan = gemv_tc_plan(M, N, K, st.sm_count);
-        if (r.plan.cost_us < 0.95 * ts_cost_us(M, N, K, st.sm_count)) {
+        r.plan = gemv_tc_plan(M, N, K, g, epi, st.sm_count);
+        if (r.plan.cost_us < 0.95 * ts_cost_us(M, N, K, epi, st.sm_count)) {
             r.kind = LinearRoute::kStream;
             return r;
         }
@@ -334,7 +335,7 @@ LinearRoute choose_linear(const DeviceState& st, int64_t M, int64_t N, int64_t K
 int launch_linear(const DeviceState& st, const void* x, const void* w, const void* s, void* out,
                   int64_t M, int64_t N, int64_t K, int64_t g, const Epilogue& epi,
                   cudaStream_t stream) {
-    const LinearRoute route = choose_linear(st, M, N, K, g);
+    const LinearRoute route = choose_linear(st, M, N, K, g, epi);
     if (route.kind == LinearRoute::kHead) {
         const HeadParams p{static_cast<const uint16_t*>(s), static_cast<uint16_t*>(out),
                            static_cast<int>(M), static_cast<int>(N), static_cast<int>(K),
@@ -414,14 +415,19 @@ extern "C" int w4a16_linear_fused(const void* x_bf16, const void* w_packed_u8,
                          static_cast<cudaStream_t>(stream));
 }
 
-extern "C" int w4a16_selftest_route(int64_t M, int64_t N, int64_t K, int64_t g, int32_t* route) {
-    if (route == nullptr || M <= 0 || N <= 0 || K <= 0 || g <= 0 || K % g != 0)
+extern "C" int w4a16_selftest_route(int64_t M, int64_t N, int64_t K, int64_t g, int activation,
+                                    int residual, int32_t* route) {
+    if (route == nullptr || M <= 0 || N <= 0 || K <= 0 || g <= 0 || K % g != 0 || activation < 0 ||
+        activation > W4A16_ACT_GELU)
         return W4A16_ERR_INVALID_ARG;
     if (g % 64 != 0 || M > kMaxDim || N > kMaxDim || K > kMaxDim) return W4A16_ERR_UNSUPPORTED;
     DeviceState* st = nullptr;
     const int rc = device_state(&st);
     if (rc != W4A16_OK) return rc;
-    const LinearRoute r = choose_linear(*st, M, N, K, g);
+    // (the choice reads whether there is a residual, not where)
+    const Epilogue epi{nullptr, residual != 0 ? reinterpret_cast<const uint16_t*>(st) : nullptr, activation,
+                       static_cast<int>(activation == W4A16_ACT_SWIGLU ? N / 2 : N)};
+    const LinearRoute r = choose_linear(*st, M, N, K, g, epi);
     const bool stream = r.kind == LinearRoute::kStream;
     route[0] = r.kind;
     route[1] = stream                           ? r.plan.tokens

@@ -1,8 +1,11 @@
 // Small-M (M <= 16, g = 128) int4-dequant + matmul for sm_103a: the bandwidth-bound
-// regime where the whole packed weight matrix streams from HBM once per call, for
-// layers with enough rows to give every SM some 165 to 235 (with fewer, gemv_tc.cu's
-// split of K over clusters is faster, with more, its three tiles; from 9 tokens on it nearly
-// always is) and for the shortest K; the dispatch compares gemv_cost_us with its plan's.
+// regime where the whole packed weight matrix streams from HBM once per call, where its
+// modelled time (gemv_cost_us) is below that of gemv_tc.cu's plan.  Up to 8 tokens, plain:
+// K <= 1024 and up to 53000 rows; longer K where splitting it no longer helps and a
+// sub-partition's two or three warps are not yet full, 29000 to 35000 and 39000 to 43500 rows
+// at K = 12288 (on 152 SMs).  With a fused output stage, of which gemv_tc.cu finishes 32
+// tokens whatever M, 29000 to 53000 and 78000 to 107000 rows.  From 9 tokens on only plain
+// layers of K <= 1024 and few rows.
 //
 // Design, GB300-first:
 //   - persistent grid, one CTA per SM; CTA c owns a contiguous range of RB
@@ -533,15 +536,25 @@ int gemv_rows_per_cta(int64_t N, int sm_count) {
     return static_cast<int>(per);
 }
 
-double gemv_cost_us(int64_t M, int64_t N, int64_t K, int sm_count) {
+double gemv_cost_us(int64_t M, int64_t N, int64_t K, const Epilogue& epi, int sm_count) {
     const int64_t rb = gemv_rows_per_cta(N, sm_count);
     const int64_t waves = ((N + rb - 1) / rb + sm_count - 1) / sm_count;
-    // per 128-k stage: a fixed part and one per row (K = 12288, M <= 8: 65.0 us in all
-    // at 324 rows per CTA, 52.8 at 244, 46.5 at 162, 33.8 at 82; M = 9..16: 81, 65,
-    // 59; K = 49152 at 82 rows 126 and 148)
-    const double stage = M <= 8 ? 0.20 + 0.00134 * static_cast<double>(rb)
-                                : 0.25 + 0.0017 * static_cast<double>(rb);
-    return 4.0 + static_cast<double>(waves * (K / kBKS)) * stage;
+    // per 128-k stage: a fixed part, one per compute warp of the busiest sub-partition
+    // and one per row (K = 12288, M <= 8: 30 us in all for 34 rows per CTA, 34.1 for 82, 43.7
+    // for 132, 51.2 for 244, 59.9 for 264, 64.4 for 324; M = 9..16: 36.4, 39.1, 55.3, 64.1,
+    // 77.6, 80.8); in several waves the last, partial one shares HBM with fewer
+    const double warps = static_cast<double>((rb + 4 * kRowsPerWarp - 1) / (4 * kRowsPerWarp));
+    const double rows = static_cast<double>(rb);
+    const double stage = (M <= 8 ? 0.21 + 0.07 * warps + 0.00065 * rows
+                                 : 0.195 + 0.133 * warps + 0.0007 * rows) *
+                         (waves > 1 ? 0.95 : 1.0);
+    // a chunk's fused output stage (M = 1, 8, 16, N = 49152, K = 256: 4.8, 5.1, 5.9 us plain,
+    // 5.5, 6.0, 8.7 with a residual, 5.6, 6.2, 9.2 GELU, 5.8, 6.6, 10.0 SwiGLU)
+    const double output = !epilogue_fused(epi) ? 0.0
+                          : M <= 8             ? (epi.act == 1 ? 1.2 : epi.act == 2 ? 1.0 : 0.8)
+                                               : (epi.act == 1 ? 4.1 : epi.act == 2 ? 3.3 : 2.8);
+    return (M <= 8 ? 1.1 : 1.6) + static_cast<double>(waves) * (1.1 + 0.004 * rows + output) +
+           static_cast<double>(waves * (K / kBKS)) * stage;
 }
 
 int gemv_tokens_per_tile(int64_t M) { return M <= 8 ? 8 : 16; }

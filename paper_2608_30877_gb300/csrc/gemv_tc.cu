@@ -648,7 +648,8 @@ int cluster_slots(int split, int sm_count) {
 
 }  // namespace
 
-GemvTcPlan gemv_tc_plan(int64_t M, int64_t N, int64_t K, int sm_count) {
+GemvTcPlan gemv_tc_plan(int64_t M, int64_t N, int64_t K, int64_t g, const Epilogue& epi,
+                        int sm_count) {
     // us per 128-k stage of a CTA that holds 1, 2 or 3 tiles of 128 rows, by token
     // columns 32, 64, 96, 112, 128 (K = 12288, N = 19000 without a split, 36864 and 49152,
     // less 4 us: 41.4 / 45.4 / 46.6 / 48.0 / 52.3, 52.6 / 58.3 / 64 / 67.3 / 72.5 and
@@ -662,6 +663,19 @@ GemvTcPlan gemv_tc_plan(int64_t M, int64_t N, int64_t K, int sm_count) {
     const int64_t per = (M + tok_tiles - 1) / tok_tiles;
     best.tokens = per <= 32 ? 32 : per <= 64 ? 64 : per <= 96 ? 96 : per <= 112 ? 112 : 128;
     const int tok = best.tokens == 32 ? 0 : best.tokens == 64 ? 1 : (best.tokens - 64) / 16;
+    // What the choice between the splits leaves out and the one between the kernels needs:
+    // up to 16 tokens, against the warp-level kernel, the same stages one launch after
+    // another (39.1, 50.4 and 60.4 us in all; fused 53 and 64), a further wave (98304
+    // rows, K = 128 6.5 us, half of them 4.0) and the fused output stage of a chunk (K = 256,
+    // 49152 rows, M = 1: 5.4 us plain, 6.0 with a residual, 7.3 GELU, 8.8 SwiGLU); beyond, that
+    // of odd widths (M = 128, K = 64: 4.1 plain, 20 with GELU) and a long walk's second
+    // scales a stage where g is not 128 (M = 129, N = 36864, g = 64 150 us, 143 on the GEMM)
+    const bool fused = epilogue_fused(epi);
+    const double kFewTokensStageUs[3] = {0.38, fused ? 0.535 : 0.495, fused ? 0.64 : 0.60};
+    const double output =
+        M <= 16 ? (!fused ? 0.0 : epi.act == kActSwiGLU ? 2.8 : epi.act == kActGELU ? 1.9 : 0.6)
+                : (epilogue_odd(epi) && epi.act == kActGELU ? 15.0 : 0.0);
+    double chosen = 0.0;
     const int64_t KS = (K + kGroupK - 1) / kGroupK;
     for (int split = 1; split <= 8; split *= 2) {
         const int64_t slots = cluster_slots(split, sm_count);
@@ -682,8 +696,13 @@ GemvTcPlan gemv_tc_plan(int64_t M, int64_t N, int64_t K, int sm_count) {
         const double stages = static_cast<double>(waves) * static_cast<double>((KS + split - 1) / split);
         const double cost = 4.0 + stages * kStageUs[nt - 1][tok] +
                             (split > 1 ? 1.5 + 0.04 * best.tokens : 0.0);
-        if (best.cost_us == 0.0 || cost < best.cost_us) {
-            best.cost_us = cost;
+        if (chosen == 0.0 || cost < chosen) {
+            chosen = cost;
+            best.cost_us = cost + static_cast<double>(waves) * output / split +
+                           (g != 128 && best.tokens <= 96 && stages >= 64.0 ? 0.1 * stages : 0.0);
+            if (M <= 16)
+                best.cost_us += (static_cast<double>(waves) - 1.0) * 1.3 + 0.35 * (nt - 3) +
+                                stages * (kFewTokensStageUs[nt - 1] - kStageUs[nt - 1][tok]);
             best.split = split;
             best.rows_per_cta = static_cast<int>(rb);
             best.row_chunks = static_cast<int>((N + rb - 1) / rb);

@@ -18,6 +18,15 @@ struct Epilogue {
     int n_out;                 // output columns: N, or N / 2 for SwiGLU
 };
 
+// Whether the output stage does more than round and store.
+inline bool epilogue_fused(const Epilogue& e) {
+    return e.bias != nullptr || e.residual != nullptr || e.act != 0;
+}
+// Fused outputs of odd width, stored (and their residuals read) one by one.
+inline bool epilogue_odd(const Epilogue& e) {
+    return epilogue_fused(e) && e.act != 1 && (e.n_out & 1) != 0;
+}
+
 // Parameters of the fused dequant + tcgen05 kernel (everything except the
 // two TMA descriptors, which are passed as __grid_constant__ arguments).
 struct TsParams {
@@ -50,7 +59,7 @@ int ts_grid(TsVariant v, const TsParams& p, int sm_count);
 // 256-token ones for an M x N product (tile padding and the last wave).
 bool ts_prefer_wide(int64_t M, int64_t N, int sm_count);
 // Modelled time of the better of the two, in us.
-double ts_cost_us(int64_t M, int64_t N, int64_t K, int sm_count);
+double ts_cost_us(int64_t M, int64_t N, int64_t K, const Epilogue& epi, int sm_count);
 cudaError_t ts_launch(TsVariant v, const CUtensorMap* tmap_x, const CUtensorMap* tmap_w,
                       const TsParams& p, int grid, cudaStream_t stream);
 
@@ -73,7 +82,7 @@ struct GemvParams {
 // the SMs, tokens per x box for M, modelled time.
 int gemv_rows_per_cta(int64_t N, int sm_count);
 int gemv_tokens_per_tile(int64_t M);
-double gemv_cost_us(int64_t M, int64_t N, int64_t K, int sm_count);
+double gemv_cost_us(int64_t M, int64_t N, int64_t K, const Epilogue& epi, int sm_count);
 cudaError_t gemv_launch(const CUtensorMap* tmap_x, const CUtensorMap* tmap_w,
                         const GemvParams& p, int sm_count, cudaStream_t stream);
 
@@ -86,9 +95,10 @@ struct GemvTcPlan {
     int rows_per_cta;  // RB
     int row_chunks;    // ceil(N / RB)
     int num_chunks;    // row_chunks x token tiles
-    double cost_us;    // modelled time (the dispatch compares it with ts_cost_us)
+    double cost_us;    // modelled time
 };
-GemvTcPlan gemv_tc_plan(int64_t M, int64_t N, int64_t K, int sm_count);
+GemvTcPlan gemv_tc_plan(int64_t M, int64_t N, int64_t K, int64_t g, const Epilogue& epi,
+                        int sm_count);
 cudaError_t gemv_tc_launch(const CUtensorMap* tmap_x, const CUtensorMap* tmap_w,
                            const GemvParams& p, int tokens, int sm_count, cudaStream_t stream);
 

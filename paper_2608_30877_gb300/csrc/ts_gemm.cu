@@ -670,12 +670,14 @@ bool ts_prefer_wide(int64_t M, int64_t N, int sm_count) {
            units_per_pair(M, N, kGemmT, sm_count) * 100;
 }
 
-double ts_cost_us(int64_t M, int64_t N, int64_t K, int sm_count) {
+double ts_cost_us(int64_t M, int64_t N, int64_t K, const Epilogue& epi, int sm_count) {
     // a 256-token unit takes 0.344 us per 64-k stage (12288 x 12288 at 256
     // tokens: 70 us for one unit per pair, 146 us for two at N = 36864)
     const double narrow = static_cast<double>(units_per_pair(M, N, kGemmT, sm_count));
     const double wide = 1.37 * static_cast<double>(units_per_pair(M, N, kWideT, sm_count));
-    return 4.0 + 0.344 * static_cast<double>(K / kBK) * (wide < narrow ? wide : narrow);
+    // (one tile of odd width at K = 64: 6.4 us plain, 14.5 with GELU)
+    const double output = epilogue_odd(epi) && epi.act == kActGELU ? 8.5 : 0.0;
+    return 4.0 + (0.344 * static_cast<double>(K / kBK) + output) * (wide < narrow ? wide : narrow);
 }
 
 int ts_grid(TsVariant v, const TsParams& p, int sm_count) {

@@ -67,7 +67,8 @@ def lib() -> ctypes.CDLL:
         L.w4a16_get_device_error.argtypes = [p]
         L.w4a16_selftest_wait_timeout.argtypes = [i64, p]
         L.w4a16_selftest_set_wait_limit.argtypes = [i64]
-        L.w4a16_selftest_route.argtypes = [i64, i64, i64, i64, ctypes.POINTER(ctypes.c_int32)]
+        L.w4a16_selftest_route.argtypes = [i64, i64, i64, i64, ctypes.c_int, ctypes.c_int,
+                                           ctypes.POINTER(ctypes.c_int32)]
         L.w4a16_status_string.argtypes = [ctypes.c_int]
         L.w4a16_status_string.restype = ctypes.c_char_p
         L.w4a16_version.restype = ctypes.c_int
@@ -289,11 +290,12 @@ def set_wait_limit(limit_ns: int) -> None:
 ROUTES = ("head", "rows", "stream", "gemm")
 
 
-def route(M: int, N: int, K: int, g: int = 128):
-    """(kernel of ROUTES, tokens per tile, CTAs per cluster, rows per CTA) that linear runs
-    with these sizes; test hook, see include/w4a16.h."""
+def route(M: int, N: int, K: int, g: int = 128, act: int = ACT_NONE, residual: bool = False):
+    """(kernel of ROUTES, tokens per tile, CTAs per cluster, rows per CTA) that linear_fused
+    runs with these arguments; test hook, see include/w4a16.h."""
     r = (ctypes.c_int32 * 4)()
-    _check("w4a16_selftest_route", lib().w4a16_selftest_route(M, N, K, g, r))
+    _check("w4a16_selftest_route", lib().w4a16_selftest_route(
+        M, N, K, g, int(act), int(residual), r))
     return ROUTES[r[0]], r[1], r[2], r[3]
 
 

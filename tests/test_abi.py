@@ -147,8 +147,9 @@ def test_current_stream_without_the_private_handle_function(monkeypatch):
 
 def test_route_hook_rejects_bad_sizes(L):
     r = (ctypes.c_int32 * 4)()
-    assert L.w4a16_selftest_route(8, 8, 256, 128, None) == W.ERR_INVALID_ARG
-    assert L.w4a16_selftest_route(0, 8, 256, 128, r) == W.ERR_INVALID_ARG
-    assert L.w4a16_selftest_route(8, 8, 200, 128, r) == W.ERR_INVALID_ARG
-    assert L.w4a16_selftest_route(8, 8, 256, 32, r) == W.ERR_UNSUPPORTED
-    assert L.w4a16_selftest_route(1 << 31, 8, 256, 128, r) == W.ERR_UNSUPPORTED
+    assert L.w4a16_selftest_route(8, 8, 256, 128, 0, 0, None) == W.ERR_INVALID_ARG
+    assert L.w4a16_selftest_route(0, 8, 256, 128, 0, 0, r) == W.ERR_INVALID_ARG
+    assert L.w4a16_selftest_route(8, 8, 200, 128, 0, 0, r) == W.ERR_INVALID_ARG
+    assert L.w4a16_selftest_route(8, 8, 256, 32, 0, 0, r) == W.ERR_UNSUPPORTED
+    assert L.w4a16_selftest_route(1 << 31, 8, 256, 128, 0, 0, r) == W.ERR_UNSUPPORTED
+    assert L.w4a16_selftest_route(8, 8, 256, 128, 3, 0, r) == W.ERR_INVALID_ARG
