@@ -287,13 +287,22 @@ struct LinearRoute {
 LinearRoute choose_linear(const DeviceState& st, int64_t M, int64_t N, int64_t K, int64_t g,
                           const Epilogue& epi) {
     LinearRoute r{};
-    // a few rows: tokens over CTAs, unless so many tokens that the GEMM's one wave of
-    // tiles is cheaper (12288 x 2: M = 64 4.9 us against 68, 65536 242 against 316;
-    // 12288 x 8: M = 1000 17 against 74, 65536 824 against 318)
-    if (N <= kHeadRows &&
-        (M <= 128 || head_cost_us(M, N, K) < ts_cost_us(M, N, K, epi, st.sm_count))) {
+    // A few rows: tokens over CTAs, unless so many tokens that tiles of them are cheaper by
+    // 10% (the models' error), the streaming kernel's or the GEMM's (12288 x 2: M = 64 4.4
+    // us against 68, 65536 241 against 265; 12288 x 8: M = 1000 17 against 72, 65536 824 against
+    // 264; 64 x 4: M = 4000 5.8 against 6.6, 65536 62 against 14)
+    if (N <= kHeadRows) {
         r.kind = LinearRoute::kHead;
-        return r;
+        if (M <= 128) return r;
+        r.plan = gemv_tc_plan(M, N, K, g, epi, st.sm_count);
+        // what it would run on otherwise: token tiles, of which nearly all is reading x (the
+        // plan's stages leave that out), or the GEMM, 2 us more than modelled at short K
+        const double gemm = ts_cost_us(M, N, K, epi, st.sm_count);
+        const double read = 4.0 + 3.1e-7 * static_cast<double>(M) * static_cast<double>(K);
+        const double other = r.plan.cost_us >= 0.95 * gemm ? gemm + 2.0
+                             : r.plan.cost_us > read       ? r.plan.cost_us
+                                                           : read;
+        if (head_cost_us(M, N, K) < 1.1 * other) return r;
     }
     // Up to 128 tokens the weights stream once per call on the streaming kernels
     // (12288 x 49152: M = 64 78 us there against 212 on the 256-token GEMM tiles,

@@ -109,11 +109,15 @@ cudaError_t launch_tokens(const void* x, const void* w, const HeadParams& p, cud
 }  // namespace
 
 double head_cost_us(int64_t M, int64_t N, int64_t K) {
-    // the larger of reading x (65536 x 12288 x 2: 242 us) and the FMAs
-    // (65536 x 12288 x 8: 824 us)
-    const double mk = static_cast<double>(M) * static_cast<double>(K);
-    const double read = mk * 3.0e-7, fma = mk * static_cast<double>(N) * 1.28e-7;
-    return 3.0 + (read > fma ? read : fma);
+    // the FMAs behind the sums over the CTA's threads (65536 tokens, K = 64: 23 us for one row,
+    // 36 for two, 60 for three or four, 16384 tokens 34 for eight; 8000 x 12288 x 4 56 us),
+    // or reading x with half of the sums next to it (65536 x 12288 x 2 241 us)
+    const double m = static_cast<double>(M), mk = m * static_cast<double>(K);
+    const double nr = N <= 1 ? 1 : N <= 2 ? 2 : N <= 4 ? 4 : 8;  // rows the kernel computes
+    const double sums = m * (1.0e-4 + 2.3e-4 * nr);
+    const double fma = sums + mk * 0.64e-7 * (nr + static_cast<double>(N));
+    const double read = 0.5 * sums + mk * 2.65e-7;
+    return 1.7 + (read > fma ? read : fma);
 }
 
 cudaError_t launch_head(const void* x, const void* w, const HeadParams& p, int sm_count,

@@ -30,3 +30,14 @@ def test_kernel_by_size(M, N, K, g, kernel):
 def test_kernel_by_output_stage_waves_and_scales(M, N, K, g, act, residual, kernel):
     from paper_2608_30877_gb300 import w4a16 as W
     assert W.route(M, N, K, g, act, residual)[0] == kernel
+
+
+# few rows: the sums over a CTA's threads cost more than the products where K is short
+@pytest.mark.parametrize("M,N,K,head", [
+    (128, 8, 64, True), (1000, 8, 64, True), (16384, 8, 64, False), (65536, 4, 64, False),
+    (65536, 3, 256, False), (65536, 2, 64, False), (8000, 5, 512, False), (65536, 2, 12288, True),
+    (65536, 8, 12288, False),
+])
+def test_few_rows_by_tokens_and_length(M, N, K, head):
+    from paper_2608_30877_gb300 import w4a16 as W
+    assert (W.route(M, N, K, 64)[0] == "head") == head
