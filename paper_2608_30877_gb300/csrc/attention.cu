@@ -249,6 +249,12 @@ struct JobCursor {
 // work on all query blocks of a few heads, whose K and V come from DRAM once:
 // numbered with the heads fastest they did not stay in L2 (64 ragged pairs 1078 us, 1005
 // so; 64 x 1024 tokens 2044 and 1740; 10007 under a window of 4096 1360 and 1282).
+// A sequence that is most of the batch, of at most kBalanceRounds jobs a CTA, has the
+// heads fastest all the same: its query blocks then come heaviest first over the whole
+// call, which balances the CTAs (one sequence, us, head by head and so: 8192 tokens, 16 heads
+// 288 and 246, 6000, 8 heads 102 and 63, 4096, 96 heads 393 and 337; 10007, 64 heads, 17 jobs a
+// CTA, 834 and 853).
+constexpr int kBalanceRounds = 14;
 __device__ __forceinline__ AttnJob job_at(const AttnParams& p, int64_t t, int lane, JobCursor& cur) {
     AttnJob j{};
     const int x = static_cast<int>(t / p.H);
@@ -271,11 +277,19 @@ __device__ __forceinline__ AttnJob job_at(const AttnParams& p, int64_t t, int la
         if (who) {
             const int src = __ffs(who) - 1;
             const int n = __shfl_sync(0xffffffffu, nqb, src);
-            const int64_t r = t - static_cast<int64_t>(__shfl_sync(0xffffffffu, excl, src)) * p.H;
+            // (the job's number within the sequence: below n H, and device memory holds no
+            // 2^31 queries of H heads)
+            const uint32_t r = static_cast<uint32_t>(
+                t - static_cast<int64_t>(__shfl_sync(0xffffffffu, excl, src)) * p.H);
             j.ss = __shfl_sync(0xffffffffu, a, src);
             j.se = __shfl_sync(0xffffffffu, b, src);
-            j.h = static_cast<int>(r / n);
-            j.q0 = j.ss + (n - 1 - static_cast<int>(r % n)) * kBQ;
+            const bool balance = 2 * n > (p.M + kBQ - 1) / kBQ &&
+                                 static_cast<int64_t>(n) * p.H <=
+                                     kBalanceRounds * static_cast<int64_t>(gridDim.x);
+            const uint32_t per = static_cast<uint32_t>(balance ? p.H : n), major = r / per;
+            const int minor = static_cast<int>(r - major * per);
+            j.h = balance ? minor : static_cast<int>(major);
+            j.q0 = j.ss + (n - 1 - (balance ? static_cast<int>(major) : minor)) * kBQ;
             j.valid = true;
             return j;
         }
