@@ -246,11 +246,14 @@ __global__ void __launch_bounds__(kTopkThreads, 1)
 }
 
 // A CTA copies one kGatherChunk-element piece of a row at a time (blockIdx.y
-// and on): 64 rows of 24 KB on one CTA each were a serial chain of six loads
-// and stores per thread.
+// and on), in 16-byte units where rows have whole ones: 64 rows of 24 KB on one CTA each
+// were a serial chain of six loads and stores per thread.  Else element by element, all
+// of a thread's eight read before any is stored (5000 rows of 12289: 72 us by whole rows, 123
+// in pieces one element after the other, 52 so).
 constexpr int kGatherThreads = 256;
 constexpr int kGatherChunk = 8 * kGatherThreads;
 
+template <bool WHOLE>
 __global__ void __launch_bounds__(kGatherThreads)
     gather_rows_kernel(const uint16_t* __restrict__ src, int64_t src_rows, int64_t D,
                        const int32_t* __restrict__ idx, int64_t P, uint16_t* __restrict__ dst,
@@ -264,18 +267,82 @@ __global__ void __launch_bounds__(kGatherThreads)
         const uint16_t* s = src + (ok ? static_cast<int64_t>(r) : 0) * D;
         uint16_t* d = dst + p * D;
         for (int64_t j0 = static_cast<int64_t>(blockIdx.y) * kGatherChunk; j0 < D; j0 += j_step) {
-            if ((D & 7) == 0) {  // rows of whole 16-byte chunks (bases are 16-byte aligned)
-                const int64_t j = j0 + 8 * threadIdx.x;
-                if (j < D)
-                    *reinterpret_cast<uint4*>(d + j) =
-                        ok ? __ldg(reinterpret_cast<const uint4*>(s + j)) : make_uint4(0, 0, 0, 0);
+            if constexpr (WHOLE) {
+                // (two pieces in flight)
+                const int64_t j = j0 + 8 * threadIdx.x, k = j + j_step;
+                uint4 a = make_uint4(0, 0, 0, 0), b = a;
+                if (ok && j < D) a = __ldg(reinterpret_cast<const uint4*>(s + j));
+                if (ok && k < D) b = __ldg(reinterpret_cast<const uint4*>(s + k));
+                if (j < D) *reinterpret_cast<uint4*>(d + j) = a;
+                if (k < D) *reinterpret_cast<uint4*>(d + k) = b;
+                j0 += j_step;
             } else {
-                const int64_t end = j0 + kGatherChunk < D ? j0 + kGatherChunk : D;
-                for (int64_t j = j0 + threadIdx.x; j < end; j += kGatherThreads)
-                    d[j] = ok ? s[j] : static_cast<uint16_t>(0);
+                const int left = static_cast<int>(D - j0 < kGatherChunk ? D - j0 : kGatherChunk);
+                const uint16_t* sj = s + j0 + threadIdx.x;
+                uint16_t* dj = d + j0 + threadIdx.x;
+                uint16_t v[8];
+#pragma unroll
+                for (int u = 0; u < 8; ++u)
+                    v[u] = ok && static_cast<int>(threadIdx.x) + u * kGatherThreads < left
+                               ? __ldg(sj + u * kGatherThreads) : static_cast<uint16_t>(0);
+#pragma unroll
+                for (int u = 0; u < 8; ++u)
+                    if (static_cast<int>(threadIdx.x) + u * kGatherThreads < left)
+                        dj[u * kGatherThreads] = v[u];
             }
         }
     }
+}
+
+// Rows of fewer units (uint4, or pairs of elements) than a CTA has threads: the units of all rows
+// in one run over the threads, kGatherUnits in flight each (100000 rows of 100 elements: a
+// row per CTA 51 us, 72 in pieces as above, 20 so; of 128: 55, 57, 6.4; of 1: 39, 56, 2.7).
+// Index: 32 bits where that counts the units.
+constexpr int kGatherUnits = 4;
+
+template <typename Unit, typename Index>
+__global__ void __launch_bounds__(kGatherThreads)
+    gather_units_kernel(const Unit* __restrict__ src, int64_t src_rows, Index per_row,
+                        const int32_t* __restrict__ idx, Index total, Unit* __restrict__ dst,
+                        int* status) {
+    constexpr Index kBlock = kGatherThreads * kGatherUnits;
+    const Index step = static_cast<Index>(gridDim.x) * kBlock;
+    for (Index i0 = static_cast<Index>(blockIdx.x) * kBlock; i0 < total;
+         i0 = total - i0 > step ? i0 + step : total) {  // (no overflow past total)
+        Unit v[kGatherUnits];
+#pragma unroll
+        for (int u = 0; u < kGatherUnits; ++u) {
+            const Index at = static_cast<Index>(threadIdx.x + u * kGatherThreads);
+            if (at >= total - i0) continue;
+            const Index p = (i0 + at) / per_row, j = i0 + at - p * per_row;
+            const int32_t r = __ldg(idx + p);
+            const bool ok = r >= 0 && r < src_rows;
+            if (!ok && j == 0) atomicCAS(status, 0, 1 /* W4A16_ERR_INVALID_ARG */);
+            v[u] = Unit{};
+            if (ok) v[u] = __ldg(src + static_cast<int64_t>(r) * per_row + j);
+        }
+#pragma unroll
+        for (int u = 0; u < kGatherUnits; ++u) {
+            const Index at = static_cast<Index>(threadIdx.x + u * kGatherThreads);
+            if (at < total - i0) dst[i0 + at] = v[u];
+        }
+    }
+}
+
+template <typename Unit>
+void launch_gather_units(const uint16_t* src, int64_t src_rows, int64_t per_row, const int32_t* idx,
+                         int64_t P, uint16_t* dst, int* status, int sm_count, cudaStream_t stream) {
+    const int64_t total = P * per_row, block = kGatherThreads * kGatherUnits;
+    const int64_t need = (total + block - 1) / block, most = 8 * static_cast<int64_t>(sm_count);
+    const unsigned grid = static_cast<unsigned>(need < most ? need : most);
+    const Unit* s = reinterpret_cast<const Unit*>(src);
+    Unit* d = reinterpret_cast<Unit*>(dst);
+    if (total < (int64_t{1} << 32) - block)
+        gather_units_kernel<Unit, uint32_t><<<grid, kGatherThreads, 0, stream>>>(
+            s, src_rows, static_cast<uint32_t>(per_row), idx, static_cast<uint32_t>(total), d, status);
+    else
+        gather_units_kernel<Unit, uint64_t><<<grid, kGatherThreads, 0, stream>>>(
+            s, src_rows, static_cast<uint64_t>(per_row), idx, static_cast<uint64_t>(total), d, status);
 }
 
 template <bool BF16, int CTAS>
@@ -350,13 +417,22 @@ cudaError_t launch_topk_smallest(const void* scores, bool bf16, int64_t n, int k
 cudaError_t launch_gather_rows(const uint16_t* src, int64_t src_rows, int64_t D,
                                const int32_t* idx, int64_t P, uint16_t* dst, int* status,
                                int sm_count, cudaStream_t stream) {
+    const bool whole = (D & 7) == 0;  // rows of 16-byte units (bases are 16-byte aligned)
+    if ((whole ? D / 8 : D / 2) < kGatherThreads) {
+        if (whole)
+            launch_gather_units<uint4>(src, src_rows, D / 8, idx, P, dst, status, sm_count, stream);
+        else
+            launch_gather_units<uint16_t>(src, src_rows, D, idx, P, dst, status, sm_count, stream);
+        return cudaGetLastError();
+    }
     // pieces of rows until the CTAs fill the SMs eight times over
     const int64_t pieces = (D + kGatherChunk - 1) / kGatherChunk;
     const int64_t want = 8 * static_cast<int64_t>(sm_count);
     const int64_t bx = P < want ? P : want;
     const int64_t by = pieces < (want + bx - 1) / bx ? pieces : (want + bx - 1) / bx;
-    gather_rows_kernel<<<dim3(static_cast<unsigned>(bx), static_cast<unsigned>(by)), kGatherThreads,
-                         0, stream>>>(src, src_rows, D, idx, P, dst, status);
+    auto kern = whole ? gather_rows_kernel<true> : gather_rows_kernel<false>;
+    kern<<<dim3(static_cast<unsigned>(bx), static_cast<unsigned>(by)), kGatherThreads, 0, stream>>>(
+        src, src_rows, D, idx, P, dst, status);
     return cudaGetLastError();
 }
 
