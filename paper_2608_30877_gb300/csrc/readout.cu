@@ -18,8 +18,8 @@
 // The selected pairs are gathered by every CTA, which ranks its share of them by
 // counting smaller pairs, and stores them.  Nothing goes through global memory.
 // Bound by latency (about five cluster barriers) and the first digit's atomics:
-// 200000 scores, k = 1000 62 -> 20 us; 10000, k = 100 28.8 -> 10.8; 2000000, k = 1024
-// 295 -> 67 (before: seven passes over the scores by scalar loads, a digit search by one
+// 200000 scores, k = 1000 56 -> 21 us; 10000, k = 100 27.7 -> 11.3; 2000000, k = 1024
+// 295 -> 90 (before: seven passes over the scores by scalar loads, a digit search by one
 // thread and 55 sorting steps on one CTA).
 #include "internal.h"
 
@@ -137,14 +137,19 @@ __global__ void __launch_bounds__(kTopkThreads, 1)
     auto key_at = [&](int i) { return cached ? sh.keys[i] : order_key<BF16>(scores, lo + i); };
 
     // ---- radix select over (key, index): the k-th smallest pair, 11 bits at a
-    // time, the digits of the index only where equal keys straddle the k-th.  A
+    // time, the digits of the index only where equal keys straddle the k-th (2000 equal
+    // scores, k = 1: 20.5 us with all 32 bits of it, 15.2 with those of n).  A
     // pass ends the search as soon as a whole bin is wanted.  `top` holds the
     // digits found, `low` the bits below them.
     unsigned long long top = 0;
     int low = 64;
     uint32_t need = static_cast<uint32_t>(k);
     for (int pass = 0;; ++pass) {
-        const int bits = pass % 3 == 2 ? 10 : 11;
+        if (pass == 3) {  // on to the index: no pass over bits that none below n has
+            low = 32 - __clz(static_cast<int>(n) - 1);
+            top <<= 32 - low;
+        }
+        const int bits = pass == 2 ? 10 : low < 11 ? low : 11;
         uint32_t* hist = sh.hist[pass & 1];
         const int b0 = 2 * tid;  // this thread's bins
         if (pass == 0) {
@@ -405,8 +410,8 @@ bool wide_cluster_fits() {
 cudaError_t launch_topk_smallest(const void* scores, bool bf16, int64_t n, int k,
                                  int32_t* out_idx, float* out_val, cudaStream_t stream) {
     // 16 CTAs (a cluster size beyond the portable 8) where 8 cannot keep their keys in
-    // shared memory and the GPU can place them: 2000000 scores 69 us against 103.
-    // Below that their longer barriers cost more (200000: 27 against 21).
+    // shared memory and the GPU can place them: 2000000 scores 89 us against 127.
+    // Below that their longer barriers cost more (200000: 28 against 21).
     const bool wide = n > 8 * kTopkCache && wide_cluster_fits();
     return bf16 ? (wide ? launch_topk<true, 16>(scores, n, k, out_idx, out_val, stream)
                         : launch_topk<true, 8>(scores, n, k, out_idx, out_val, stream))

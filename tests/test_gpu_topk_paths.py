@@ -28,3 +28,19 @@ def test_topk_sizes_match_the_oracle(n, k, ties, bf16):
     torch.cuda.synchronize()
     assert idx.cpu().numpy().tolist() == want_i.tolist()
     assert val.cpu().numpy().tobytes() == want_v.tobytes()
+
+
+@pytest.mark.parametrize("n", [2, 3, 1024, 1025, 2048, 2049, 4097, 70000, 4194305])
+@pytest.mark.parametrize("kind", ["equal", "two"])
+def test_topk_among_equal_scores(n, kind):
+    """The k-th falls among equal scores, so the search goes on to the index: sizes around
+    the powers of two where its digits change."""
+    from paper_2608_30877_gb300 import w4a16 as W
+    s = np.full(n, -7.25, dtype=np.float32)
+    if kind == "two":
+        s[np.random.default_rng(n).random(n) < 0.5] = np.nan
+    for k in [777] if n > 1000000 else sorted({1, min(n, 2), min(n, 777), min(n, 1024)}):
+        want_i, want_v = O.topk_smallest(s, k)
+        idx, val = W.topk_smallest(torch.from_numpy(s).cuda(), k)
+        assert idx.cpu().numpy().tolist() == want_i.tolist()
+        assert val.cpu().numpy().tobytes() == want_v.tobytes()
