@@ -2,6 +2,10 @@
 generator, oracle-side quantisation on the CPU, device uploads, tolerances."""
 from __future__ import annotations
 
+import os
+import subprocess
+import sys
+
 import numpy as np
 import torch
 
@@ -118,3 +122,29 @@ def assert_close_fused(gpu: np.ndarray, y: np.ndarray, ref: np.ndarray, act: int
     assert worst <= 1.0, f"{what}: worst error / bound = {worst:.3f}, {m}"
     assert m["rel_fro"] <= REL_FRO, f"{what}: {m}"
     return m
+
+
+# Environments that force a GEMM variant for every layer beyond 128 tokens (the library
+# reads them once, so they take a child process), with the route they give: tokens per
+# tile, CTAs per cluster.
+GEMM_ENVS = {
+    "wide": ({"W4A16_GEMM_WIDE": "1"}, (384, 2)),
+    "pair": ({"W4A16_GEMM_WIDE": "0"}, (256, 2)),
+    "one-cta": ({"W4A16_GEMM_PAIR": "0"}, (256, 1)),
+}
+
+
+def run_in_child(env: dict, module: str, function: str, *args) -> None:
+    """Runs tests.<module>.<function>(*args) in a child process with `env` added."""
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    code = (f"import sys; sys.path.insert(0, {root!r})\nfrom tests import {module}\n"
+            f"{module}.{function}(*{args!r})\nprint('ok')")
+    r = subprocess.run([sys.executable, "-c", code], env=dict(os.environ, **env),
+                       capture_output=True, text=True, timeout=600)
+    assert r.returncode == 0 and "ok" in r.stdout, r.stdout[-3000:] + r.stderr[-3000:]
+
+
+def assert_gemm(W, variant: str, *sizes) -> None:
+    """The layer of these sizes (and act, residual) runs on the GEMM variant named."""
+    name, tokens, ctas, _ = W.route(*sizes)
+    assert (name, tokens, ctas) == ("gemm", *GEMM_ENVS[variant][1]), (sizes, name, tokens, ctas)

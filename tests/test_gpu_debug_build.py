@@ -1,7 +1,8 @@
 """The W4A16_DEBUG build on the GPU: every kernel runs its index checks (TMA
 coordinates and destinations, tensor-memory columns, store rows) on ragged
 shapes of every dispatch path, no check fails, and the results still match
-the oracle.  Runs in a child process that loads libw4a16_debug.so."""
+the oracle.  Runs in child processes that load libw4a16_debug.so, one per way of
+forcing the kernels that shapes of this size would not reach."""
 import os
 import subprocess
 import sys
@@ -21,12 +22,8 @@ from paper_2608_30877_gb300 import synthetic as S
 from paper_2608_30877_gb300 import w4a16 as W
 from tests.gpu_helpers import assert_close, bf16_to_f64, host_case, to_device
 assert W.LIB_PATH.endswith("libw4a16_debug.so"), W.LIB_PATH
-# (M, N, K, g): CTA-pair GEMM with a ragged last pair, warp-level and
-# tensor-core small-M kernels (32, 64 and 128 token columns), 32-token tiles
-# (g = 64)
-for (M, N, K, g) in [(300, 1000, 1024, 128), (520, 384, 512, 128), (8, 2000, 1280, 128),
-                     (24, 1234, 640, 128), (48, 1234, 640, 128), (100, 1234, 640, 128),
-                     (5, 200, 256, 64)]:
+for (M, N, K, g) in {cases!r}:
+    assert W.route(M, N, K, g)[0] == {kernel!r}, (M, N, K, g, W.route(M, N, K, g))
     x, xb, packed, scales = host_case(M, N, K, g, M + 1, N + 2)
     xd, wd, sd = to_device(x, packed, scales)
     out = W.linear(xd, wd, sd, g)
@@ -52,10 +49,24 @@ print("ok")
 """
 
 
-def test_debug_build_checks_pass_and_results_match():
+GEMM_CASES = [(300, 1000, 1024, 128), (520, 384, 512, 128), (129, 257, 576, 192), (900, 130, 320, 64)]
+
+
+@pytest.mark.parametrize("kernel,env,cases", [
+    # 32, 64, 96, 112 and 128 token columns, K split and whole, K ending inside a stage, token tiles
+    ("stream", {"W4A16_SMALL_M": "tc"}, [(8, 2000, 1280, 128), (24, 1234, 640, 128), (48, 1234, 4096, 128),
+                                         (90, 300, 1088, 64), (100, 1234, 640, 128), (128, 60010, 256, 128),
+                                         (5, 200, 256, 64), (300, 1000, 1024, 128)]),
+    ("rows", {"W4A16_SMALL_M": "mma"}, [(1, 300, 128, 128), (8, 2000, 1280, 128), (13, 60010, 256, 128)]),
+    ("head", {}, [(64, 2, 1024, 128), (700, 8, 192, 64)]),
+    ("gemm", {"W4A16_GEMM_WIDE": "1"}, GEMM_CASES),
+    ("gemm", {"W4A16_GEMM_WIDE": "0"}, GEMM_CASES),
+    ("gemm", {"W4A16_GEMM_PAIR": "0"}, GEMM_CASES),
+])
+def test_debug_build_checks_pass_and_results_match(kernel, env, cases):
     from paper_2608_30877_gb300 import build as B
     B.build(debug=True)
-    env = dict(os.environ, W4A16_DEBUG="1")
-    r = subprocess.run([sys.executable, "-c", _CHILD.format(root=ROOT)], env=env,
-                       capture_output=True, text=True, timeout=900)
+    env = dict(os.environ, W4A16_DEBUG="1", **env)
+    r = subprocess.run([sys.executable, "-c", _CHILD.format(root=ROOT, cases=cases, kernel=kernel)],
+                       env=env, capture_output=True, text=True, timeout=900)
     assert r.returncode == 0 and "ok" in r.stdout, r.stdout[-3000:] + r.stderr[-3000:]

@@ -7,6 +7,7 @@ import pytest
 import torch
 
 from oracle import oracle as O
+from tests.gpu_helpers import GEMM_ENVS, assert_gemm, run_in_child
 
 pytestmark = pytest.mark.gpu
 
@@ -15,13 +16,13 @@ EDGE_SCALES = [0.0, 0.25, 0.2490234375, -0.25, -0.2490234375, 9.2e-41, -1e-38, 3
                -7.25e-3, 0.0014982223510742188, 1.5, 250.0, -3e30, 1e37]
 
 
-@pytest.mark.parametrize("M,N,K,g", [
-    (20, 66, 64, 64), (64, 300, 128, 128),               # streaming kernels
-    (128, 400, 192, 64), (100, 130, 256, 256),
-    (300, 300, 320, 64), (300, 257, 256, 128),           # 256- and 384-token GEMM tiles
-    (700, 40, 384, 128),
-])
-def test_one_hot_activations_give_the_dequantised_weights(M, N, K, g):
+STREAM_CASES = [(20, 66, 64, 64), (64, 300, 128, 128), (128, 400, 192, 64), (100, 130, 256, 256),
+                (300, 300, 320, 64), (700, 40, 384, 128)]
+# every form of the GEMM's scale index: one per stage, two stages per scale, a shift, a division
+GEMM_CASES = [(300, 300, 320, 64), (300, 257, 256, 128), (700, 40, 512, 256), (200, 130, 576, 192)]
+
+
+def check_values(M, N, K, g):
     from paper_2608_30877_gb300 import w4a16 as W
     rng = np.random.default_rng(M + N + K)
     packed = rng.integers(0, 256, size=(N, K // 2), dtype=np.uint8)
@@ -42,3 +43,22 @@ def test_one_hot_activations_give_the_dequantised_weights(M, N, K, g):
     # equal as numbers: the sign of a zero is not kept through the accumulation
     assert np.array_equal(got, want[:, :n])
     assert W.get_device_error() == W.OK
+
+
+def check_gemm_values(variant):
+    from paper_2608_30877_gb300 import w4a16 as W
+    for case in GEMM_CASES:
+        assert_gemm(W, variant, *case)
+        check_values(*case)
+
+
+@pytest.mark.parametrize("M,N,K,g", STREAM_CASES)
+def test_one_hot_activations_give_the_dequantised_weights(M, N, K, g):
+    from paper_2608_30877_gb300 import w4a16 as W
+    assert W.route(M, N, K, g)[0] == "stream"
+    check_values(M, N, K, g)
+
+
+@pytest.mark.parametrize("variant", GEMM_ENVS)
+def test_one_hot_activations_on_the_gemm(variant):
+    run_in_child(GEMM_ENVS[variant][0], "test_gpu_dequant_values", "check_gemm_values", variant)

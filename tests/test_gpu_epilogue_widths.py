@@ -7,14 +7,16 @@ import torch
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("M,N,K", [
-    (23, 513, 1024), (101, 514, 1024), (33, 1001, 2048),  # K split over a cluster
-    (40, 40001, 256), (127, 40002, 256),                  # whole K per CTA
-    (2047, 8193, 256), (2049, 8194, 256),                 # GEMM tiles
+@pytest.mark.parametrize("kernel,split,M,N,K", [
+    ("stream", 8, 23, 513, 4096), ("stream", 8, 101, 514, 4096), ("stream", 8, 33, 1001, 4224),
+    ("stream", 1, 23, 513, 1024), ("stream", 1, 101, 514, 1024),
+    ("stream", 1, 40, 40001, 256), ("stream", 1, 127, 40002, 256),   # whole K per CTA
+    ("gemm", 2, 2047, 8193, 256), ("gemm", 2, 2049, 8194, 256),
 ])
 @pytest.mark.parametrize("act", [0, 2])
-def test_in_place_residual_at_every_width(M, N, K, act):
+def test_in_place_residual_at_every_width(kernel, split, M, N, K, act):
     from paper_2608_30877_gb300 import w4a16 as W
+    assert W.route(M, N, K, 128, act, True)[::2] == (kernel, split)
     gen = torch.Generator(device="cuda").manual_seed(M + N)
     rnd = lambda *s: torch.randn(s, generator=gen, device="cuda")
     x = rnd(M, K).bfloat16()

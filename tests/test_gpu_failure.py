@@ -13,7 +13,7 @@ import torch
 
 from oracle import oracle as O
 from paper_2608_30877_gb300 import synthetic as S
-from tests.gpu_helpers import assert_close, bf16_to_f64, host_case, to_device
+from tests.gpu_helpers import GEMM_ENVS, assert_close, bf16_to_f64, host_case, run_in_child, to_device
 
 pytestmark = pytest.mark.gpu
 
@@ -70,37 +70,59 @@ def short_waits():
         W.set_wait_limit(0)
 
 
-# (M, N, K, g): large-M tcgen05 GEMM on CTA pairs (several tiles per pair),
-# the warp-level small-M streaming kernel, the tcgen05 small-M streaming
-# kernel with 32, 64 and 128 token columns, the 32-token tcgen05 tiles (g = 64)
-ABORT_CASES = [(600, 128 * 400, 2048, 128), (8, 8192, 4096, 128), (24, 8192, 4096, 128),
-               (48, 8192, 4096, 128), (96, 8192, 4096, 128),
-               (16, 4096, 1024, 64)]
+# (M, N, K, g, kernel): large-M tcgen05 GEMM on CTA pairs (several tiles per pair), the
+# tcgen05 streaming kernel with 32, 64 and 96 token columns, K split, and with g = 64
+ABORT_CASES = [(600, 128 * 400, 2048, 128, "gemm"), (8, 8192, 4096, 128, "stream"),
+               (24, 8192, 4096, 128, "stream"), (48, 8192, 4096, 128, "stream"),
+               (96, 8192, 4096, 128, "stream"), (16, 4096, 1024, 64, "stream"),
+               (24, 49152, 2048, 128, "stream")]
 
 
-@pytest.mark.parametrize("M,N,K,g", ABORT_CASES)
-def test_linear_abort_path_under_short_waits(short_waits, M, N, K, g):
-    W = short_waits
+def check_abort(M, N, K, g, kernel, act=0, residual=False):
+    W = _W()
+    assert W.route(M, N, K, g, act, residual)[0] == kernel
     x = S.make_x(M, K, 3, "cuda")
     w = torch.zeros((N, K // 2), dtype=torch.uint8, device="cuda")
     s = torch.zeros((N, K // g), dtype=torch.bfloat16, device="cuda")
-    W.linear(x, w, s, g)
-    assert W.get_device_error() == W.ERR_TIMEOUT
-    W.set_wait_limit(0)
+    assert W.get_device_error() == W.OK
+    W.set_wait_limit(1)
+    try:
+        if act or residual:
+            n_out = N // 2 if act == W.ACT_SWIGLU else N
+            res = torch.zeros((M, n_out), dtype=torch.bfloat16, device="cuda") if residual else None
+            W.linear_fused(x, w, s, g, act=act, residual=res, out=res)
+        else:
+            W.linear(x, w, s, g)
+        assert W.get_device_error() == W.ERR_TIMEOUT
+    finally:
+        W.set_wait_limit(0)
     _linear_still_correct(M=M if M <= 128 else 200, g=g)
 
 
-def test_fused_abort_path_under_short_waits(short_waits):
-    W = short_waits
-    M, N, K = 300, 128 * 200, 2048
-    x = S.make_x(M, K, 3, "cuda")
-    w = torch.zeros((N, K // 2), dtype=torch.uint8, device="cuda")
-    s = torch.zeros((N, K // 128), dtype=torch.bfloat16, device="cuda")
-    res = torch.zeros((M, N // 2), dtype=torch.bfloat16, device="cuda")
-    W.linear_fused(x, w, s, 128, act=W.ACT_SWIGLU, residual=res, out=res)
-    assert W.get_device_error() == W.ERR_TIMEOUT
-    W.set_wait_limit(0)
-    _linear_still_correct()
+@pytest.mark.parametrize("M,N,K,g,kernel", ABORT_CASES)
+def test_linear_abort_path_under_short_waits(M, N, K, g, kernel):
+    check_abort(M, N, K, g, kernel)
+
+
+def test_fused_abort_path_under_short_waits():
+    W = _W()
+    check_abort(300, 128 * 200, 2048, 128, "stream", W.ACT_SWIGLU, True)
+
+
+def check_abort_forced(kernel, *cases):
+    for case in cases:
+        check_abort(*case[:4], kernel, *case[4:])
+
+
+def test_warp_level_abort_path_under_short_waits():
+    run_in_child({"W4A16_SMALL_M": "mma"}, "test_gpu_failure", "check_abort_forced", "rows",
+                 (8, 8192, 4096, 128), (16, 60000, 1024, 128), (3, 8192, 4096, 128, 1, True))
+
+
+@pytest.mark.parametrize("variant", GEMM_ENVS)
+def test_fused_gemm_abort_path_under_short_waits(variant):
+    run_in_child(GEMM_ENVS[variant][0], "test_gpu_failure", "check_abort_forced", "gemm",
+                 (300, 128 * 200, 2048, 128, 1, True), (900, 128 * 100, 2048, 128, 2, False))
 
 
 def test_attention_abort_path_under_short_waits(short_waits):

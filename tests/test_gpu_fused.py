@@ -1,14 +1,15 @@
 """Parity of the fused epilogue (w4a16_linear_fused) with the oracle:
 act(x W^T + bias) + residual for every activation, with and without bias and
-residual (also in place), on the small-M streaming kernel (g = 128), the
-32-token tcgen05 tiles (small M, g = 64) and the large-M tcgen05 GEMM."""
+residual (also in place), on both streaming kernels and, forced, on every variant of
+the large-M tcgen05 GEMM."""
 import numpy as np
 import pytest
 import torch
 
 from oracle import oracle as O
 from paper_2608_30877_gb300 import synthetic as S
-from tests.gpu_helpers import assert_close_fused, bf16_to_f64, host_case, prepare_weights, to_device
+from tests.gpu_helpers import (GEMM_ENVS, assert_close_fused, assert_gemm, bf16_to_f64, host_case,
+                               prepare_weights, run_in_child, to_device)
 
 pytestmark = pytest.mark.gpu
 
@@ -34,7 +35,7 @@ def _case(M, N, K, g, seed, act, with_bias, with_res):
             (None if res is None else to_dev(res)), ref, y, bias)
 
 
-SHAPES = [  # (M, N, K, g): streaming kernel, 32-token tcgen05 tiles, large-M GEMM
+SHAPES = [  # (M, N, K, g): streaming kernels, with token tiles from 300 on
     (8, 1000, 1024, 128), (16, 4096, 512, 128), (24, 1234, 384, 128), (5, 200, 256, 64),
     (300, 1000, 1024, 128), (40, 258, 512, 128), (64, 1000, 1024, 128),
     (100, 1000, 1024, 128),
@@ -63,6 +64,49 @@ def test_fused_residual_in_place(M):
     W.linear_fused(xd, wd, sd, g, act=W.ACT_GELU, bias=bias, residual=buf, out=buf)
     torch.cuda.synchronize()
     assert_close_fused(bf16_to_f64(buf), y, ref, W.ACT_GELU, bias_bits, f"in-place residual M={M}")
+
+
+# odd and even widths, several token tiles and weight pairs, every activation with a residual
+GEMM_SHAPES = [(300, 1000, 1024, 128), (700, 514, 576, 192), (257, 129, 320, 64)]
+
+
+def check_gemm(variant):
+    W = _W()
+    for M, N, K, g in GEMM_SHAPES:
+        for act in (0, 1, 2):
+            if act == W.ACT_SWIGLU and N % 2:
+                continue
+            for with_bias, with_res in ((True, False), (True, True), (False, True)):
+                assert_gemm(W, variant, M, N, K, g, act, with_res)
+                xd, wd, sd, bias, res, ref, y, bias_bits = _case(M, N, K, g, 19 * M + N + act, act,
+                                                                 with_bias, with_res)
+                out = W.linear_fused(xd, wd, sd, g, act=act, bias=bias, residual=res)
+                what = f"{variant} {M}x{K}x{N} g{g} act{act} b{with_bias} r{with_res}"
+                assert_close_fused(bf16_to_f64(out), y, ref, act, bias_bits, what)
+                if with_res:  # in place
+                    W.linear_fused(xd, wd, sd, g, act=act, bias=bias, residual=res, out=res)
+                    assert torch.equal(res, out), what
+    assert W.get_device_error() == W.OK
+
+
+@pytest.mark.parametrize("variant", GEMM_ENVS)
+def test_fused_on_every_gemm_variant(variant):
+    run_in_child(GEMM_ENVS[variant][0], "test_gpu_fused", "check_gemm", variant)
+
+
+def check_rows():
+    W = _W()
+    for M, N, K in ((1, 1000, 1024), (8, 60002, 256), (9, 514, 1280), (16, 4096, 512)):
+        for act in (0, 1, 2):
+            assert W.route(M, N, K, 128, act, True)[0] == "rows"
+            xd, wd, sd, bias, res, ref, y, bias_bits = _case(M, N, K, 128, 23 * M + N + act, act, True, True)
+            W.linear_fused(xd, wd, sd, 128, act=act, bias=bias, residual=res, out=res)
+            assert_close_fused(bf16_to_f64(res), y, ref, act, bias_bits, f"rows {M}x{K}x{N} act{act}")
+    assert W.get_device_error() == W.OK
+
+
+def test_fused_on_the_warp_level_kernel():
+    run_in_child({"W4A16_SMALL_M": "mma"}, "test_gpu_fused", "check_rows")
 
 
 def test_fused_none_equals_plain_linear():
@@ -160,6 +204,8 @@ def test_fused_swiglu_small_m_readout_scale(M):
     2 x 49152 interleaved rows: more row chunks than SMs), on sampled output
     columns for every token."""
     W = _W()
+    assert W.route(M, S.MLP_SWIGLU.N, S.MLP_SWIGLU.K, 128, W.ACT_SWIGLU, True)[0] == \
+        ("rows" if M == 8 else "stream")
     c = S.MLP_SWIGLU
     packed, scales, wd, sd = prepare_weights(c.N, c.K, c.g, c.w_seed)
     x = S.make_x(M, c.K, 700 + M, "cuda")

@@ -8,7 +8,7 @@ import torch
 
 from oracle import oracle as O
 from paper_2608_30877_gb300 import synthetic as S
-from tests.gpu_helpers import (assert_close, assert_close_chain, bf16_to_f64, host_case,
+from tests.gpu_helpers import (GEMM_ENVS, assert_close, assert_close_chain, bf16_to_f64, host_case,
                                oracle_chain, to_device)
 
 pytestmark = pytest.mark.gpu
@@ -189,7 +189,7 @@ def test_error_codes_launch_nothing():
     (72, 4100, 1152, 128),
 ])
 def test_small_m_streaming_kernel_shapes(M, N, K, g):
-    """M <= 128 with g = 128 runs a row-range streaming kernel: ragged row
+    """M <= 128 runs a row-range streaming kernel: ragged row
     ranges, 8 to 128 token columns, group counts that leave padding stages
     in the last round of stage slots, and N large enough that a CTA takes a
     second row range (more row ranges than SMs)."""
@@ -205,6 +205,7 @@ from oracle import oracle as O
 from tests.gpu_helpers import assert_close, bf16_to_f64, host_case, to_device
 from paper_2608_30877_gb300 import w4a16 as W
 for (M, N, K) in {cases!r}:
+    assert W.route(M, N, K, 128)[0] == {kernel!r}
     x, xb, packed, scales = host_case(M, N, K, 128, 300 + M, 301 + M)
     xd, wd, sd = to_device(x, packed, scales)
     out = W.linear(xd, wd, sd, 128)
@@ -218,18 +219,20 @@ print("ok")
 
 @pytest.mark.parametrize("kernel", ["tc", "mma"])
 def test_small_m_kernels_every_m(kernel):
-    """Both small-M streaming kernels at every M they can be forced to
-    (W4A16_SMALL_M), on ragged shapes: the dispatch picks one by M, and
-    each must be correct everywhere."""
+    """Both small-M streaming kernels at every M they serve (W4A16_SMALL_M forces
+    one up to 16 tokens; beyond, up to 128, it is always the tensor-core one), on
+    ragged shapes: the dispatch picks one by modelled time, and each must be
+    correct everywhere."""
     import os
     import subprocess
     import sys
     root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
-    Ms = (1, 2, 5, 8, 13, 16, 17, 24, 31, 32) + ((33, 40, 57, 64, 65, 99, 128) if kernel == "tc"
-                                                 else ())
+    Ms = (1, 2, 5, 8, 9, 13, 16) + ((17, 24, 31, 32, 33, 40, 57, 64, 65, 99, 128)
+                                    if kernel == "tc" else ())
     cases = [(M, 1000 + 2 * M, 384 if M % 2 else 1280) for M in Ms]
     env = dict(os.environ, W4A16_SMALL_M=kernel)
-    r = subprocess.run([sys.executable, "-c", _FORCED_KERNEL_CHECK.format(root=root, cases=cases)],
+    r = subprocess.run([sys.executable, "-c", _FORCED_KERNEL_CHECK.format(
+        root=root, cases=cases, kernel="rows" if kernel == "mma" else "stream")],
                        env=env, capture_output=True, text=True, timeout=600)
     assert r.returncode == 0 and "ok" in r.stdout, r.stdout + r.stderr
 
@@ -245,9 +248,10 @@ def test_small_m_kernels_several_chunks_per_cta(kernel):
     import subprocess
     import sys
     root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
-    cases = [(M, 60010, 256) for M in (3, 16, 24, 32) + ((40, 64, 96, 128) if kernel == "tc" else ())]
+    cases = [(M, 60010, 256) for M in (3, 16) + ((24, 32, 40, 64, 96, 128) if kernel == "tc" else ())]
     env = dict(os.environ, W4A16_SMALL_M=kernel)
-    r = subprocess.run([sys.executable, "-c", _FORCED_KERNEL_CHECK.format(root=root, cases=cases)],
+    r = subprocess.run([sys.executable, "-c", _FORCED_KERNEL_CHECK.format(
+        root=root, cases=cases, kernel="rows" if kernel == "mma" else "stream")],
                        env=env, capture_output=True, text=True, timeout=600)
     assert r.returncode == 0 and "ok" in r.stdout, r.stdout + r.stderr
 
@@ -258,15 +262,18 @@ import numpy as np, torch
 sys.path.insert(0, {root!r})
 from oracle import oracle as O
 from paper_2608_30877_gb300 import synthetic as S
-from tests.gpu_helpers import assert_close, bf16_to_f64, host_case, to_device
+from tests.gpu_helpers import assert_close, assert_gemm, bf16_to_f64, host_case, to_device
 from paper_2608_30877_gb300 import w4a16 as W
-for (M, N, K) in {cases!r}:
-    x, xb, packed, scales = host_case(M, N, K, 128, 500 + M, 501 + N)
+for (M, N, K, g) in {cases!r}:
+    assert_gemm(W, {variant!r}, M, N, K, g)
+    x, xb, packed, scales = host_case(M, N, K, g, 500 + M, 501 + N)
     xd, wd, sd = to_device(x, packed, scales)
-    out = W.linear(xd, wd, sd, 128)
+    out = W.linear(xd, wd, sd, g)
+    again = W.linear(xd, wd, sd, g)
     torch.cuda.synchronize()
-    ref = O.linear_rows(xb, packed, scales, N, K, 128, nthreads=O.max_threads())
-    assert_close(bf16_to_f64(out), ref, f"M={{M}} N={{N}} K={{K}}")
+    ref = O.linear_rows(xb, packed, scales, N, K, g, nthreads=O.max_threads())
+    assert_close(bf16_to_f64(out), ref, f"M={{M}} N={{N}} K={{K}} g={{g}}")
+    assert torch.equal(out, again)
 assert W.get_device_error() == W.OK
 # the abort path under a lowered wait limit, then a correct call again
 W.set_wait_limit(1)
@@ -284,18 +291,21 @@ print("ok")
 """
 
 
-@pytest.mark.parametrize("env", [{"W4A16_GEMM_WIDE": "1"}, {"W4A16_GEMM_WIDE": "0"},
-                                 {"W4A16_GEMM_PAIR": "0"}])
-def test_large_m_gemm_variants_ragged(env):
+@pytest.mark.parametrize("variant", GEMM_ENVS)
+def test_large_m_gemm_variants_ragged(variant):
     """Every large-M GEMM variant forced on ragged shapes (ragged token tiles,
     an odd number of 128-row weight tiles, K not a multiple of the 384-token
-    tile's stage count), then its abort path: the 384-token CTA pairs (the
-    default from 16384 tokens), the 256-token CTA pairs and one CTA per tile."""
+    tile's stage count, every form of the scale index), twice, then its abort
+    path: the 384-token CTA pairs, the 256-token CTA pairs and one CTA per tile."""
     import os
     import subprocess
     import sys
     root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
-    cases = [(33, 128, 128), (300, 384, 256), (385, 1000, 640), (769, 640, 1152), (1200, 2048, 512)]
-    r = subprocess.run([sys.executable, "-c", _FORCED_GEMM_CHECK.format(root=root, cases=cases)],
-                       env=dict(os.environ, **env), capture_output=True, text=True, timeout=600)
+    cases = [(129, 128, 128, 128), (300, 384, 256, 128), (385, 1000, 640, 128), (769, 640, 1152, 128),
+             (1200, 2048, 512, 128), (300, 1000, 320, 64), (500, 257, 1024, 256), (257, 300, 576, 192),
+             (400, 130, 960, 320)]
+    r = subprocess.run([sys.executable, "-c", _FORCED_GEMM_CHECK.format(root=root, cases=cases,
+                                                                        variant=variant)],
+                       env=dict(os.environ, **GEMM_ENVS[variant][0]), capture_output=True, text=True,
+                       timeout=600)
     assert r.returncode == 0 and "ok" in r.stdout, r.stdout + r.stderr
