@@ -63,20 +63,20 @@ __device__ __forceinline__ void store_tokens_act(const Epilogue& e, uint16_t* ou
 #pragma unroll
                 for (int j = 0; j < CNT; ++j, dst += e.n_out)
                     if (j < count) *dst = f32_to_bf16_rn(v[j]);
-                return;
-            }
-            float r[CNT];
+            } else {
+                float r[CNT];
 #pragma unroll
-            for (int j = 0; j < CNT; ++j)
-                r[j] = e.residual != nullptr && ok && m0 + j < m_end
-                           ? bf16_to_f32(e.residual[static_cast<int64_t>(m0 + j) * e.n_out + n])
-                           : 0.0f;
+                for (int j = 0; j < CNT; ++j)
+                    r[j] = e.residual != nullptr && ok && m0 + j < m_end
+                               ? bf16_to_f32(e.residual[static_cast<int64_t>(m0 + j) * e.n_out + n])
+                               : 0.0f;
 #pragma unroll
-            for (int j = 0; j < CNT; ++j) {
-                const float z = v[j] + bias;
-                const float h = (ACT == kActGELU ? gelu_f32(z) : z) + r[j];
-                if (ok && m0 + j < m_end)
-                    out[static_cast<int64_t>(m0 + j) * e.n_out + n] = f32_to_bf16_rn(h);
+                for (int j = 0; j < CNT; ++j) {
+                    const float z = v[j] + bias;
+                    const float h = (ACT == kActGELU ? gelu_f32(z) : z) + r[j];
+                    if (ok && m0 + j < m_end)
+                        out[static_cast<int64_t>(m0 + j) * e.n_out + n] = f32_to_bf16_rn(h);
+                }
             }
             return;
         }

@@ -68,16 +68,27 @@ __device__ __forceinline__ void mbar_arrive_expect_tx(uint32_t bar, uint32_t byt
 // warps do not take issue slots from the working ones.
 constexpr uint32_t kSuspendHintNs = 0x20000;
 
-// Whether the phase has completed, without suspending the thread.
+// Whether the phase has completed, without suspending the thread (kCluster: see below).
+template <bool kCluster = false>
 __device__ __forceinline__ bool mbar_test_wait(uint32_t bar, uint32_t parity) {
     uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"(bar), "r"(parity)
-        : "memory");
+    if constexpr (kCluster) {
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "mbarrier.test_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+            "selp.u32 %0, 1, 0, p;\n\t}"
+            : "=r"(ok)
+            : "r"(bar), "r"(parity)
+            : "memory");
+    } else {
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+            "selp.u32 %0, 1, 0, p;\n\t}"
+            : "=r"(ok)
+            : "r"(bar), "r"(parity)
+            : "memory");
+    }
     return ok != 0;
 }
 
@@ -147,21 +158,22 @@ __device__ __forceinline__ bool tma_box_ok(uint32_t dst, uint32_t box_bytes, uin
 // launch's wait limit, kWaitLimitNs unless a test lowers it) or kWaitIterCap
 // polls the waiter gives up, raises the CTA's abort flag and records a
 // timeout in the device status word.  With the default limit the clock and
-// the flag are checked every few polls; with a lowered one (a test of the
-// abort path) after every failed poll, so that the first wait that does not
-// complete at once gives up.  The drains before a kernel exits (its own
-// copies and MMAs in flight) always use kWaitLimitNs.
+// the flag are checked every few polls, with a lowered one (a test of the
+// abort path) after every failed poll.  A poll may suspend its thread until the
+// phase completes, so a lowered limit does not by itself make a wait run out:
+// each producer waits for its first copy with polls that do not suspend
+// (short_limit_ok), and a debug build polls that way in every wait, so that there
+// any role can be the first to give up.  The drains before a kernel exits (its
+// own copies and MMAs in flight) always use kWaitLimitNs.
 constexpr uint64_t kWaitLimitNs = 4000000000ull;  // 4 s
 constexpr uint32_t kWaitIterCap = 1u << 26;
 
-// The producers' check for a lowered limit (a test of the abort path): a poll of the
-// waits below may suspend its thread until the phase completes, whatever the
-// limit, so each producer waits for its first copy here, with polls that do not.
-// Always true with the default limit.
+// The producers' check for a lowered limit.  Always true with the default one, and in a
+// debug build.
 __device__ __forceinline__ bool short_limit_ok(uint32_t bar, uint32_t parity,
                                                volatile int* abort_flag, int* status,
                                                uint64_t limit_ns) {
-    if (limit_ns >= kWaitLimitNs) return true;
+    if (kDebugChecks || limit_ns >= kWaitLimitNs) return true;
     const uint64_t t0 = global_timer_ns();
     while (!mbar_test_wait(bar, parity)) {
         if (global_timer_ns() - t0 > limit_ns) {
@@ -173,6 +185,15 @@ __device__ __forceinline__ bool short_limit_ok(uint32_t bar, uint32_t parity,
     return true;
 }
 
+// A poll of the waits below.
+template <bool kCluster>
+__device__ __forceinline__ bool mbar_poll(uint32_t bar, uint32_t parity, uint64_t limit_ns) {
+    if constexpr (kDebugChecks) {
+        if (limit_ns < kWaitLimitNs) return mbar_test_wait<kCluster>(bar, parity);
+    }
+    return mbar_try_wait<kCluster>(bar, parity);
+}
+
 // Wait by one thread.  Returns false if the wait ran out or the CTA aborted.
 // With SLEEP_NS the thread sleeps between polls, for waits that have stages in
 // hand (a TMA producer with a full ring): its polls then take no issue slots
@@ -180,11 +201,11 @@ __device__ __forceinline__ bool short_limit_ok(uint32_t bar, uint32_t parity,
 template <bool kCluster = false, uint32_t SLEEP_NS = 0>
 __device__ __forceinline__ bool wait_one(uint32_t bar, uint32_t parity, volatile int* abort_flag,
                                          int* status, uint64_t limit_ns) {
-    if (mbar_try_wait<kCluster>(bar, parity)) return true;
+    if (mbar_poll<kCluster>(bar, parity, limit_ns)) return true;
     const uint64_t t0 = global_timer_ns();
     for (uint32_t it = 1;; ++it) {
         if (SLEEP_NS > 0) __nanosleep(SLEEP_NS);
-        if (mbar_try_wait<kCluster>(bar, parity)) return true;
+        if (mbar_poll<kCluster>(bar, parity, limit_ns)) return true;
         if ((it & 31u) == 0u || limit_ns < kWaitLimitNs) {
             if (*abort_flag) return false;
             if (it > kWaitIterCap || global_timer_ns() - t0 > limit_ns) {
@@ -204,12 +225,12 @@ template <bool kCluster = false, uint32_t SLEEP_NS = 0>
 __device__ __forceinline__ bool wait_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag,
                                           int* status, uint64_t limit_ns) {
     // (the timer is slow to read: only once a poll has failed)
-    if (__all_sync(0xffffffffu, mbar_try_wait<kCluster>(bar, parity))) return true;
+    if (__all_sync(0xffffffffu, mbar_poll<kCluster>(bar, parity, limit_ns))) return true;
     const uint32_t lane = threadIdx.x & 31u;
     const uint64_t t0 = global_timer_ns();
     for (uint32_t it = 1;; ++it) {
         if (SLEEP_NS > 0) __nanosleep(SLEEP_NS);
-        const bool done = mbar_try_wait<kCluster>(bar, parity);
+        const bool done = mbar_poll<kCluster>(bar, parity, limit_ns);
         if (__all_sync(0xffffffffu, done)) return true;
         if ((it & (SLEEP_NS > 0 ? 7u : 31u)) == 0u || limit_ns < kWaitLimitNs) {
             int give_up = 0;
@@ -231,7 +252,8 @@ __device__ __forceinline__ bool wait_warp(uint32_t bar, uint32_t parity, volatil
 __device__ __forceinline__ bool wait_warp2(uint32_t bar0, uint32_t parity0, uint32_t bar1,
                                            uint32_t parity1, volatile int* abort_flag, int* status,
                                            uint64_t limit_ns) {
-    const bool d0 = mbar_try_wait<false>(bar0, parity0), d1 = mbar_try_wait<false>(bar1, parity1);
+    const bool d0 = mbar_poll<false>(bar0, parity0, limit_ns),
+               d1 = mbar_poll<false>(bar1, parity1, limit_ns);
     if (__all_sync(0xffffffffu, d0 && d1)) return true;
     return wait_warp(bar0, parity0, abort_flag, status, limit_ns) &&
            wait_warp(bar1, parity1, abort_flag, status, limit_ns);
@@ -314,12 +336,6 @@ __device__ __forceinline__ void tma_load_2d_hint(uint32_t dst, const CUtensorMap
 __device__ __forceinline__ uint64_t l2_policy_evict_first() {
     uint64_t p;
     asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));
-    return p;
-}
-
-__device__ __forceinline__ uint64_t l2_policy_evict_last() {
-    uint64_t p;
-    asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(p));
     return p;
 }
 

@@ -70,3 +70,46 @@ def test_debug_build_checks_pass_and_results_match(kernel, env, cases):
     r = subprocess.run([sys.executable, "-c", _CHILD.format(root=ROOT, cases=cases, kernel=kernel)],
                        env=env, capture_output=True, text=True, timeout=900)
     assert r.returncode == 0 and "ok" in r.stdout, r.stdout[-3000:] + r.stderr[-3000:]
+
+
+_ABORT = r"""
+import sys
+sys.path.insert(0, {root!r})
+import torch
+from paper_2608_30877_gb300 import w4a16 as W
+from paper_2608_30877_gb300 import synthetic as S
+from tests.test_gpu_failure import check_abort_forced, _linear_still_correct
+assert W.LIB_PATH.endswith("libw4a16_debug.so"), W.LIB_PATH
+check_abort_forced({kernel!r}, *{cases!r})
+H = 8
+qkv = S.make_x(4096, 3 * H * 128, 9, "cuda")
+st = torch.arange(0, 4097, 1024, dtype=torch.int32, device="cuda")
+want = W.attention_prefill(qkv, st, H)
+W.set_wait_limit(1)
+got = W.attention_prefill(qkv, st, H)
+assert W.get_device_error() == W.ERR_TIMEOUT
+W.set_wait_limit(0)
+rows = lambda t: t.view(4096, H, 128)
+assert ((rows(got) == rows(want)).all(-1) | (rows(got) == 0).all(-1)).all()
+_linear_still_correct()
+print("ok")
+"""
+
+
+@pytest.mark.parametrize("kernel,env,cases", [
+    ("stream", {"W4A16_SMALL_M": "tc"}, [(8, 8192, 4096, 128), (96, 8192, 4096, 128),
+                                         (24, 49152, 2048, 128), (300, 25600, 2048, 128, 1, True)]),
+    ("rows", {"W4A16_SMALL_M": "mma"}, [(8, 8192, 4096, 128), (16, 60000, 1024, 128)]),
+    ("gemm", {"W4A16_GEMM_WIDE": "1"}, [(900, 12800, 2048, 128), (300, 25600, 2048, 128, 1, True)]),
+    ("gemm", {"W4A16_GEMM_WIDE": "0"}, [(900, 12800, 2048, 128), (300, 25600, 2048, 128, 1, True)]),
+    ("gemm", {"W4A16_GEMM_PAIR": "0"}, [(900, 12800, 2048, 128), (300, 25600, 2048, 128, 1, True)]),
+])
+def test_any_role_may_give_up_first(kernel, env, cases):
+    """With a lowered wait limit the debug build's waits poll without suspending, in every
+    role, so the first to give up is not only the producer."""
+    from paper_2608_30877_gb300 import build as B
+    B.build(debug=True)
+    env = dict(os.environ, W4A16_DEBUG="1", **env)
+    r = subprocess.run([sys.executable, "-c", _ABORT.format(root=ROOT, cases=cases, kernel=kernel)],
+                       env=env, capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0 and "ok" in r.stdout, r.stdout[-3000:] + r.stderr[-3000:]

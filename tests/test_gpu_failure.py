@@ -3,9 +3,11 @@ reported through the device status word, and the context stays usable.
 
 Two forms.  The self test runs the kernels' own wait helpers on a barrier
 that nothing arrives on.  The abort-path tests lower the wait limit of the
-real kernels (w4a16_selftest_set_wait_limit) so that their first wait that
-does not complete at once gives up: the kernel records the timeout, drains
-the copies and MMAs it has in flight, frees its tensor memory and returns.
+real kernels (w4a16_selftest_set_wait_limit) so that the wait for a producer's
+first copy gives up (in a debug build, where tests/test_gpu_debug_build.py does the
+same, the first wait of any role that does not complete at once): the kernel
+records the timeout, drains the copies and MMAs it has in flight, frees its
+tensor memory and returns.
 A correct linear right after shows that the context survived."""
 import numpy as np
 import pytest
