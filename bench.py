@@ -41,27 +41,30 @@ NCU_TRAFFIC = {
     # mean of one launch per stack shape at M = 16384 (384-token tiles, as in
     # the benched stack), scaled by 4 to M = 65536
     # (profiles/gemm_pair_wide_stack_traffic_m16384.md)
-    ("stack", "ts", "96e8156fb430b201"): 7.1506e9 * 4,
+    ("stack", "ts", "755eda9058f870bf"): 7.1498e9 * 4,
     # QKV prefill 4096x12288x36864 (384-token CTA pairs), one launch
     # (profiles/gemm_pair_wide_qkv_prefill_4096x12288x36864.md)
-    ("qkv", "ts", "96e8156fb430b201"): 1.4726e9 + 0.2892e9,
+    ("qkv", "ts", "755eda9058f870bf"): 1.4728e9 + 0.2891e9,
     # MLP up / down at 8192 tokens (384-token CTA pairs), one launch each
     # (DRAM counters only; profiles/gemm_pair_mlp_traffic_8192.md)
-    ("mlp_up", "ts", "96e8156fb430b201"): 3.9457e9 + 0.8025e9,
-    ("mlp_down", "ts", "96e8156fb430b201"): 4.7834e9 + 0.1975e9,
-    # small-M readout, M = 8 and M = 32 (tensor-core streaming kernel, 32 token
-    # columns), 12288x49152, one launch each (profiles/gemv_tc_m32_12288x49152.md)
-    ("gemv", "gemv", "7dfe2915b3327dfb"): 0.32543e9 + 0.00322e9,
-    ("gemv32", "gemvtc", "7dfe2915b3327dfb"): 0.32668e9 + 0.00322e9,
+    ("mlp_up", "ts", "755eda9058f870bf"): 3.9444e9 + 0.8024e9,
+    ("mlp_down", "ts", "755eda9058f870bf"): 4.7834e9 + 0.1975e9,
+    # small-M readout, M = 8, 16 and 32 (tensor-core streaming kernel, 32 token columns),
+    # 12288x49152, one launch each (profiles/gemv_tc_m32_12288x49152.md)
+    ("gemv8", "gemv", "8fcee59793c4dbda"): 0.32545e9 + 0.00320e9,
+    ("gemv16", "gemv", "8fcee59793c4dbda"): 0.32529e9 + 0.00319e9,
+    ("gemv32", "gemv", "8fcee59793c4dbda"): 0.32670e9 + 0.00321e9,
     # attention prefill per 8 pairs of 1024 tokens x 96 heads (full capture of
     # one 8-pair launch); scaled by pairs / 8 for the benched launch
-    ("attention", "attn", "2c879819e8d835be"): 0.6044e9 + 0.1733e9,
+    ("attention", "attn", "721466a15446229a"): 0.6045e9 + 0.1727e9,
 }
 
-KERNEL_FILES = {"ts": ("ts_gemm.cu", "dequant.cuh", "ptx.cuh"),
-                "gemv": ("gemv_tc.cu", "dequant.cuh", "ptx.cuh"),  # M <= 16 at this width
-                "gemvtc": ("gemv_tc.cu", "dequant.cuh", "ptx.cuh"),
-                "attn": ("attention.cu",)}
+# what decides a launch's traffic: the kernel, what it includes, and the dispatch that
+# picks it and its tiles
+KERNEL_FILES = {"ts": ("ts_gemm.cu", "epilogue.cuh", "dequant.cuh", "ptx.cuh", "internal.h", "api.cu"),
+                "gemv": ("gemv_tc.cu", "gemv_rows.cu", "epilogue.cuh", "dequant.cuh", "ptx.cuh",
+                         "internal.h", "api.cu"),
+                "attn": ("attention.cu", "ptx.cuh", "internal.h")}
 
 
 def kernel_source_hash(kind: str = "ts") -> str:
@@ -80,14 +83,10 @@ def ncu_traffic(config: str, m: int, pairs: int = 8):
         t = NCU_TRAFFIC.get((config, "attn", kernel_source_hash("attn")))
         return None if t is None else t * pairs / 8  # qkv and out grow with the pairs
     if config == "gemv":
-        if 17 <= m <= 32:  # the capture is of M = 32
-            return NCU_TRAFFIC.get(("gemv32", "gemvtc", kernel_source_hash("gemvtc")))
-        if m > 8:  # no capture of M = 9..16
-            return NCU_TRAFFIC.get(("gemv16", "gemv", kernel_source_hash("gemv")))
-        kind = "gemv"
-    else:
-        kind = "ts"
-    return NCU_TRAFFIC.get((config, kind, kernel_source_hash(kind)))
+        # captured at M = 8, 16 and 32; fewer tokens read that much less of x only
+        config = "gemv8" if m <= 8 else "gemv16" if m <= 16 else "gemv32"
+        return NCU_TRAFFIC.get((config, "gemv", kernel_source_hash("gemv"))) if m <= 32 else None
+    return NCU_TRAFFIC.get((config, "ts", kernel_source_hash("ts")))
 
 
 # The GB300's nominal dense bf16 tensor rate and HBM3e bandwidth: each

@@ -32,8 +32,8 @@
 //
 // What bounds it (96 heads, us; before and after the job order below, the job ring,
 // the streaming hints and the order of the issuers' waits): 64 ragged pairs of 200 to
-// 1024 tokens 1105 -> 973, 64 x 1024 tokens 2110 -> 1684, 10007 tokens under a window of
-// 4096 1390 -> 1247 (64% of the bf16 peak).  DRAM traffic was the limit of the short
+// 1024 tokens 1148 -> 945, 64 x 1024 tokens 2210 -> 1660, 10007 tokens under a window of
+// 4096 1498 -> 1275 (63% of the bf16 peak).  DRAM traffic was the limit of the short
 // sequences (76% of its rate, 6.4 GB for 3.8 GB of input and output) and is now 4.6 GB.
 // In the steady state a block takes ~1560 clocks per CTA: 8 MMAs of S (N = 64, whose 6 KB
 // of operands from shared memory take longer than their math) and 4 of PV of each of the
@@ -251,9 +251,9 @@ struct JobCursor {
 // so; 64 x 1024 tokens 2044 and 1740; 10007 under a window of 4096 1360 and 1282).
 // A sequence that is most of the batch, of at most kBalanceRounds jobs a CTA, has the
 // heads fastest all the same: its query blocks then come heaviest first over the whole
-// call, which balances the CTAs (one sequence, us, head by head and so: 8192 tokens, 16 heads
-// 288 and 246, 6000, 8 heads 102 and 63, 4096, 96 heads 393 and 337; 10007, 64 heads, 17 jobs a
-// CTA, 834 and 853).
+// call, which balances the CTAs (one sequence under a window of 4096, us, head by head and so: 8192
+// tokens, 16 heads 227 and 181, 6000, 8 heads 106 and 70, 4096, 96 heads 385 and 344; 10007, 64
+// heads, 17 jobs a CTA, 834 and 853).
 constexpr int kBalanceRounds = 14;
 __device__ __forceinline__ AttnJob job_at(const AttnParams& p, int64_t t, int lane, JobCursor& cur) {
     AttnJob j{};

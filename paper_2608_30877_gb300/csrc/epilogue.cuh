@@ -43,8 +43,9 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
 // columns; SwiGLU pairs rows (n, n ^ 1) = (gate, up) of one column, whose values
 // meet the same way.  The residuals are read before anything is stored: they may be
 // the output, and read one by one after the stores they are a chain of memory latencies
-// (333 x 12288 x 12288 with a residual: 117 us one by one in 16-bit loads, 88 read
-// first, 69 in pairs; with SwiGLU 79 us at 16 bits and no swap, 72 so).
+// (333 x 12288 x 12288 on the same buffers call after call, with a residual: 117 us one by
+// one in 16-bit loads, 88 read first, 70 in pairs; with SwiGLU 79 us at 16 bits and no
+// swap, 70 so).
 template <int ACT, int CNT, bool PLAIN = false>
 __device__ __forceinline__ void store_tokens_act(const Epilogue& e, uint16_t* out,
                                                  const float (&v)[CNT], int m0, int m_end, int n,

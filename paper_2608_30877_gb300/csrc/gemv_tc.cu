@@ -29,9 +29,9 @@
 // tokens at a time, each CTA finishing its share of them in the order of the
 // ranks (deterministic).  12288 rows on 152 SMs are 82 rows, one 128-row tile, per
 // CTA without a split, and a lone tile runs at the latency of its four row
-// warps (0.47 us per stage whatever M): K = 49152 at M = 100 with bias and residual 398
-// us (before) -> 126 us (clusters of 4, 342 rows each); 12288 x 12288 at M = 24
-// 56 -> 24 us.
+// warps (0.47 us per stage whatever M): K = 49152 at M = 100 with bias and residual,
+// L2 flushed, 398 us (before) -> 120 us (clusters of 4, 342 rows each); 12288 x 12288 at M =
+// 24 56 -> 23 us.
 //
 // What bounds it (K = 12288, 152 SMs): the row warps' latency and issue slots, not the
 // tensor pipe: a stage costs 0.39-0.50, 0.51-0.71, 0.62-1.05 us for one, two, three
@@ -47,8 +47,17 @@
 // tcgen05.mma with A in tensor memory runs at 18 / 32 / 64 clocks for 32 / 64 /
 // 128 columns with three independent accumulators, 44 with one (measured alone), so
 // the MMAs need 0.22-0.8 us of a stage.  From 97 tokens on three tiles leave the A ring
-// only two or three slots of a quarter stage.  Measured and not kept (M <= 32): two groups
-// of row warps per tile (99 us: the A ring is too short for them), the next stage's codes
+// only two or three slots of a quarter stage.  Token columns: whole output slices of 32, and
+// 112, which leave the ring a third slot there and cost less of a stage (M = 112 with 112 columns
+// and 128 with 128: 111 and 112 us at N = 49152, 74 and 80 at 36864, 45 and 46 at 19456); 48 and 80
+// have not been tried.
+// A stage in which a row of the warp has a scale of 2^-2 or more takes the general dequantisation
+// (dequant.cuh): if all do, M = 8 to 32 95 us at N = 49152, 80 at 36864, where the warp-level
+// kernel takes 65 and 52 up to 8 tokens (W4A16_SMALL_M=mma keeps a model of such scales on
+// it; those of weights N(0, 0.02) are near 2^-7).  Constants shifted for such rows were measured: the
+// ordinary call then takes 2 to 4% more, whichever way the second walk is kept out of the
+// first one's code.
+// Measured and not kept (M <= 32): two groups of row warps per tile (99 us: the A ring is too short for them), the next stage's codes
 // read before this one's stores end (71) or after (66), one issuing warp for all tiles
 // (92), a rolled dequant loop (78), 16 token columns for M <= 16 (67).
 //

@@ -131,8 +131,9 @@ __device__ __forceinline__ void unit_tile(int unit, const TsParams& p, int rank,
 
 // Epilogue of one tile for the epilogue thread that owns weight row n (TMEM lane
 // `lane` of its sub-partition): the 32-token chunks c0, c0 + cs, ... of the T tokens
-// from TMEM column d_col; fused, 16 tokens at a time (32 spill next to the residuals;
-// plain, 16 at a time are slower: 200 x 36864 x 12288 131 against 118 us).
+// from TMEM column d_col; fused, 16 tokens at a time (832 threads leave 78 registers
+// each: 32 tokens next to their residuals would not fit them, with 16 it is 8 to 28 bytes that
+// spill; plain, 16 at a time are slower: 200 x 36864 x 12288 131 against 118 us).
 template <int T, bool FUSED>
 __device__ __forceinline__ void epilogue_tile(const TsParams& p, uint32_t d_col, int m0, int n,
                                               int lane, int c0, int cs) {

@@ -46,11 +46,30 @@ def test_attention_traffic_scales_with_pairs():
         return
     assert bench.ncu_traffic("attention", 0, 64) == t8 * 8
     assert bench.ncu_traffic("topk", 0) is None
-    # M = 9..16 read the M = 16 capture, M = 17..32 the tensor-core kernel's
-    h = bench.kernel_source_hash("gemv")
-    assert bench.ncu_traffic("gemv", 12) == bench.NCU_TRAFFIC.get(("gemv16", "gemv", h))
-    assert bench.ncu_traffic("gemv", 3) == bench.NCU_TRAFFIC.get(("gemv", "gemv", h))
     t = bench.kernel_source_hash("ts")
     for c in ("mlp_up", "mlp_down", "qkv"):
         assert bench.ncu_traffic(c, 8192) == bench.NCU_TRAFFIC.get((c, "ts", t))
     assert bench.ncu_traffic("mlp_swiglu", 8192) is None
+
+
+def test_small_m_traffic_reads_the_capture_of_its_tokens(monkeypatch):
+    captured = {c: v for (c, kind, _), v in bench.NCU_TRAFFIC.items() if kind == "gemv"}
+    assert sorted(captured) == ["gemv16", "gemv32", "gemv8"]
+    # as if captured with the present sources
+    h = bench.kernel_source_hash("gemv")
+    monkeypatch.setattr(bench, "NCU_TRAFFIC", {(c, "gemv", h): v for c, v in captured.items()})
+    for m, c in ((1, "gemv8"), (8, "gemv8"), (9, "gemv16"), (16, "gemv16"), (17, "gemv32"), (32, "gemv32")):
+        assert bench.ncu_traffic("gemv", m) == captured[c]
+    assert bench.ncu_traffic("gemv", 33) is None
+
+
+def test_traffic_follows_the_dispatch_and_the_output_stage():
+    for kind in ("ts", "gemv"):
+        assert {"api.cu", "epilogue.cuh"} <= set(bench.KERNEL_FILES[kind])
+    csrc = os.path.join(ROOT, "paper_2608_30877_gb300", "csrc")
+    for files in bench.KERNEL_FILES.values():  # and every header that a kernel includes
+        for name in files:
+            for line in open(os.path.join(csrc, name)):
+                if line.startswith('#include "') and name != "api.cu":
+                    header = line.split('"')[1]
+                    assert header in files or header == "w4a16.h", (name, header)
