@@ -51,11 +51,11 @@ NCU_TRAFFIC = {
     ("mlp_down", "ts", "755eda9058f870bf"): 4.7834e9 + 0.1975e9,
     # small-M readout, M = 8, 16 and 32 (tensor-core streaming kernel, 32 token columns),
     # 12288x49152, one launch each (profiles/gemv_tc_m32_12288x49152.md)
-    ("gemv8", "gemv", "8fcee59793c4dbda"): 0.32545e9 + 0.00320e9,
-    ("gemv16", "gemv", "8fcee59793c4dbda"): 0.32529e9 + 0.00319e9,
-    ("gemv32", "gemv", "8fcee59793c4dbda"): 0.32670e9 + 0.00321e9,
-    # attention prefill per 8 pairs of 1024 tokens x 96 heads (full capture of
-    # one 8-pair launch); scaled by pairs / 8 for the benched launch
+    ("gemv8", "gemv", "41e14d876a04c6b5"): 0.32545e9 + 0.00320e9,
+    ("gemv16", "gemv", "41e14d876a04c6b5"): 0.32529e9 + 0.00319e9,
+    ("gemv32", "gemv", "41e14d876a04c6b5"): 0.32670e9 + 0.00321e9,
+    # attention prefill per 8 pairs of 1024 tokens x 96 heads (one 8-pair launch);
+    # scaled by pairs / 8 for the benched launch (profiles/attention_prefill_8x1024_h96.md)
     ("attention", "attn", "721466a15446229a"): 0.6045e9 + 0.1727e9,
 }
 

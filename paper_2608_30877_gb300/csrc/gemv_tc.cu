@@ -35,7 +35,8 @@
 //
 // What bounds it (K = 12288, 152 SMs): the row warps' latency and issue slots, not the
 // tensor pipe: a stage costs 0.39-0.50, 0.51-0.71, 0.62-1.05 us for one, two, three
-// tiles (N = 49152: 63 us at M <= 32, 78 at 64, 84 at 96, 103 at 112, 104 at 128).  In order,
+// tiles (N = 49152, one launch after another: 61 us at M <= 32, 77 at 64, 85 at 96, 111 at
+// 112, 112 at 128; 63, 78, 84, 103 and 104 where these stages were fitted).  In order,
 // what brought it there from 92, 103, 137, 137 and 139: weights dequantised in k order,
 // with no x reorder warp, through one FMA, operands in uniform registers, addresses that
 // only advance (72, 80, 86, -, 110); then, from stamps of a row warp, whose 1540 clocks
@@ -57,9 +58,10 @@
 // it; those of weights N(0, 0.02) are near 2^-7).  Constants shifted for such rows were measured: the
 // ordinary call then takes 2 to 4% more, whichever way the second walk is kept out of the
 // first one's code.
-// Measured and not kept (M <= 32): two groups of row warps per tile (99 us: the A ring is too short for them), the next stage's codes
-// read before this one's stores end (71) or after (66), one issuing warp for all tiles
-// (92), a rolled dequant loop (78), 16 token columns for M <= 16 (67).
+// Measured and not kept (M <= 32): two groups of row warps per tile (99 us: the A ring is
+// too short for them), the next stage's codes read before this one's stores end (71) or
+// after (66), one issuing warp for all tiles (92), a rolled dequant loop (78), 16 token
+// columns for M <= 16 (67).
 //
 // Every wait is bounded (ptx.cuh); on a timeout the kernel records
 // W4A16_ERR_TIMEOUT, drains its copies and MMAs, frees tensor memory and

@@ -19,7 +19,7 @@
 // counting smaller pairs, and stores them.  Nothing goes through global memory.
 // Bound by latency (about five cluster barriers) and the first digit's atomics:
 // 200000 scores, k = 1000 56 -> 21 us; 10000, k = 100 27.7 -> 11.3; 2000000, k = 1024
-// 295 -> 90 (before: seven passes over the scores by scalar loads, a digit search by one
+// 295 -> 89 (before: seven passes over the scores by scalar loads, a digit search by one
 // thread and 55 sorting steps on one CTA).
 #include "internal.h"
 
