@@ -41,19 +41,19 @@ NCU_TRAFFIC = {
     # mean of one launch per stack shape at M = 16384 (384-token tiles, as in
     # the benched stack), scaled by 4 to M = 65536
     # (profiles/gemm_pair_wide_stack_traffic_m16384.md)
-    ("stack", "ts", "755eda9058f870bf"): 7.1498e9 * 4,
+    ("stack", "ts", "12867246fbba2cb2"): 7.1498e9 * 4,
     # QKV prefill 4096x12288x36864 (384-token CTA pairs), one launch
     # (profiles/gemm_pair_wide_qkv_prefill_4096x12288x36864.md)
-    ("qkv", "ts", "755eda9058f870bf"): 1.4728e9 + 0.2891e9,
+    ("qkv", "ts", "12867246fbba2cb2"): 1.4728e9 + 0.2891e9,
     # MLP up / down at 8192 tokens (384-token CTA pairs), one launch each
     # (DRAM counters only; profiles/gemm_pair_mlp_traffic_8192.md)
-    ("mlp_up", "ts", "755eda9058f870bf"): 3.9444e9 + 0.8024e9,
-    ("mlp_down", "ts", "755eda9058f870bf"): 4.7834e9 + 0.1975e9,
+    ("mlp_up", "ts", "12867246fbba2cb2"): 3.9444e9 + 0.8024e9,
+    ("mlp_down", "ts", "12867246fbba2cb2"): 4.7834e9 + 0.1975e9,
     # small-M readout, M = 8, 16 and 32 (tensor-core streaming kernel, 32 token columns),
     # 12288x49152, one launch each (profiles/gemv_tc_m32_12288x49152.md)
-    ("gemv8", "gemv", "41e14d876a04c6b5"): 0.32545e9 + 0.00320e9,
-    ("gemv16", "gemv", "41e14d876a04c6b5"): 0.32529e9 + 0.00319e9,
-    ("gemv32", "gemv", "41e14d876a04c6b5"): 0.32670e9 + 0.00321e9,
+    ("gemv8", "gemv", "a01ab34f117a1094"): 0.32545e9 + 0.00320e9,
+    ("gemv16", "gemv", "a01ab34f117a1094"): 0.32529e9 + 0.00319e9,
+    ("gemv32", "gemv", "a01ab34f117a1094"): 0.32670e9 + 0.00321e9,
     # attention prefill per 8 pairs of 1024 tokens x 96 heads (one 8-pair launch);
     # scaled by pairs / 8 for the benched launch (profiles/attention_prefill_8x1024_h96.md)
     ("attention", "attn", "721466a15446229a"): 0.6045e9 + 0.1727e9,

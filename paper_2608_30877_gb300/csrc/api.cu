@@ -311,12 +311,20 @@ LinearRoute choose_linear(const DeviceState& st, int64_t M, int64_t N, int64_t K
     // from HBM): K = 12288, N = 12288 34 against 22 us, 25000 45 / 35 (both K split), 30000
     // 48.5 / 50, 36864 51 / 50.5, 49152 64.5 / 60.5, with SwiGLU 66 / 69; K = 1024, N = 12288 5.0
     // / 6.2, 49152 9.9 / 10.1, with SwiGLU 10.7 / 13.9; K = 128, 98304 5.9 / 6.5.  M = 9..16: K =
-    // 12288, 30000 60 / 50; K = 1024, 12288 6.2 / 6.2.
+    // 12288, 30000 60 / 50; K = 1024, 12288 6.2 / 6.2.  A fused output stage alone moves
+    // no layer of K > 4096: it makes 3 to 9% there (K = 12288, M = 1, SwiGLU, N = 36864 53 / 57, 98304
+    // 127 / 136; K = 4096, 21 / 26 and 48 / 55), and the streaming kernel multiplies the weights as the
+    // format rounds them (error 0.0017 of the output's norm), while the warp-level one rounds
+    // no product and is 0.0021 from that definition.
     if (M <= 128) {
         r.plan = gemv_tc_plan(M, N, K, g, epi, st.sm_count);
-        const bool rows = M <= 16 && g == 128 &&
-                          (g_small_m == 0 ? gemv_cost_us(M, N, K, epi, st.sm_count) < r.plan.cost_us
-                                          : g_small_m == 'm');
+        bool rows = M <= 16 && g == 128 && g_small_m != 't';
+        if (rows && g_small_m == 0) {
+            rows = gemv_cost_us(M, N, K, epi, st.sm_count) < r.plan.cost_us;
+            if (rows && K > 4096 && epilogue_fused(epi))
+                rows = gemv_cost_us(M, N, K, Epilogue{}, st.sm_count) <
+                       gemv_tc_plan(M, N, K, g, Epilogue{}, st.sm_count).cost_us;
+        }
         r.kind = rows ? LinearRoute::kRows : LinearRoute::kStream;
         return r;
     }

@@ -4,8 +4,8 @@
 // K <= 1024 and up to 53000 rows; longer K where splitting it no longer helps and a
 // sub-partition's two or three warps are not yet full, 29000 to 35000 and 39000 to 43500 rows
 // at K = 12288 (on 152 SMs).  With a fused output stage, of which gemv_tc.cu finishes 32
-// tokens whatever M, 29000 to 53000 and 78000 to 107000 rows.  From 9 tokens on only plain
-// layers of K <= 1024 and few rows.
+// tokens whatever M, also 29000 to 53000 and 78000 to 107000 rows up to K = 4096.  From 9
+// tokens on only plain layers of K <= 1024 and few rows.
 //
 // Design, GB300-first:
 //   - persistent grid, one CTA per SM; CTA c owns a contiguous range of RB

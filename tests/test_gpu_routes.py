@@ -21,7 +21,9 @@ def test_kernel_by_size(M, N, K, g, kernel):
 # layers that a kernel with a higher rate, but more to start or to finish, had taken
 @pytest.mark.parametrize("M,N,K,g,act,residual,kernel", [
     (1, 98304, 1024, 128, 1, False, "rows"), (8, 49152, 256, 128, 2, False, "rows"),
-    (1, 49152, 1024, 128, 0, False, "rows"), (8, 98304, 12288, 128, 1, False, "rows"),
+    (1, 49152, 1024, 128, 0, False, "rows"), (8, 98304, 12288, 128, 1, False, "stream"),
+    (1, 36864, 12288, 128, 1, False, "stream"), (1, 36864, 1024, 128, 1, False, "rows"),
+    (8, 30000, 12288, 128, 1, True, "rows"),
     (8, 98304, 12288, 128, 0, False, "stream"), (16, 49152, 1024, 128, 1, False, "stream"),
     (1, 49152, 12288, 128, 0, False, "stream"),
     (129, 36864, 12288, 64, 0, False, "gemm"), (129, 36864, 12288, 128, 0, False, "stream"),
