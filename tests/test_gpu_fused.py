@@ -197,15 +197,21 @@ def test_fused_gelu_bias_residual_in_place_fullsize_sampled():
 
 
 @pytest.mark.slow
-@pytest.mark.parametrize("M", [8, 24])
-def test_fused_swiglu_small_m_readout_scale(M):
+@pytest.mark.parametrize("M,kernel", [(8, "rows"), (8, "stream"), (24, "stream")])
+def test_fused_swiglu_small_m_readout_scale(M, kernel):
     """SwiGLU + bias + residual on the small-M streaming kernels (warp-level
-    at M = 8, tensor-core at M = 24) over the full gate/up weights (K 12288 x
+    at M = 8, tensor-core at M = 8 and 24) over the full gate/up weights (K 12288 x
     2 x 49152 interleaved rows: more row chunks than SMs), on sampled output
     columns for every token."""
+    if kernel == "rows":
+        run_in_child({"W4A16_SMALL_M": "mma"}, "test_gpu_fused", "check_readout_scale", M, kernel)
+    else:
+        check_readout_scale(M, kernel)
+
+
+def check_readout_scale(M, kernel):
     W = _W()
-    assert W.route(M, S.MLP_SWIGLU.N, S.MLP_SWIGLU.K, 128, W.ACT_SWIGLU, True)[0] == \
-        ("rows" if M == 8 else "stream")
+    assert W.route(M, S.MLP_SWIGLU.N, S.MLP_SWIGLU.K, 128, W.ACT_SWIGLU, True)[0] == kernel
     c = S.MLP_SWIGLU
     packed, scales, wd, sd = prepare_weights(c.N, c.K, c.g, c.w_seed)
     x = S.make_x(M, c.K, 700 + M, "cuda")
